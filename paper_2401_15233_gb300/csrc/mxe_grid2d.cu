@@ -86,69 +86,32 @@ __device__ __forceinline__ void load_prim_f64(const Stage2DArgs& a, int gi, int 
     PH::cons2prim_rn(U, Q);
 }
 
-// Numerical face flux from two face states (HLL with Davis speeds, or
-// Rusanov), Sec. 3.1.
+// Numerical face flux of the face between box cells c and c + stride.
 template <class PH, int K>
-__device__ __forceinline__ void riemann_f64(const double* QL, const double* QR,
-                                            const ParamsT<double>& p, double* Fo) {
+__device__ __forceinline__ void face_flux_f64(const double* W, int c, int stride, double phl,
+                                              double phr, const ParamsT<double>& p, double* F) {
     constexpr int NF = PH::NF;
-    double UL[NF], FL[NF], lminL, lmaxL;
-    PH::template face<double, K>(QL, p.sigma_lim, p.k_ws, UL, FL, lminL, lmaxL);
-    double UR[NF], FR[NF], lminR, lmaxR;
-    PH::template face<double, K>(QR, p.sigma_lim, p.k_ws, UR, FR, lminR, lmaxR);
-    if (p.flux == 1) {
-        double s = fabs(lminL);
-        s = fabs(lmaxL) > s ? fabs(lmaxL) : s;
-        s = fabs(lminR) > s ? fabs(lminR) : s;
-        s = fabs(lmaxR) > s ? fabs(lmaxR) : s;
-#pragma unroll
-        for (int k = 0; k < NF; ++k) Fo[k] = 0.5 * (FL[k] + FR[k]) - 0.5 * s * (UR[k] - UL[k]);
-        return;
-    }
-    double SL = lminL < lminR ? lminL : lminR;
-    double SR = lmaxL > lmaxR ? lmaxL : lmaxR;
-    if (SL >= 0.0) {
-#pragma unroll
-        for (int k = 0; k < NF; ++k) Fo[k] = FL[k];
-    } else if (SR <= 0.0) {
-#pragma unroll
-        for (int k = 0; k < NF; ++k) Fo[k] = FR[k];
-    } else {
-        double inv = 1.0 / (SR - SL);
-        double SLR = SL * SR;
-#pragma unroll
-        for (int k = 0; k < NF; ++k) Fo[k] = (SR * FL[k] - SL * FR[k] + SLR * (UR[k] - UL[k])) * inv;
-    }
-}
-
-template <int NF>
-__device__ __forceinline__ double phi_box(const double* W, int c, int stride, int lim) {
-    double phi = 1.0;
-    const FlatRef<double> fr = flat_ref<NF>(W + c, NBOX);
+    double Q[NF], UL[NF], FL[NF], UR[NF], FR[NF], l0, l1, r0, r1;
+    const double hl = 0.25 * phl, hr = -0.25 * phr;
 #pragma unroll
     for (int k = 0; k < NF; ++k) {
         const double* w = W + k * NBOX + c;
-        phi_accumulate<NF>(phi, w[0] - w[-stride], w[stride] - w[0], lim, fr, k);
+        Q[k] = f64::face_value(w[-stride], w[0], w[stride], hl);
     }
-    return phi;
-}
-
-template <int NF>
-__device__ __forceinline__ void face_state_box(const double* W, int c, int stride, double phi,
-                                               double sgn, double* Qf) {
-    double hs = mul_rn(sgn, 0.5);
+    PH::template face<double, K>(Q, p.sigma_lim, p.k_ws, UL, FL, l0, l1);
 #pragma unroll
     for (int k = 0; k < NF; ++k) {
-        const double* w = W + k * NBOX + c;
-        Qf[k] = muscl_face(w[-stride], w[0], w[stride], phi, hs);
+        const double* w = W + k * NBOX + c + stride;
+        Q[k] = f64::face_value(w[-stride], w[0], w[stride], hr);
     }
+    PH::template face<double, K>(Q, p.sigma_lim, p.k_ws, UR, FR, r0, r1);
+    f64::riemann<NF>(UL, FL, l0, l1, UR, FR, r0, r1, p.flux, F);
 }
 
 __device__ __forceinline__ void block_max_atomic(double r, unsigned long long* dst, double* red) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        double v = __shfl_xor_sync(0xffffffffu, r, o);
-        r = v > r ? v : r;
+        r = f64::max_(r, __shfl_xor_sync(0xffffffffu, r, o));
     }
     int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (lane == 0) red[wid] = r;
@@ -157,8 +120,7 @@ __device__ __forceinline__ void block_max_atomic(double r, unsigned long long* d
         r = lane < (NT2 / 32) ? red[lane] : 0.0;
 #pragma unroll
         for (int o = 4; o > 0; o >>= 1) {
-            double v = __shfl_xor_sync(0xffffffffu, r, o);
-            r = v > r ? v : r;
+            r = f64::max_(r, __shfl_xor_sync(0xffffffffu, r, o));
         }
         if (lane == 0) atomicMax(dst, (unsigned long long)__double_as_longlong(r));
     }
@@ -198,7 +160,7 @@ __device__ __forceinline__ void stage_f64(const Stage2DArgs& a) {
     double* phx = Fb + NF * NT2;                     // [TY][TX+2]
     double* phy = phx + NPHX;                        // [TY+2][TX]
     double* red = phy + NPHY;                        // [8]
-    __shared__ double sdt[2];
+    __shared__ double sdt[3];
 
     const int tid = threadIdx.x;
     if (tid == 0) {
@@ -206,6 +168,7 @@ __device__ __forceinline__ void stage_f64(const Stage2DArgs& a) {
         sdt[0] = step_dt(a.clk, a.slot, a.cfl, a.t_end, a.dt_fixed, tt);
         sdt[1] = tt;
     }
+    if (tid == 32) sdt[2] = f64::tau_factor(a.rp.model, a.rp.tau_ref, a.rp.rho_ref, a.rp.T_ref);
     __syncthreads();
     const double dt = sdt[0], t = sdt[1];
     if (a.final_stage && blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) advance_clock(a, dt, t);
@@ -224,19 +187,18 @@ __device__ __forceinline__ void stage_f64(const Stage2DArgs& a) {
     __syncthreads();
     for (int n = tid; n < NPHX; n += NT2) {
         int bx = 1 + n % (TX + 2), by = 2 + n / (TX + 2);
-        phx[n] = p.order == 2 ? phi_box<NF>(W, by * BX + bx, 1, p.limiter) : 0.0;
+        phx[n] = p.order == 2 ? f64::limiter<NF>(W, by * BX + bx, 1, NBOX, p.limiter) : 0.0;
     }
     for (int n = tid; n < NPHY; n += NT2) {
         int bx = 2 + n % TX, by = 1 + n / TX;
-        phy[n] = p.order == 2 ? phi_box<NF>(W, by * BX + bx, BX, p.limiter) : 0.0;
+        phy[n] = p.order == 2 ? f64::limiter<NF>(W, by * BX + bx, BX, NBOX, p.limiter) : 0.0;
     }
     __syncthreads();
     {   // x faces: face fx in [0,16) of row cy, between box cells fx+1 | fx+2
         int fx = tid & 15, cy = tid >> 4, by = cy + 2;
-        double QL[NF], QR[NF], F[NF];
-        face_state_box<NF>(W, by * BX + fx + 1, 1, phx[cy * (TX + 2) + fx], 1.0, QL);
-        face_state_box<NF>(W, by * BX + fx + 2, 1, phx[cy * (TX + 2) + fx + 1], -1.0, QR);
-        riemann_f64<PH, 0>(QL, QR, p, F);
+        double F[NF];
+        face_flux_f64<PH, 0>(W, by * BX + fx + 1, 1, phx[cy * (TX + 2) + fx],
+                             phx[cy * (TX + 2) + fx + 1], p, F);
 #pragma unroll
         for (int k = 0; k < NF; ++k) Fb[k * NT2 + tid] = F[k];
     }
@@ -249,7 +211,8 @@ __device__ __forceinline__ void stage_f64(const Stage2DArgs& a) {
 #pragma unroll
         for (int k = 0; k < NF; ++k) Qc[k] = W[k * NBOX + (cy + 2) * BX + cx + 2];
         if (p.tau_model != 0 && !p.src_implicit) {
-            PH::source(Qc, PH::tau(p, Qc), L);
+            const double pr = PH::pressure64(Qc);
+            PH::source64(Qc, pr, f64::inv_tau(p.tau_model, sdt[2], Qc[0], pr), L);
         } else {
 #pragma unroll
             for (int k = 0; k < NF; ++k) L[k] = 0.0;
@@ -261,10 +224,9 @@ __device__ __forceinline__ void stage_f64(const Stage2DArgs& a) {
     __syncthreads();
     if (tid < TX * (TY + 1)) {   // y faces: face fy in [0,17) of column cx
         int fcx = tid % TX, fy = tid / TX, bx = fcx + 2;
-        double QL[NF], QR[NF], F[NF];
-        face_state_box<NF>(W, (fy + 1) * BX + bx, BX, phy[fy * TX + fcx], 1.0, QL);
-        face_state_box<NF>(W, (fy + 2) * BX + bx, BX, phy[(fy + 1) * TX + fcx], -1.0, QR);
-        riemann_f64<PH, 1>(QL, QR, p, F);
+        double F[NF];
+        face_flux_f64<PH, 1>(W, (fy + 1) * BX + bx, BX, phy[fy * TX + fcx],
+                             phy[(fy + 1) * TX + fcx], p, F);
 #pragma unroll
         for (int k = 0; k < NF; ++k) Fb[k * NT2 + tid] = F[k];
     }
@@ -292,19 +254,19 @@ __device__ __forceinline__ void stage_f64(const Stage2DArgs& a) {
 #pragma unroll
             for (int k = 0; k < NF; ++k) {
                 a.Uout[o + PH::ufield(k) * g.fstride] = Un[k];
-                bad |= !isfinite(Un[k]);
+                bad |= !f64::is_finite(Un[k]);
             }
             if (a.final_stage) {
                 double Qn[NF];
                 PH::cons2prim_rn(Un, Qn);
-                if (PH::nonpositive(Qn)) atomicOr(&a.clk->status, ST_NONPOSITIVE);
+                if (PH::nonpositive64(Qn)) atomicOr(&a.clk->status, ST_NONPOSITIVE);
                 if (bad) atomicOr(&a.clk->status, ST_NONFINITE);
                 if (!a.skip_rate) {
                     double ax, ay;
                     PH::rates(Qn, p.sigma_lim, p.k_ws, ax, ay);
                     r = ax * g.idx;
                     r = r + ay * g.idy;
-                    if (!(r >= 0.0)) r = __longlong_as_double(0x7ff0000000000000ll);  // NaN -> inf
+                    if (!f64::ge0(r)) r = __longlong_as_double(0x7ff0000000000000ll);  // NaN -> inf
                 }
             }
         }

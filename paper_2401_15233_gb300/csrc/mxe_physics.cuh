@@ -19,6 +19,8 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include "mxe_fast64.cuh"
+
 namespace mxe {
 
 // ---------------------------------------------------------------- math shims
@@ -133,7 +135,7 @@ __device__ __forceinline__ void cons2prim5(const T* U, T* Q) {
 // r = U4 - (((rho u) u) u) u - ((6u) u) P - (4u) q.
 __device__ __forceinline__ void cons2prim5_rn(const double* U, double* Q) {
     double rho = U[0];
-    double u = U[1] / rho;
+    double u = f64::div_by(U[1], rho, f64::rcp(rho));
     double ru = mul_rn(rho, u), ruu = mul_rn(ru, u), ruuu = mul_rn(ruu, u);
     double P = sub_rn(U[2], ruu);
     double q = sub_rn(sub_rn(U[3], ruuu), mul_rn(mul_rn(3.0, u), P));
@@ -329,7 +331,9 @@ __device__ __forceinline__ void cons2prim14(const T* U, T* Q) {
 //   R = (((E4 - (rho |u|^2)|u|^2) - (2|u|^2) tr P) - 4 u.P.u) - 4 u.q
 __device__ __forceinline__ void cons2prim14_rn(const double* U, double* Q) {
     double rho = U[0];
-    double u[3] = {U[1] / rho, U[2] / rho, U[3] / rho};
+    const double ir = f64::rcp(rho);
+    double u[3] = {f64::div_by(U[1], rho, ir), f64::div_by(U[2], rho, ir),
+                   f64::div_by(U[3], rho, ir)};
     double P[3][3];
     int idx = 4;
 #pragma unroll
@@ -829,6 +833,16 @@ __device__ __forceinline__ bool field_flat(const FlatRef<T>& f, int k, T m) {
     case 3: return mul_rn(mul_rn(m, m), f.rho) <= mul_rn(mul_rn(mul_rn(ch, f.s), f.s), f.s);
     default: return mul_rn(m, f.rho) <= mul_rn(mul_rn(cr, f.s), f.s);
     }
+}
+
+// the same for a field known at run time
+template <int NF>
+__device__ __forceinline__ bool field_flat_at(const FlatRef<double>& f, int k, double m) {
+    constexpr int v1 = NF == 5 ? 1 : NF == 10 ? 2 : 3, p1 = NF == 5 ? 2 : NF == 10 ? 6 : 9;
+    if (k == 0) return field_flat<NF>(f, 0, m);
+    if (k <= v1) return field_flat<NF>(f, 1, m);
+    if (k <= p1) return field_flat<NF>(f, p1, m);
+    return k < NF - 1 ? field_flat<NF>(f, NF - 2, m) : field_flat<NF>(f, NF - 1, m);
 }
 
 template <class T>

@@ -68,7 +68,8 @@ __device__ __forceinline__ void cons2prim_p(const T* U, T* Q) {
 // (the vanishing terms it adds are exact zeros).
 __device__ __forceinline__ void cons2prim_p_rn(const double* U, double* Q) {
     double rho = U[0];
-    double ux = U[1] / rho, uy = U[2] / rho;
+    const double ir = f64::rcp(rho);
+    double ux = f64::div_by(U[1], rho, ir), uy = f64::div_by(U[2], rho, ir);
     double Pxx = sub_rn(U[3], mul_rn(mul_rn(rho, ux), ux));
     double Pxy = sub_rn(U[4], mul_rn(mul_rn(rho, ux), uy));
     double Pyy = sub_rn(U[5], mul_rn(mul_rn(rho, uy), uy));

@@ -3,6 +3,7 @@
 // ten active fields).  A policy supplies the number of active fields, their
 // positions in the 14-field conserved layout, and the point functions.
 #pragma once
+#include "mxe_face64.cuh"
 #include "mxe_planar.cuh"
 
 namespace mxe {
@@ -44,7 +45,8 @@ struct PhysGeneral {
     }
     template <class T, int K>
     static __device__ __forceinline__ void face(const T* Q, T sl, T kw, T* U, T* F, T& lo, T& hi) {
-        face_eval14<T, K>(Q, sl, kw, U, F, lo, hi);
+        if constexpr (sizeof(T) == 8) f64::face_14<K>(Q, sl, kw, U, F, lo, hi);
+        else face_eval14<T, K>(Q, sl, kw, U, F, lo, hi);
     }
     // with the conditioning of the closure (raw sigma, det P*)
     template <class T, int K>
@@ -62,17 +64,35 @@ struct PhysGeneral {
     }
     template <class T>
     static __device__ __forceinline__ void rates(const T* Q, T sl, T kw, T& ax, T& ay) {
-        Dimless14<T> d;
-        dimless14(Q, d);
-        ax = amax14<T, 0>(Q, d, sl, kw);
-        ay = amax14<T, 1>(Q, d, sl, kw);
+        if constexpr (sizeof(T) == 8) {
+            f64::rates_14(Q, sl, kw, ax, ay);
+        } else {
+            Dimless14<T> d;
+            dimless14(Q, d);
+            ax = amax14<T, 0>(Q, d, sl, kw);
+            ay = amax14<T, 1>(Q, d, sl, kw);
+        }
     }
     // x rate alone (1D problems)
     template <class T>
     static __device__ __forceinline__ T rate_x(const T* Q, T sl, T kw) {
-        Dimless14<T> d;
-        dimless14(Q, d);
-        return amax14<T, 0>(Q, d, sl, kw);
+        if constexpr (sizeof(T) == 8) {
+            return f64::rate_x_14(Q, sl, kw);
+        } else {
+            Dimless14<T> d;
+            dimless14(Q, d);
+            return amax14<T, 0>(Q, d, sl, kw);
+        }
+    }
+    static __device__ __forceinline__ double pressure64(const double* Q) {
+        return (Q[4] + Q[7] + Q[9]) * (1.0 / 3.0);
+    }
+    static __device__ __forceinline__ void source64(const double* Q, double p, double it,
+                                                    double* C) {
+        f64::source_14(Q, p, it, C);
+    }
+    static __device__ __forceinline__ bool nonpositive64(const double* Q) {
+        return f64::le0(Q[0]) || f64::le0(Q[4]) || f64::le0(Q[7]) || f64::le0(Q[9]);
     }
     static __device__ __forceinline__ void increment(const float* W, const float* dU, float* Wn) {
         prim_increment14(W, dU, Wn);
@@ -102,7 +122,8 @@ struct PhysPlanar {
     }
     template <class T, int K>
     static __device__ __forceinline__ void face(const T* Q, T sl, T kw, T* U, T* F, T& lo, T& hi) {
-        face_eval_p<T, K>(Q, sl, kw, U, F, lo, hi);
+        if constexpr (sizeof(T) == 8) f64::face_p<K>(Q, sl, kw, U, F, lo, hi);
+        else face_eval_p<T, K>(Q, sl, kw, U, F, lo, hi);
     }
     template <class T, int K>
     static __device__ __forceinline__ void face_c(const T* Q, T sl, T kw, T* U, T* F, T& lo,
@@ -117,16 +138,34 @@ struct PhysPlanar {
     }
     template <class T>
     static __device__ __forceinline__ void rates(const T* Q, T sl, T kw, T& ax, T& ay) {
-        DimlessP<T> g;
-        dimless_p(Q, g);
-        ax = amax_p<T, 0>(Q, g, sl, kw);
-        ay = amax_p<T, 1>(Q, g, sl, kw);
+        if constexpr (sizeof(T) == 8) {
+            f64::rates_p(Q, sl, kw, ax, ay);
+        } else {
+            DimlessP<T> g;
+            dimless_p(Q, g);
+            ax = amax_p<T, 0>(Q, g, sl, kw);
+            ay = amax_p<T, 1>(Q, g, sl, kw);
+        }
     }
     template <class T>
     static __device__ __forceinline__ T rate_x(const T* Q, T sl, T kw) {
-        DimlessP<T> g;
-        dimless_p(Q, g);
-        return amax_p<T, 0>(Q, g, sl, kw);
+        if constexpr (sizeof(T) == 8) {
+            return f64::rate_x_p(Q, sl, kw);
+        } else {
+            DimlessP<T> g;
+            dimless_p(Q, g);
+            return amax_p<T, 0>(Q, g, sl, kw);
+        }
+    }
+    static __device__ __forceinline__ double pressure64(const double* Q) {
+        return (Q[3] + Q[5] + Q[6]) * (1.0 / 3.0);
+    }
+    static __device__ __forceinline__ void source64(const double* Q, double p, double it,
+                                                    double* C) {
+        f64::source_p(Q, p, it, C);
+    }
+    static __device__ __forceinline__ bool nonpositive64(const double* Q) {
+        return f64::le0(Q[0]) || f64::le0(Q[3]) || f64::le0(Q[5]) || f64::le0(Q[6]);
     }
     static __device__ __forceinline__ void increment(const float* W, const float* dU, float* Wn) {
         prim_increment_p(W, dU, Wn);

@@ -10,6 +10,7 @@
 // 2-cell halo in shared memory, one shared limiter per cell, one thread per
 // face (two face states, closure, flux, wave speeds, HLL/Rusanov), then
 // flux differences, BGK source and the RK update.
+#include "mxe_face64.cuh"
 #include "mxe_internal.h"
 
 namespace mxe {
@@ -27,12 +28,10 @@ template <> struct Sys<5> {
     }
     static __device__ __forceinline__ void eval(const double* Q, const SchemeParams& sp, double* U,
                                                 double* F, double& lo, double& hi) {
-        face_eval5(Q, sp, U, F, lo, hi);
+        f64::face_5(Q, sp.sigma_lim, sp.k_ws, U, F, lo, hi);
     }
     static __device__ __forceinline__ double amax(const double* Q, const SchemeParams& sp) {
-        double a, s;
-        rate5(Q, sp, a, s);
-        return a;
+        return f64::rate_5(Q, sp.sigma_lim, sp.k_ws);
     }
     static __device__ __forceinline__ void source(const double* Q, double tau, double* C) {
         source5(Q, tau, C);
@@ -46,12 +45,10 @@ template <> struct Sys<14> {
     }
     static __device__ __forceinline__ void eval(const double* Q, const SchemeParams& sp, double* U,
                                                 double* F, double& lo, double& hi) {
-        face_eval14<double, 0>(Q, sp, U, F, lo, hi);
+        f64::face_14<0>(Q, sp.sigma_lim, sp.k_ws, U, F, lo, hi);
     }
     static __device__ __forceinline__ double amax(const double* Q, const SchemeParams& sp) {
-        Dimless14<double> d;
-        dimless14(Q, d);
-        return amax14<double, 0>(Q, d, sp);
+        return f64::rate_x_14(Q, sp.sigma_lim, sp.k_ws);
     }
     static __device__ __forceinline__ void source(const double* Q, double tau, double* C) {
         source14(Q, tau, C);

@@ -247,19 +247,22 @@ static mxe_status check_cfg(mxe_ctx* c, const mxe_config* cfg, bool batch) {
     return MXE_OK;
 }
 
+// Buffers are cleared and filled on the context's own stream: the default
+// stream's work is not ordered before it (the stream is non-blocking), and a
+// late clear would wipe what set_bc or set_state uploaded meanwhile.
 static mxe_status alloc_common(mxe_ctx* c) {
     CK(cudaStreamCreateWithFlags(&c->own_stream, cudaStreamNonBlocking));
     c->stream = c->own_stream;
     CK(cudaMalloc(&c->U, sizeof(double) * c->nelem));
-    CK(cudaMemset(c->U, 0, sizeof(double) * c->nelem));
+    CK(cudaMemsetAsync(c->U, 0, sizeof(double) * c->nelem, c->own_stream));
     if (c->mixed) {
         CK(cudaMalloc(&c->W, sizeof(float) * c->nelem));
         CK(cudaMalloc(&c->Ws, sizeof(float) * c->nelem));
-        CK(cudaMemset(c->W, 0, sizeof(float) * c->nelem));
-        CK(cudaMemset(c->Ws, 0, sizeof(float) * c->nelem));
+        CK(cudaMemsetAsync(c->W, 0, sizeof(float) * c->nelem, c->own_stream));
+        CK(cudaMemsetAsync(c->Ws, 0, sizeof(float) * c->nelem, c->own_stream));
     } else {
         CK(cudaMalloc(&c->Us, sizeof(double) * c->nelem));
-        CK(cudaMemset(c->Us, 0, sizeof(double) * c->nelem));
+        CK(cudaMemsetAsync(c->Us, 0, sizeof(double) * c->nelem, c->own_stream));
     }
     CK(cudaMalloc(&c->stage, sizeof(double) * c->nf * c->ncell));
     CK(cudaMalloc(&c->scratch, sizeof(unsigned long long) * 8));
@@ -267,7 +270,7 @@ static mxe_status alloc_common(mxe_ctx* c) {
     CK(cudaMalloc(&c->ghost_in, sizeof(double) * 4 * GHOST_SLOTS * 14));
     CK(cudaMalloc(&c->ghost_d, sizeof(double) * 4 * GHOST_SLOTS * 14));
     memset(c->ghost_h, 0, sizeof c->ghost_h);
-    CK(cudaMemset(c->ghost_d, 0, sizeof(double) * 4 * GHOST_SLOTS * 14));
+    CK(cudaMemsetAsync(c->ghost_d, 0, sizeof(double) * 4 * GHOST_SLOTS * 14, c->own_stream));
     c->sp.sigma_lim = c->cfg.sigma_lim;
     c->sp.k_ws = c->cfg.k_ws;
     c->sp.flux = c->cfg.flux;
@@ -284,8 +287,9 @@ static mxe_status tubes_setup(mxe_ctx* c) {
     const int n = c->ntubes;
     CK(cudaMalloc(&c->tdesc_d, sizeof(TubeDesc) * n));
     CK(cudaMalloc(&c->tclk, sizeof(TubeClock) * n));
-    CK(cudaMemset(c->tclk, 0, sizeof(TubeClock) * n));
-    CK(cudaMemcpy(c->tdesc_d, c->tdesc.data(), sizeof(TubeDesc) * n, cudaMemcpyHostToDevice));
+    CK(cudaMemsetAsync(c->tclk, 0, sizeof(TubeClock) * n, c->own_stream));
+    CK(cudaMemcpyAsync(c->tdesc_d, c->tdesc.data(), sizeof(TubeDesc) * n, cudaMemcpyHostToDevice,
+                       c->own_stream));
     if (!c->mixed) return MXE_OK;
     std::vector<int> order(n);
     for (int b = 0; b < n; ++b) order[b] = b;
@@ -293,11 +297,12 @@ static mxe_status tubes_setup(mxe_ctx* c) {
         return c->tdesc[x].n / c->tdesc[x].dx > c->tdesc[y].n / c->tdesc[y].dx;
     });
     CK(cudaMalloc(&c->order_d, sizeof(int) * n));
-    CK(cudaMemcpy(c->order_d, order.data(), sizeof(int) * n, cudaMemcpyHostToDevice));
+    CK(cudaMemcpyAsync(c->order_d, order.data(), sizeof(int) * n, cudaMemcpyHostToDevice,
+                       c->own_stream));
     c->order_h = order;
     CK(cudaMalloc(&c->rates_d, sizeof(float) * n));
     CK(cudaMalloc(&c->queue_d, 2 * sizeof(int)));
-    CK(cudaMemset(c->queue_d, 0, 2 * sizeof(int)));
+    CK(cudaMemsetAsync(c->queue_d, 0, 2 * sizeof(int), c->own_stream));
     CK(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
     CK(cudaStreamCreateWithFlags(&c->fill_stream, cudaStreamNonBlocking));
     CK(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
@@ -355,7 +360,7 @@ extern "C" mxe_status mxe_create(const mxe_config* cfg, mxe_ctx** out) {
         s = tubes_setup(c);
     } else if (s == MXE_OK) {
         cudaError_t e = cudaMalloc(&c->clk, sizeof(DevClock));
-        if (e == cudaSuccess) e = cudaMemset(c->clk, 0, sizeof(DevClock));
+        if (e == cudaSuccess) e = cudaMemsetAsync(c->clk, 0, sizeof(DevClock), c->own_stream);
         if (e != cudaSuccess) s = fail(c, MXE_ECUDA, "clock: %s", cudaGetErrorString(e));
     }
     if (s != MXE_OK) {
@@ -1510,7 +1515,7 @@ extern "C" mxe_status mxe_set_dt_history(mxe_ctx* c, long long capacity) {
     c->dth_cap = 0;
     if (capacity > 0) {
         CK(cudaMalloc(&c->dth, sizeof(double) * capacity));
-        CK(cudaMemset(c->dth, 0, sizeof(double) * capacity));
+        CK(cudaMemsetAsync(c->dth, 0, sizeof(double) * capacity, c->stream));
         c->dth_cap = capacity;
     }
     return MXE_OK;

@@ -243,7 +243,9 @@ const char *mxe_last_error(const mxe_ctx *ctx);
  * precision, scheme, CFL and boundary conditions (transmissive by default);
  * each has its own state, relaxation time and clock.  mxe_set_state /
  * mxe_get_moments act on the concatenation of all tubes.  The whole batch
- * advances in one persistent launch.  MXE_FP64: one thread block per tube.
+ * advances in one persistent launch.  MXE_FP64: a team of thread blocks per
+ * tube, as many as the tubes' lengths and the device allow (a cooperative
+ * launch; with more tubes than block slots one block per tube).
  * MXE_MIXED (14-moment system): teams of CTAs (thread-block clusters of
  * 1, 2, 4 or 8 CTAs of 128 or 256 threads, see mxe_batch_autotune) take
  * tubes from a device work queue, longest expected work (cells / dx) first;
@@ -261,7 +263,8 @@ mxe_status mxe_batch_set_relaxation(mxe_ctx *ctx, int tube, int model, double ta
 mxe_status mxe_batch_get_clock(mxe_ctx *ctx, double *t, long long *steps);
 
 /* Advance every tube until its own t reaches t_end or it has taken
- * max_steps steps in this call.  MXE_FP64: one launch, one block per tube.
+ * max_steps steps in this call.  MXE_FP64: one launch (see mxe_batch_create);
+ * MXE_ETIMEOUT if the blocks of a team lost each other.
  * MXE_MIXED: one persistent launch of teams of CTAs (clusters) over a work
  * queue ordered by expected work (largest first); when the teams cannot use
  * every CTA slot of the device (clusters are placed whole within a GPU

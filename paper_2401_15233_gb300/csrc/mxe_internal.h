@@ -13,6 +13,8 @@ constexpr int GHOST_SLOTS = 1 + MAX_SPANS;     // base state + slots
 // status bits (device status word)
 constexpr unsigned ST_NONFINITE = 1u;
 constexpr unsigned ST_NONPOSITIVE = 2u;
+constexpr unsigned ST_TIMEOUT = 4u;            // a bounded wait of a tube team gave up
+constexpr int TEAM_SPIN_LIMIT = 1 << 24;       // polls of a team barrier, about 0.35 us each
 
 // Boundary side: base type and Dirichlet slots as inclusive index ranges of
 // the cells along the side (computed on the host from [lo, hi]).
@@ -81,7 +83,22 @@ struct TubeClock {
     unsigned long long n_face, n_face64;
 };
 
+// One CTA's place in an FP64 tube launch
+struct TubeTeam {
+    int tube, rank, size, pad;
+};
+
+// Barrier and reduction slots of one tube's team (zero at launch)
+struct alignas(64) TubeSync {
+    unsigned count;                 // arrivals since the launch
+    unsigned stat[3];
+    unsigned long long rate[3];     // bit pattern of a non-negative double
+};
+
 struct TubeArgs {
+    const TubeTeam* teams;          // per CTA; NULL: all CTAs work on tube 0
+    TubeSync* sync;                 // per tube
+    const unsigned* nonplanar;      // general kernel: 0 there selects the planar state (or NULL)
     double* U;                      // all tubes, FP64 conserved
     double* Us;                     // stage buffer (same layout)
     const TubeDesc* tubes;

@@ -19,8 +19,9 @@
 #include "mxe_internal.h"
 
 namespace mxe {
-extern "C" __global__ void mxe_tubes5_f64(const TubeArgs a);
-extern "C" __global__ void mxe_tubes14_f64(const TubeArgs a);
+const void* tubes_f64_kernel(int system, bool planar, int chunk);
+cudaError_t launch_tubes_f64(const void* kern, int ctas, bool coop, const TubeArgs& a,
+                             cudaStream_t st);
 int tubes_threads();
 
 constexpr int NOALLOC_MAX_CELLS = 16384;    // 14 x 16384 doubles = 1.75 MiB of stage buffer
@@ -29,6 +30,8 @@ static __device__ __align__(256) double g_stage[14 * NOALLOC_MAX_CELLS];
 static __device__ __align__(256) TubeDesc g_tube[1];
 static __device__ __align__(256) TubeClock g_clock[1];
 static __device__ __align__(256) double g_ghost[2 * 14];
+static __device__ __align__(256) TubeSync g_sync[1];
+static __device__ __align__(256) unsigned g_nonplanar[1];
 
 struct NoallocPtrs {
     bool ready = false;
@@ -36,6 +39,9 @@ struct NoallocPtrs {
     TubeDesc* tube = nullptr;
     TubeClock* clock = nullptr;
     double* ghost = nullptr;
+    TubeSync* sync = nullptr;
+    unsigned* nonplanar = nullptr;
+    int slots = 0;                  // CTAs that are resident at once
 };
 constexpr int MAX_DEVICES = 64;
 static NoallocPtrs g_ptrs[MAX_DEVICES];
@@ -56,19 +62,46 @@ static cudaError_t noalloc_ptrs(NoallocPtrs& out) {
         if ((e = cudaGetSymbolAddress((void**)&p.tube, g_tube)) != cudaSuccess) return e;
         if ((e = cudaGetSymbolAddress((void**)&p.clock, g_clock)) != cudaSuccess) return e;
         if ((e = cudaGetSymbolAddress((void**)&p.ghost, g_ghost)) != cudaSuccess) return e;
+        if ((e = cudaGetSymbolAddress((void**)&p.sync, g_sync)) != cudaSuccess) return e;
+        if ((e = cudaGetSymbolAddress((void**)&p.nonplanar, g_nonplanar)) != cudaSuccess)
+            return e;
+        int nsm = 0, per = 2;
+        if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) !=
+            cudaSuccess)
+            return e;
+        for (int system : {5, 14})
+            for (int chunk : {31, 63}) {
+                int v = 0;
+                if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                         &v, tubes_f64_kernel(system, false, chunk), tubes_threads(), 0)) !=
+                    cudaSuccess)
+                    return e;
+                per = v < per ? v : per;
+            }
+        p.slots = per * nsm;
         p.ready = true;
     }
     out = p;
     return cudaSuccess;
 }
 
-// Writes the tube descriptor and a fresh clock into the fixed arrays.  Both
-// arrive by value as kernel arguments, so no host buffer has to outlive the
-// call (a cudaMemcpyAsync from a stack variable would).
-__global__ void mxe_noalloc_init(const TubeDesc td, const TubeClock ck) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
+// Writes the tube descriptor, a fresh clock and zeroed barrier slots into the
+// fixed arrays, and finds out whether the 14-moment state in U is planar (its
+// z-odd moments 3, 6, 8, 12 zero): the march then carries the other ten, as a
+// context's does.  Everything arrives by value as kernel arguments, so no host
+// buffer has to outlive the call (a cudaMemcpyAsync from a stack variable would).
+__global__ void __launch_bounds__(1024)
+mxe_noalloc_init(const TubeDesc td, const TubeClock ck, const double* U, int system) {
+    bool np = system != 14;
+    for (int i = threadIdx.x; i < td.n && !np; i += blockDim.x)
+        np = U[3LL * td.n + i] != 0.0 || U[6LL * td.n + i] != 0.0 || U[8LL * td.n + i] != 0.0 ||
+             U[12LL * td.n + i] != 0.0;
+    np = __syncthreads_or(np);
+    if (threadIdx.x == 0) {
         g_tube[0] = td;
         g_clock[0] = ck;
+        g_sync[0] = TubeSync{};
+        g_nonplanar[0] = np ? 1u : 0u;
     }
 }
 
@@ -111,7 +144,7 @@ extern "C" mxe_status mxe_tube_run_noalloc(const mxe_config* cfg, int bc_lo, int
     td.rp = RelaxParams{tau_model, tau_ref, rho_ref, T_ref};
     TubeClock ck{};               // the clock must start from t0 with no steps and no status
     ck.t = t0;
-    mxe_noalloc_init<<<1, 32, 0, st>>>(td, ck);
+    mxe_noalloc_init<<<1, 1024, 0, st>>>(td, ck, U, cfg->system);
     if (cudaGetLastError() != cudaSuccess) return MXE_ECUDA;
 
     TubeArgs a{};
@@ -133,15 +166,27 @@ extern "C" mxe_status mxe_tube_run_noalloc(const mxe_config* cfg, int bc_lo, int
     a.cfl = cfg->cfl;
     a.t_end = t_end;
     a.max_steps = max_steps;
-    if (cfg->system == 5) mxe_tubes5_f64<<<1, tubes_threads(), 0, st>>>(a);
-    else mxe_tubes14_f64<<<1, tubes_threads(), 0, st>>>(a);
-    if (cudaGetLastError() != cudaSuccess) return MXE_ECUDA;
+    a.teams = nullptr;            // every CTA of the launch works on the one tube
+    a.sync = p.sync;
+    a.nonplanar = p.nonplanar;
+    // one CTA per 31 cells while they are all resident, else chunks of 63 in
+    // equal passes (the rule of a context's team plan)
+    int chunk = 31, ctas = (cfg->nx + 30) / 31;
+    if (ctas > p.slots) {
+        chunk = 63;
+        const int ch = (cfg->nx + 62) / 63, pass = (ch + p.slots - 1) / p.slots;
+        ctas = (ch + pass - 1) / pass;
+    }
+    if (launch_tubes_f64(tubes_f64_kernel(cfg->system, false, chunk), ctas, ctas > 1, a, st) !=
+        cudaSuccess)
+        return MXE_ECUDA;
     if (t_out || steps_out) {
         if (cudaMemcpyAsync(&ck, p.clock, sizeof ck, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
             cudaStreamSynchronize(st) != cudaSuccess)
             return MXE_ECUDA;
         if (t_out) *t_out = ck.t;
         if (steps_out) *steps_out = (int)ck.steps;
+        if (ck.status & ST_TIMEOUT) return MXE_ETIMEOUT;
         if (ck.status & ST_NONFINITE) return MXE_ENONFINITE;
     }
     return MXE_OK;

@@ -33,6 +33,40 @@ __host__ __device__ inline ParamsT<T> make_params(const SchemeParams& sp, const 
     return p;
 }
 
+// the 5-moment system (1D, FP64 only)
+struct Phys5 {
+    static constexpr int NF = 5;
+    static __host__ __device__ constexpr int ufield(int k) { return k; }
+    static __device__ __forceinline__ void cons2prim_rn(const double* U, double* Q) {
+        cons2prim5_rn(U, Q);
+    }
+    template <class T, int K>
+    static __device__ __forceinline__ void face(const T* Q, T sl, T kw, T* U, T* F, T& lo, T& hi) {
+        f64::face_5(Q, sl, kw, U, F, lo, hi);
+    }
+    template <class T>
+    static __device__ __forceinline__ T tau(const ParamsT<T>& p, const T* Q) {
+        if (p.tau_model == 1) return p.tau_ref;
+        return p.tau_ref * (p.rho_ref / Q[0]) * M<T>::sqrt_(p.T_ref / (Q[2] / Q[0]));
+    }
+    template <class T>
+    static __device__ __forceinline__ T rate_x(const T* Q, T sl, T kw) {
+        return f64::rate_5(Q, sl, kw);
+    }
+    static __device__ __forceinline__ double pressure64(const double* Q) { return Q[2]; }
+    static __device__ __forceinline__ void source64(const double* Q, double, double it,
+                                                    double* C) {
+        f64::source_5(Q, it, C);
+    }
+    static __device__ __forceinline__ bool nonpositive_x(const double* Q) {
+        return f64::le0(Q[0]) || f64::le0(Q[2]);
+    }
+    static __device__ __forceinline__ void relax_cons(double* U, const double* Q, double tau,
+                                                      double h) {
+        relax5_cons(U, Q, tau, h);
+    }
+};
+
 struct PhysGeneral {
     static constexpr int NF = 14;
     static __host__ __device__ constexpr int ufield(int k) { return k; }
@@ -90,6 +124,10 @@ struct PhysGeneral {
     static __device__ __forceinline__ void source64(const double* Q, double p, double it,
                                                     double* C) {
         f64::source_14(Q, p, it, C);
+    }
+    // density and the pressure along x (1D problems)
+    static __device__ __forceinline__ bool nonpositive_x(const double* Q) {
+        return f64::le0(Q[0]) || f64::le0(Q[4]);
     }
     static __device__ __forceinline__ bool nonpositive64(const double* Q) {
         return f64::le0(Q[0]) || f64::le0(Q[4]) || f64::le0(Q[7]) || f64::le0(Q[9]);
@@ -163,6 +201,9 @@ struct PhysPlanar {
     static __device__ __forceinline__ void source64(const double* Q, double p, double it,
                                                     double* C) {
         f64::source_p(Q, p, it, C);
+    }
+    static __device__ __forceinline__ bool nonpositive_x(const double* Q) {
+        return f64::le0(Q[0]) || f64::le0(Q[3]);
     }
     static __device__ __forceinline__ bool nonpositive64(const double* Q) {
         return f64::le0(Q[0]) || f64::le0(Q[3]) || f64::le0(Q[5]) || f64::le0(Q[6]);

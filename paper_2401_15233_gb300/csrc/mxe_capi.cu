@@ -105,8 +105,9 @@ struct mxe_ctx {
     TubeClock* tclk = nullptr;
     int* order_d = nullptr;           // mixed tubes: hand-out order (longest work first)
     std::vector<int> order_h;         // the same order on the host
-    // FP64 tubes: the teams of the launch, one plan for runs of equal step
-    // counts and one for runs to a common time
+    // tubes: the teams of the launch, one plan for runs of equal step counts
+    // and one for runs to a common time (mixed tubes: while the block shape is
+    // the library's own choice; team_ctas[0] == 0 if teams do not pay)
     TubeTeam* team_d[2] = {nullptr, nullptr};
     int team_ctas[2] = {0, 0}, team_chunk[2] = {63, 63};
     bool team_coop[2] = {false, false};
@@ -119,12 +120,13 @@ struct mxe_ctx {
     int g_lay_teams = 0, g_lay_nA = 0, g_lay_fill = 0;   // layout captured in the graph
     int tune_nt = 128, tune_cl = 1;   // block shape of the mixed tube launch
     bool tuned = false;
+    bool shape_set = false;           // the caller chose a block shape (or had it tuned)
     int nsm = 0;
     cudaStream_t cap_stream = nullptr;     // graph capture only (never executes work)
     cudaGraphExec_t gexec = nullptr;       // captured [queue reset, persistent launch]
     double g_tend = -1.0;
     int g_steps = -1, g_nt = 0, g_cl = 0;
-    bool g_planar = false;
+    bool g_planar = false, g_set = false;
     long long g_gen = -1;
     long long gen = 0;                // bumped whenever launch arguments change
     // dt history of 2D grids (steps counted from set_state)
@@ -286,34 +288,35 @@ static mxe_status alloc_common(mxe_ctx* c) {
     return MXE_OK;
 }
 
-// Teams of an FP64 tube launch.  A CTA pass advances C cells by a stage in a
+// Teams of a tube launch.  An FP64 CTA pass advances C cells by a stage in a
 // time that hardly depends on C up to 31 (two warps on two sub-partitions) or
 // 63 (four warps), so:
-//   * if one CTA per 31 cells of every tube fits in two CTAs per SM, that is
-//     the launch (C = 31): every stage is one pass;
-//   * otherwise C = 63 (fewer halo cells and idle lanes per cell) and the CTA
-//     slots, two per SM, go one after another to the tube whose time, steps x
-//     passes, is the longest (steps: equal, or proportional to 1/dx when the
-//     tubes march to a common time);
+//   * if one CTA per 31 cells (`small`) of every tube fits in two CTAs per SM,
+//     that is the launch (C = 31): every stage is one pass;
+//   * otherwise C = 63 (`large`: fewer halo cells and idle lanes per cell) and
+//     the CTA slots, two per SM, go one after another to the tube whose time,
+//     steps x passes, is the longest (steps: equal, or proportional to 1/dx
+//     when the tubes march to a common time);
 //   * with more tubes than slots every tube has one CTA and nothing waits.
+// Mixed tubes have one chunk size (126).
 // Measured on GB300 (152 SMs), per step, one CTA a tube before / teams now:
 //   5 moments, 1000 cells, first order Euler          288   ->  18.5 us
 //   14 moments, 4096 cells, MUSCL RK2, planar        8350   ->  64.7 us
 //   24 tubes of 100 .. 700 cells, MUSCL RK2, planar  1300   ->  64.6 us
-static void team_plan(const mxe_ctx* c, bool to_time, int slots, std::vector<TubeTeam>& out,
-                      int* chunk, bool* coop) {
+static void team_plan(const mxe_ctx* c, bool to_time, int slots, int small, int large,
+                      std::vector<TubeTeam>& out, int* chunk, bool* coop) {
     const int n = c->ntubes;
     std::vector<int> size(n, 1);
-    long long all31 = 0;
-    for (int b = 0; b < n; ++b) all31 += (c->tn[b] + 30) / 31;
-    *chunk = all31 <= slots ? 31 : 63;
-    if (*chunk == 31) {
-        for (int b = 0; b < n; ++b) size[b] = (c->tn[b] + 30) / 31;
+    long long all = 0;
+    for (int b = 0; b < n; ++b) all += (c->tn[b] + small - 1) / small;
+    *chunk = all <= slots ? small : large;
+    if (all <= slots) {
+        for (int b = 0; b < n; ++b) size[b] = (c->tn[b] + small - 1) / small;
     } else if (n < slots) {
         std::vector<int> ch(n), pass(n);
         std::vector<std::pair<double, int>> heap(n);
         for (int b = 0; b < n; ++b) {
-            ch[b] = pass[b] = (c->tn[b] + 62) / 63;
+            ch[b] = pass[b] = (c->tn[b] + large - 1) / large;
             heap[b] = {(to_time ? 1.0 / c->tdesc[b].dx : 1.0) * pass[b], b};
         }
         std::make_heap(heap.begin(), heap.end());
@@ -340,20 +343,24 @@ static void team_plan(const mxe_ctx* c, bool to_time, int slots, std::vector<Tub
 }
 
 static mxe_status team_plans(mxe_ctx* c) {
-    int dev = 0, nsm = 0, per = 2;
+    int dev = 0, nsm = 0, per = c->mixed ? 4 : 2;
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     for (int pl = 0; pl < 2; ++pl)
         for (int ch : {31, 63}) {
             int v = 0;
-            CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                &v, tubes_f64_kernel(c->nf, pl, ch), tubes_threads(), 0));
+            CK(c->mixed ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                              &v, tubes_mixed_kernel(pl, 128), 128, tubes_mixed_smem(pl, 128))
+                        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                              &v, tubes_f64_kernel(c->nf, pl, ch), tubes_threads(), 0));
             per = std::min(per, v);
         }
     if (per < 1) return fail(c, MXE_ECUDA, "the tube kernel does not fit on the device");
+    if (c->mixed && c->ntubes > nsm) return MXE_OK;      // one CTA a tube fills the chip
     for (int k = 0; k < 2; ++k) {
         std::vector<TubeTeam> t;
-        team_plan(c, k == 1, per * nsm, t, &c->team_chunk[k], &c->team_coop[k]);
+        team_plan(c, k == 1, per * nsm, c->mixed ? 126 : 31, c->mixed ? 126 : 63, t,
+                  &c->team_chunk[k], &c->team_coop[k]);
         c->team_ctas[k] = (int)t.size();
         CK(cudaMalloc(&c->team_d[k], sizeof(TubeTeam) * t.size()));
         CK(cudaMemcpyAsync(c->team_d[k], t.data(), sizeof(TubeTeam) * t.size(), cudaMemcpyHostToDevice,
@@ -399,7 +406,7 @@ static mxe_status tubes_setup(mxe_ctx* c) {
             CK(cudaFuncSetAttribute(tubes_mixed_kernel(pl, nt),
                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)tubes_mixed_smem(pl, nt)));
-    return MXE_OK;
+    return team_plans(c);
 }
 
 extern "C" mxe_status mxe_create(const mxe_config* cfg, mxe_ctx** out) {
@@ -992,6 +999,7 @@ struct TubeLaunch {
     int nt, cl, teams;
     int nA;              // tubes handed to the teams (order[0, nA))
     int fill;            // single-CTA fill launch over order[nA, ntubes), 0 for none
+    int plan;            // teams across the chip: the team plan to launch (else -1)
 };
 
 // Estimated steps of every tube in a run (indexed by tube): the prescribed
@@ -1091,6 +1099,7 @@ static mxe_status tube_launch_shape(mxe_ctx* c, int nt, int cl, TubeLaunch* L,
     L->smem = tubes_mixed_smem(pl, nt);
     L->nt = nt;
     L->cl = cl;
+    L->plan = -1;
     int per = 0;
     CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, L->kern, nt, L->smem));
     int teams = 0;
@@ -1118,9 +1127,27 @@ static mxe_status tube_launch_shape(mxe_ctx* c, int nt, int cl, TubeLaunch* L,
     return MXE_OK;
 }
 
+// Launch of a run: the caller's block shape, or while there is none teams
+// across the chip where the tubes are few enough.
+static mxe_status tube_launch(mxe_ctx* c, bool to_time, TubeLaunch* L,
+                              const std::vector<double>* est) {
+    const int k = to_time ? 1 : 0;
+    if (c->shape_set || c->team_ctas[k] == 0)
+        return tube_launch_shape(c, c->tune_nt, c->tune_cl, L, est);
+    const bool pl = tubes_planar(c);
+    L->kern = tubes_mixed_kernel(pl, 128);
+    L->smem = tubes_mixed_smem(pl, 128);
+    L->nt = 128;
+    L->cl = 1;
+    L->teams = L->nA = c->ntubes;
+    L->fill = 0;
+    L->plan = k;
+    return MXE_OK;
+}
+
 static cudaError_t launch_tube_grid(cudaStream_t st, const TubeLaunch& L, int cl, int nblocks,
                                     const TubeMixedArgs& a, const ParamsT<float>& p,
-                                    const MixedPolicy& mp) {
+                                    const MixedPolicy& mp, bool coop = false) {
     cudaLaunchConfig_t lc = {};
     cudaLaunchAttribute at[1];
     lc.blockDim = dim3(L.nt, 1, 1);
@@ -1132,6 +1159,11 @@ static cudaError_t launch_tube_grid(cudaStream_t st, const TubeLaunch& L, int cl
         at[0].val.clusterDim.x = cl;
         at[0].val.clusterDim.y = 1;
         at[0].val.clusterDim.z = 1;
+        lc.attrs = at;
+        lc.numAttrs = 1;
+    } else if (coop) {               // CTAs that wait for one another are all resident
+        at[0].id = cudaLaunchAttributeCooperative;
+        at[0].val.cooperative = 1;
         lc.attrs = at;
         lc.numAttrs = 1;
     }
@@ -1150,6 +1182,14 @@ static mxe_status launch_tubes_mixed(mxe_ctx* c, cudaStream_t st, const TubeMixe
     c->lay_teams = L.teams;
     c->lay_nA = L.nA;
     c->lay_fill = L.fill;
+    if (L.plan >= 0) {
+        TubeMixedArgs at = a;
+        at.teams = c->team_d[L.plan];
+        at.sync = c->sync_d;
+        CK(cudaMemsetAsync(c->sync_d, 0, sizeof(TubeSync) * c->ntubes, st));
+        CK(launch_tube_grid(st, L, 1, c->team_ctas[L.plan], at, p, mp, c->team_coop[L.plan]));
+        return MXE_OK;
+    }
     CK(cudaMemsetAsync(c->queue_d, 0, 2 * sizeof(int), st));
     if (L.fill > 0) {
         CK(cudaEventRecord(c->ev_fork, st));
@@ -1180,7 +1220,7 @@ static mxe_status run_tubes_mixed(mxe_ctx* c, int max_steps, double t_end, const
     mxe_status s;
     if (dts) {                                   // prescribed steps: direct launch
         s = tube_steps(c, ndts, INFINITY, ndts, est);
-        if (s == MXE_OK) s = tube_launch_shape(c, c->tune_nt, c->tune_cl, &L, &est);
+        if (s == MXE_OK) s = tube_launch(c, false, &L, &est);
         if (s == MXE_OK) s = upload_dts(c, dts, ndts);
         if (s != MXE_OK) return s;
         TubeMixedArgs a = tubes_mixed_args(c, ndts, INFINITY);
@@ -1189,7 +1229,8 @@ static mxe_status run_tubes_mixed(mxe_ctx* c, int max_steps, double t_end, const
         return launch_tubes_mixed(c, c->stream, a, L);
     }
     if (!c->gexec || c->g_tend != t_end || c->g_steps != max_steps || c->g_nt != c->tune_nt ||
-        c->g_cl != c->tune_cl || c->g_gen != c->gen || c->g_planar != tubes_planar(c)) {
+        c->g_cl != c->tune_cl || c->g_set != c->shape_set || c->g_gen != c->gen ||
+        c->g_planar != tubes_planar(c)) {
         if (c->gexec) {
             cudaGraphExecDestroy(c->gexec);
             c->gexec = nullptr;
@@ -1197,7 +1238,7 @@ static mxe_status run_tubes_mixed(mxe_ctx* c, int max_steps, double t_end, const
         // the team / fill division of the captured launch, from the current
         // state's step estimates
         s = tube_steps(c, max_steps, t_end, 0, est);
-        if (s == MXE_OK) s = tube_launch_shape(c, c->tune_nt, c->tune_cl, &L, &est);
+        if (s == MXE_OK) s = tube_launch(c, std::isfinite(t_end), &L, &est);
         if (s != MXE_OK) return s;
         TubeMixedArgs a = tubes_mixed_args(c, max_steps, t_end);
         CK(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
@@ -1219,6 +1260,7 @@ static mxe_status run_tubes_mixed(mxe_ctx* c, int max_steps, double t_end, const
         c->g_steps = max_steps;
         c->g_nt = c->tune_nt;
         c->g_cl = c->tune_cl;
+        c->g_set = c->shape_set;
         c->g_gen = c->gen;
         c->g_planar = tubes_planar(c);
         c->g_lay_teams = c->lay_teams;
@@ -1510,7 +1552,7 @@ extern "C" mxe_status mxe_batch_autotune(mxe_ctx* c, double t_probe, int* nt_out
     if (!(best < INFINITY)) return fail(c, MXE_ECUDA, "autotune: no block shape could be launched");
     c->tune_nt = bnt;
     c->tune_cl = bcl;
-    c->tuned = true;
+    c->tuned = c->shape_set = true;
     c->lay_nA = 0;                   // the layout of the next launch is not known yet
     if (nt_out) *nt_out = bnt;
     if (cl_out) *cl_out = bcl;
@@ -1524,7 +1566,7 @@ extern "C" mxe_status mxe_batch_get_layout(mxe_ctx* c, int* teams, int* team_tub
     if (!c->tubes || !c->mixed) return fail(c, MXE_ESTATE, "layout of an MXE_MIXED 1D context only");
     if (c->lay_nA == 0) {            // nothing launched yet: the teams alone
         TubeLaunch L;
-        mxe_status s = tube_launch_shape(c, c->tune_nt, c->tune_cl, &L);
+        mxe_status s = tube_launch(c, false, &L, nullptr);
         if (s != MXE_OK) return s;
         c->lay_teams = L.teams;
         c->lay_nA = L.nA;
@@ -1543,6 +1585,7 @@ extern "C" mxe_status mxe_batch_set_shape(mxe_ctx* c, int nt, int cl) {
         return fail(c, MXE_EINVAL, "shape must be nt in {128, 256}, cl in {1, 2, 4, 8}");
     c->tune_nt = nt;
     c->tune_cl = cl;
+    c->shape_set = true;
     c->lay_nA = 0;                   // the layout of the next launch is not known yet
     return MXE_OK;
 }

@@ -83,7 +83,7 @@ struct TubeClock {
     unsigned long long n_face, n_face64;
 };
 
-// One CTA's place in an FP64 tube launch
+// One CTA's place in a launch of tube teams
 struct TubeTeam {
     int tube, rank, size, pad;
 };
@@ -120,6 +120,8 @@ struct TubeMixedArgs {
     float* W;                       // FP32 primitives, NF fields per tube at NF * coff
     float* Ws;                      // FP32 primitives of the stage state (same layout)
     const TubeDesc* tubes;
+    const TubeTeam* teams;          // per CTA of a launch of teams across the chip (or NULL)
+    TubeSync* sync;                 // per tube, of such a launch
     const int* order;               // tube indices in the order they are handed out
     int* queue;                     // next position in `order` (zero at launch)
     TubeClock* clk;

@@ -26,39 +26,11 @@
 // a team that gives up sets ST_TIMEOUT and returns.
 #include "mxe_internal.h"
 #include "mxe_policy.cuh"
+#include "mxe_team.cuh"
 
 namespace mxe {
 
 constexpr int NTT = 128;
-
-// ---------------------------------------------------------------- team barrier
-// All threads of all `nb` CTAs; `target` counts arrivals since the launch.
-// Returns false (in every thread of the CTA) if the wait gave up.
-__device__ __forceinline__ bool team_barrier(TubeSync* s, unsigned nb, unsigned& target) {
-    __shared__ int ok;
-    if (nb == 1u) {
-        __syncthreads();
-        return true;
-    }
-    target += nb;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();                       // the CTA's writes before its arrival
-        atomicAdd(&s->count, 1u);
-        int left = TEAM_SPIN_LIMIT, good = 1;
-        unsigned v;
-        do {
-            asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(v) : "l"(&s->count) : "memory");
-            if (--left == 0) {
-                good = 0;
-                break;
-            }
-        } while ((int)(v - target) < 0);
-        ok = good;
-    }
-    __syncthreads();
-    return ok != 0;
-}
 
 // primitive state of tube cell gi (boundary ghosts included); other CTAs of
 // the team wrote it in the previous stage: read from L2

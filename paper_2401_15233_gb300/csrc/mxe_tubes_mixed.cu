@@ -18,11 +18,17 @@
 // per thread (planar states: both face states as one packed FP32 pair) and
 // updates its cells.  Cluster barriers separate the stages; the team's CFL maximum and
 // status bits are combined in the shared memory of CTA 0 of the cluster
-// (distributed shared memory).  Every wait in this file is a hardware
-// barrier reached by all threads of the team in the same order: there is no
-// spin loop.
+// (distributed shared memory).
+//
+// While the block shape is left to the library and the tubes are few, a tube's
+// team is instead one CTA per chunk, up to the whole chip: a cooperative
+// launch whose CTAs meet at the barrier of mxe_team.cuh.  One tube
+// on one CTA runs on 1/152 of the chip, pass after pass over its chunks, while
+// a stage takes 3 us for one chunk as for many side by side.  4096 cells, planar,
+// per RK2 step: 201 -> 11.5 us (33 CTAs; set-up and read-back not counted).
 #include "mxe_internal.h"
 #include "mxe_mixed_x2.cuh"
+#include "mxe_team.cuh"
 
 namespace mxe {
 
@@ -320,6 +326,55 @@ __device__ __forceinline__ void team_reduce(float r, unsigned st, unsigned& epoc
     ++epoch;
 }
 
+// The same for a team across the chip, in the slots of its TubeSync (the
+// rotation of the three slots is that of team_reduce).
+template <int NT>
+__device__ __forceinline__ bool team_reduce_grid(TubeSync* s, float r, unsigned st,
+                                                 unsigned& epoch, unsigned& target, unsigned rank,
+                                                 unsigned team, float* wred, unsigned* wst,
+                                                 float& m, unsigned& st_out) {
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) r = fmaxf(r, __shfl_xor_sync(0xffffffffu, r, o));
+    st = __reduce_or_sync(0xffffffffu, st);
+    if (lane == 0) {
+        wred[wid] = r;
+        wst[wid] = st;
+    }
+    __syncthreads();
+    float rb = wred[0];
+    unsigned sb = wst[0];
+#pragma unroll
+    for (int w = 1; w < NT / 32; ++w) {
+        rb = fmaxf(rb, wred[w]);
+        sb |= wst[w];
+    }
+    const unsigned slot = epoch++ % 3u;
+    if (team == 1u) {
+        __syncthreads();             // every thread has read the scratch
+        m = rb;
+        st_out = sb;
+        return true;
+    }
+    if (tid == 0) {
+        atomicMax(&s->rate[slot], (unsigned long long)__float_as_uint(rb));
+        if (sb) atomicOr(&s->stat[slot], sb);
+    }
+    if (!team_barrier(s, team, target)) return false;
+    m = __uint_as_float((unsigned)__ldcg(&s->rate[slot]));
+    st_out = __ldcg(&s->stat[slot]);
+    if (rank == 0 && tid == 0) {
+        const unsigned old = (slot + 2u) % 3u;
+        __stcg(&s->rate[old], 0ull);
+        __stcg(&s->stat[old], 0u);
+    }
+    return true;
+}
+
+// With a.teams the CTA belongs to the team a.teams[blockIdx.x] of one tube (128
+// threads; the same kernel, so that the stage is the same code and its result
+// the same to the bit); otherwise a cluster is a team and takes tubes from
+// the queue.
 template <class PH, int NT>
 __device__ void tubes_mixed_body(const TubeMixedArgs& a, const ParamsT<float>& p0,
                                  const MixedPolicy& mp) {
@@ -330,7 +385,11 @@ __device__ void tubes_mixed_body(const TubeMixedArgs& a, const ParamsT<float>& p
     __shared__ unsigned s_red[3], s_stat[3], s_st, s_cnt;
     __shared__ int s_tube;
     __shared__ float s_m;
-    const unsigned rank = cl_rank(), team = cl_size();
+    const bool grid = NT == 128 && a.teams;
+    const TubeTeam tm = grid ? a.teams[blockIdx.x] : TubeTeam{};
+    const unsigned rank = grid ? (unsigned)tm.rank : cl_rank();
+    const unsigned team = grid ? (unsigned)tm.size : cl_size();
+    TubeSync* sy = grid ? a.sync + tm.tube : nullptr;
     const int tid = threadIdx.x;
     if (tid == 0) {
         s_red[0] = s_red[1] = s_red[2] = 0u;
@@ -340,17 +399,29 @@ __device__ void tubes_mixed_body(const TubeMixedArgs& a, const ParamsT<float>& p
     const unsigned r_tube = cl_map(&s_tube, 0);
     float* wred = sm + LY::R_OFF;
     unsigned* wst = (unsigned*)(sm + LY::S_OFF);
-    unsigned epoch = 0;
+    unsigned epoch = 0, target = 0;
+    bool ok = true;
+    // the team's CFL maximum and status bits; false if the team's barrier gave up
+    auto reduce = [&](float r, unsigned st, float& m, unsigned& st_out) {
+        if (grid)
+            return team_reduce_grid<NT>(sy, r, st, epoch, target, rank, team, wred, wst, m, st_out);
+        team_reduce<NT>(r, st, epoch, r_red, r_stat, rank, s_red, s_stat, wred, wst, &s_m, &s_st,
+                        m, st_out);
+        return true;
+    };
     for (;;) {
-        if (rank == 0 && tid == 0) s_tube = atomicAdd(a.queue, 1);
         if (tid == 0) s_cnt = 0u;
-        cl_sync();
-        const int q = (int)cl_ld(r_tube);
-        if (q >= a.ntubes) {
-            cl_sync();               // CTA 0 stays until every CTA has read s_tube
-            return;
+        int b = tm.tube;
+        if (!grid) {
+            if (rank == 0 && tid == 0) s_tube = atomicAdd(a.queue, 1);
+            cl_sync();
+            const int q = (int)cl_ld(r_tube);
+            if (q >= a.ntubes) {
+                cl_sync();               // CTA 0 stays until every CTA has read s_tube
+                return;
+            }
+            b = a.order[q];
         }
-        const int b = a.order[q];
         const TubeDesc td = a.tubes[b];
         TubeView v;
         v.n = td.n;
@@ -389,8 +460,7 @@ __device__ void tubes_mixed_body(const TubeMixedArgs& a, const ParamsT<float>& p
         }
         float m;
         unsigned bst;
-        team_reduce<NT>(r, 0u, epoch, r_red, r_stat, rank, s_red, s_stat, wred, wst, &s_m, &s_st,
-                        m, bst);
+        ok = reduce(r, 0u, m, bst);
         double t = ck->t;
         long long steps = ck->steps;
         double last_dt = ck->last_dt;
@@ -398,7 +468,7 @@ __device__ void tubes_mixed_body(const TubeMixedArgs& a, const ParamsT<float>& p
         float* Wc = v.W;
         float* Wn = v.Ws;
         bst = 0u;
-        for (int s = 0; s < a.max_steps; ++s) {
+        for (int s = 0; ok && s < a.max_steps; ++s) {
             double dt;
             if (a.dt_fixed) {
                 if (s >= a.n_fixed) break;
@@ -415,7 +485,11 @@ __device__ void tubes_mixed_body(const TubeMixedArgs& a, const ParamsT<float>& p
             if (a.integrator == 1) {
                 tube_stage_m<PH, NT>(a, v, mp, Wc, nullptr, Wn, (float)(0.5 * dt), false, false,
                                      rank, team, sm, status, nflag);
-                cl_sync();
+                if (grid) {
+                    if (!(ok = team_barrier(sy, team, target))) break;
+                } else {
+                    cl_sync();
+                }
                 rr = tube_stage_m<PH, NT>(a, v, mp, Wn, Wc, Wc, (float)dt, true, rs, rank, team,
                                           sm, status, nflag);
                 nface += 2u;
@@ -427,8 +501,7 @@ __device__ void tubes_mixed_body(const TubeMixedArgs& a, const ParamsT<float>& p
                 Wn = tmp;
                 nface += 1u;
             }
-            team_reduce<NT>(rr, status, epoch, r_red, r_stat, rank, s_red, s_stat, wred, wst,
-                            &s_m, &s_st, m, bst);
+            if (!(ok = reduce(rr, status, m, bst))) break;
             t += dt;
             last_dt = dt;
             ++steps;
@@ -443,7 +516,8 @@ __device__ void tubes_mixed_body(const TubeMixedArgs& a, const ParamsT<float>& p
             for (int c0 = (int)rank * C; c0 < n; c0 += (int)team * C) ++nch;
             atomicAdd(&ck->n_face, (unsigned long long)nface * nch * 2ull * (C + 1));
             if (s_cnt) atomicAdd(&ck->n_face64, (unsigned long long)s_cnt);
-            if (rank == 0) {
+            if (!ok) atomicOr(&ck->status, ST_TIMEOUT);
+            if (rank == 0 && ok) {
                 ck->t = t;
                 ck->steps = steps;
                 ck->last_dt = last_dt;
@@ -451,6 +525,7 @@ __device__ void tubes_mixed_body(const TubeMixedArgs& a, const ParamsT<float>& p
                 if (bst) atomicOr(&ck->status, bst);
             }
         }
+        if (grid) return;
     }
 }
 

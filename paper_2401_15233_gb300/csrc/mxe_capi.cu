@@ -21,8 +21,6 @@
 
 namespace mxe {
 // kernels defined in the other translation units
-extern "C" __global__ void mxe_stage14_2d_f64(const Stage2DArgs a);
-extern "C" __global__ void mxe_stage14_2d_f64_planar(const Stage2DArgs a);
 extern "C" __global__ void mxe_rate14_2d(const double* U, Grid2D g, SchemeParams sp,
                                          DevClock* clk, int slot);
 extern "C" __global__ void mxe_rate14_2d_planar(const double* U, Grid2D g, SchemeParams sp,
@@ -30,7 +28,7 @@ extern "C" __global__ void mxe_rate14_2d_planar(const double* U, Grid2D g, Schem
 const void* tubes_f64_kernel(int system, bool planar, int chunk);
 cudaError_t launch_tubes_f64(const void* kern, int ctas, bool coop, const TubeArgs& a,
                              cudaStream_t st);
-size_t stage14_2d_f64_smem(bool planar);
+F64Tile f64_tile_kernel(bool planar, int tx);
 extern "C" __global__ void mxe_stage14_2d_mixed(const Stage2DArgs a, const ParamsT<float> p,
                                                 const MixedPolicy mp);
 extern "C" __global__ void mxe_stage14_2d_mixed_planar(const Stage2DArgs a,
@@ -460,18 +458,24 @@ extern "C" mxe_status mxe_create(const mxe_config* cfg, mxe_ctx** out) {
     }
     c->g.ghost = c->ghost_d;
     if (!c->tubes) {
-        cudaError_t e = c->mixed
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess)
+            e = cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, dev);
+        if (e == cudaSuccess)
+            e = c->mixed
             ? cudaFuncSetAttribute(mxe_stage14_2d_mixed, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)stage14_2d_mixed_smem(false, 2))
-            : cudaFuncSetAttribute(mxe_stage14_2d_f64, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)stage14_2d_f64_smem(false));
+            : cudaFuncSetAttribute((const void*)f64_tile_kernel(false, 15).kern,
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)f64_tile_kernel(false, 15).smem);
         if (e == cudaSuccess)
             e = c->mixed ? cudaFuncSetAttribute(mxe_stage14_2d_mixed_planar,
                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                 (int)stage14_2d_mixed_smem(true, 2))
-                         : cudaFuncSetAttribute(mxe_stage14_2d_f64_planar,
+                         : cudaFuncSetAttribute((const void*)f64_tile_kernel(true, 15).kern,
                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                (int)stage14_2d_f64_smem(true));
+                                                (int)f64_tile_kernel(true, 15).smem);
         if (e == cudaSuccess && c->mixed)
             e = cudaFuncSetAttribute(mxe_stage14_2d_mixed_planar_b3,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -863,6 +867,33 @@ static mxe_status periodic_ok(mxe_ctx* c) {
     return MXE_OK;
 }
 
+// Tile of the FP64 stage.  Time of an RK2 step on GB300 (152 SMs), us, by
+// tile, planar (general states take 1.35 to 1.45 times as long on each):
+//            24 x 24   97 x 65  128 x 128  160 x 160  200 x 200  256 x 256  512 x 512
+//   15 x 16      343       348        347        347        648        658       2531
+//    7 x  8      115       115        189        341        432        672       2577
+//    5 x  5       82       109        231        325        503        766       2977
+// that is at least `first`, and `wave` per block of the fullest SM.
+static F64Tile f64_tile(const mxe_ctx* c, bool pl) {
+    static const struct {
+        int tx;
+        long long first, wave;
+    } t[3] = {{15, 345, 322}, {7, 115, 84}, {5, 82, 46}};
+    F64Tile best{};
+    long long cost = 0;
+    for (int n = 0; n < 3; ++n) {
+        const F64Tile f = f64_tile_kernel(pl, t[n].tx);
+        const long long blocks = (long long)((c->g.nx + f.tx - 1) / f.tx) *
+                                 ((c->g.ny + f.ty - 1) / f.ty);
+        const long long w = std::max(t[n].first, (blocks + c->nsm - 1) / c->nsm * t[n].wave);
+        if (n == 0 || w < cost) {
+            cost = w;
+            best = f;
+        }
+    }
+    return best;
+}
+
 // One step of a 2D grid.  ustar (FP64 RK2 only, optional): where stage 1
 // writes U* (default: the context's stage buffer).
 static mxe_status launch_2d_step(mxe_ctx* c, double t_end, double dt_fixed,
@@ -922,17 +953,17 @@ static mxe_status launch_2d_step(mxe_ctx* c, double t_end, double dt_fixed,
         ++c->launched;
         return MXE_OK;
     }
-    auto kern = pl ? mxe_stage14_2d_f64_planar : mxe_stage14_2d_f64;
-    size_t smem = stage14_2d_f64_smem(pl);
+    const F64Tile tl = f64_tile(c, pl);
+    const dim3 gt((c->g.nx + tl.tx - 1) / tl.tx, (c->g.ny + tl.ty - 1) / tl.ty);
     if (c->cfg.integrator == MXE_RK2) {
         double* us = ustar ? ustar : c->Us;
         a.Uin = c->U; a.Ubase = c->U; a.Uout = us; a.coef = 0.5; a.final_stage = 0;
-        kern<<<grid, 256, smem, c->stream>>>(a);
+        tl.kern<<<gt, tl.threads, tl.smem, c->stream>>>(a);
         a.Uin = us; a.Ubase = c->U; a.Uout = c->U; a.coef = 1.0; a.final_stage = 1;
-        kern<<<grid, 256, smem, c->stream>>>(a);
+        tl.kern<<<gt, tl.threads, tl.smem, c->stream>>>(a);
     } else {
         a.Uin = c->U; a.Ubase = c->U; a.Uout = c->Us; a.coef = 1.0; a.final_stage = 1;
-        kern<<<grid, 256, smem, c->stream>>>(a);
+        tl.kern<<<gt, tl.threads, tl.smem, c->stream>>>(a);
         std::swap(c->U, c->Us);
     }
     CK(cudaGetLastError());

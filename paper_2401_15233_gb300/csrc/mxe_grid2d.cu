@@ -13,7 +13,9 @@
 //
 // Tile shape: 16 x 16 x-faces and 15 x 17 y-faces map onto 256 threads with
 // at most one idle thread.  The kernel is instantiated for the general
-// 14-moment state and for planar states (ten active moments).
+// 14-moment state and for planar states (ten active moments).  Grids of few
+// such tiles take one of two smaller tiles with one thread per face state
+// (stage_f64_lanes below).
 #include "mxe_internal.h"
 #include "mxe_policy.cuh"
 
@@ -108,6 +110,7 @@ __device__ __forceinline__ void face_flux_f64(const double* W, int c, int stride
     f64::riemann<NF>(UL, FL, l0, l1, UR, FR, r0, r1, p.flux, F);
 }
 
+template <int NT = NT2>
 __device__ __forceinline__ void block_max_atomic(double r, unsigned long long* dst, double* red) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -117,7 +120,7 @@ __device__ __forceinline__ void block_max_atomic(double r, unsigned long long* d
     if (lane == 0) red[wid] = r;
     __syncthreads();
     if (wid == 0) {
-        r = lane < (NT2 / 32) ? red[lane] : 0.0;
+        r = lane < (NT / 32) ? red[lane] : 0.0;
 #pragma unroll
         for (int o = 4; o > 0; o >>= 1) {
             r = f64::max_(r, __shfl_xor_sync(0xffffffffu, r, o));
@@ -138,6 +141,57 @@ __device__ __forceinline__ void advance_clock(const Stage2DArgs& a, double dt, d
         a.clk->last_dt = dt;
         if (a.dt_hist && a.clk->steps < a.dt_hist_cap) a.dt_hist[a.clk->steps] = dt;
         a.clk->steps += 1;
+    }
+}
+
+// The owned cell (gi, gj) from its residual L: the stage's state, written out,
+// and in the final stage its status bits and CFL rate (returned).
+template <class PH>
+__device__ __forceinline__ double update_cell(const Stage2DArgs& a, const ParamsT<double>& p,
+                                              double dt, int gi, int gj, const double* L) {
+    constexpr int NF = PH::NF;
+    const Grid2D& g = a.g;
+    const long long o = (long long)gj * g.pitch + gi;
+    double Un[NF];
+    bool bad = false;
+    const double cdt = mul_rn(a.coef, dt);
+#pragma unroll
+    for (int k = 0; k < NF; ++k)
+        Un[k] = add_rn(a.Ubase[o + PH::ufield(k) * g.fstride], mul_rn(cdt, L[k]));
+    if (p.tau_model != 0 && p.src_implicit) {   // point-implicit source over cdt
+        double Qv[NF];
+        PH::cons2prim_rn(Un, Qv);
+        PH::relax_cons(Un, Qv, PH::tau(p, Qv), cdt);
+    }
+#pragma unroll
+    for (int k = 0; k < NF; ++k) {
+        a.Uout[o + PH::ufield(k) * g.fstride] = Un[k];
+        bad |= !f64::is_finite(Un[k]);
+    }
+    if (!a.final_stage) return 0.0;
+    double Qn[NF];
+    PH::cons2prim_rn(Un, Qn);
+    if (PH::nonpositive64(Qn)) atomicOr(&a.clk->status, ST_NONPOSITIVE);
+    if (bad) atomicOr(&a.clk->status, ST_NONFINITE);
+    if (a.skip_rate) return 0.0;
+    double ax, ay;
+    PH::rates(Qn, p.sigma_lim, p.k_ws, ax, ay);
+    double r = ax * g.idx;
+    r = r + ay * g.idy;
+    if (!f64::ge0(r)) r = __longlong_as_double(0x7ff0000000000000ll);  // NaN -> inf
+    return r;
+}
+
+// The explicit source of a cell (zero otherwise)
+template <class PH>
+__device__ __forceinline__ void cell_source(const ParamsT<double>& p, double tau_factor,
+                                            const double* Qc, double* L) {
+    if (p.tau_model != 0 && !p.src_implicit) {
+        const double pr = PH::pressure64(Qc);
+        PH::source64(Qc, pr, f64::inv_tau(p.tau_model, tau_factor, Qc[0], pr), L);
+    } else {
+#pragma unroll
+        for (int k = 0; k < PH::NF; ++k) L[k] = 0.0;
     }
 }
 
@@ -210,13 +264,7 @@ __device__ __forceinline__ void stage_f64(const Stage2DArgs& a) {
         double Qc[NF];
 #pragma unroll
         for (int k = 0; k < NF; ++k) Qc[k] = W[k * NBOX + (cy + 2) * BX + cx + 2];
-        if (p.tau_model != 0 && !p.src_implicit) {
-            const double pr = PH::pressure64(Qc);
-            PH::source64(Qc, pr, f64::inv_tau(p.tau_model, sdt[2], Qc[0], pr), L);
-        } else {
-#pragma unroll
-            for (int k = 0; k < NF; ++k) L[k] = 0.0;
-        }
+        cell_source<PH>(p, sdt[2], Qc, L);
 #pragma unroll
         for (int k = 0; k < NF; ++k)
             L[k] -= (Fb[k * NT2 + cy * 16 + cx + 1] - Fb[k * NT2 + cy * 16 + cx]) * g.idx;
@@ -237,39 +285,8 @@ __device__ __forceinline__ void stage_f64(const Stage2DArgs& a) {
 #pragma unroll
         for (int k = 0; k < NF; ++k)
             L[k] -= (Fb[k * NT2 + (cy + 1) * TX + cx] - Fb[k * NT2 + cy * TX + cx]) * g.idy;
-        int gi = i0 + cx, gj = j0 + cy;
-        if (gi < g.nx && gj < g.ny) {
-            long long o = (long long)gj * g.pitch + gi;
-            double Un[NF];
-            bool bad = false;
-            double cdt = mul_rn(a.coef, dt);
-#pragma unroll
-            for (int k = 0; k < NF; ++k)
-                Un[k] = add_rn(a.Ubase[o + PH::ufield(k) * g.fstride], mul_rn(cdt, L[k]));
-            if (p.tau_model != 0 && p.src_implicit) {   // point-implicit source over cdt
-                double Qv[NF];
-                PH::cons2prim_rn(Un, Qv);
-                PH::relax_cons(Un, Qv, PH::tau(p, Qv), cdt);
-            }
-#pragma unroll
-            for (int k = 0; k < NF; ++k) {
-                a.Uout[o + PH::ufield(k) * g.fstride] = Un[k];
-                bad |= !f64::is_finite(Un[k]);
-            }
-            if (a.final_stage) {
-                double Qn[NF];
-                PH::cons2prim_rn(Un, Qn);
-                if (PH::nonpositive64(Qn)) atomicOr(&a.clk->status, ST_NONPOSITIVE);
-                if (bad) atomicOr(&a.clk->status, ST_NONFINITE);
-                if (!a.skip_rate) {
-                    double ax, ay;
-                    PH::rates(Qn, p.sigma_lim, p.k_ws, ax, ay);
-                    r = ax * g.idx;
-                    r = r + ay * g.idy;
-                    if (!f64::ge0(r)) r = __longlong_as_double(0x7ff0000000000000ll);  // NaN -> inf
-                }
-            }
-        }
+        const int gi = i0 + cx, gj = j0 + cy;
+        if (gi < g.nx && gj < g.ny) r = update_cell<PH>(a, p, dt, gi, gj, L);
     }
     if (a.final_stage) block_max_atomic(r, &a.clk->rate[(a.slot + 1) % 3], red);
 }
@@ -282,8 +299,143 @@ mxe_stage14_2d_f64_planar(const Stage2DArgs a) {
     stage_f64<PhysPlanar>(a);
 }
 
-size_t stage14_2d_f64_smem(bool planar) {
-    return planar ? smem_f64<NP>() : smem_f64<14>();
+// ---------------------------------------------------------------------------
+// The same stage on a smaller tile, one thread per face STATE (the two states
+// of a face in adjacent lanes, which exchange them by shuffle and form half
+// of the face's fluxes each), x and y faces side by side on different warps.
+//
+// FP64 is bound per SM (2 operations a clock), and below one warp on each of
+// the four sub-partitions by the chain of a single warp, whatever its active
+// lanes: the 15 x 16 tile has 8 warps walk through 4 face states each, and a
+// grid of a few such tiles leaves the other SMs idle meanwhile.  The 5 x 5
+// tile (30 + 30 faces: two warps of x and two of y states) is the least work
+// an SM can do in one pass; the 7 x 8 tile (64 + 63 faces, 8 warps) computes 5 % fewer
+// faces per cell.  f64_tile() in mxe_capi.cu chooses and has the times.
+// ---------------------------------------------------------------------------
+template <int TX_, int TY_, int NT_>
+struct LaneGeo {
+    static constexpr int TX = TX_, TY = TY_, NT = NT_;
+    static constexpr int BX = TX + 4, NBOX = BX * (TY + 4);
+    static constexpr int NPX = (TX + 2) * TY, NPY = TX * (TY + 2);
+    static constexpr int NFX = (TX + 1) * TY, NFY = TX * (TY + 1);
+    static constexpr int NSX = (2 * NFX + 31) / 32 * 32;          // x states, whole warps
+    static_assert(NSX + 2 * NFY <= NT && TX * TY <= NT && NT % 32 == 0, "one pass of the threads");
+};
+template <class PH, class G>
+struct LaneShared {
+    double W[PH::NF * G::NBOX];                 // primitives of the tile and its halo
+    double F[PH::NF * (G::NFX + G::NFY)];       // face fluxes
+    double ph[G::NPX + G::NPY];                 // limiters
+    double red[8], sdt[3];
+};
+
+// The pair of lanes evaluates the face between box cells c and c + stride;
+// phl points to the left cell's limiter, the right one's is dph further on.
+template <class PH, class G, int K>
+__device__ __forceinline__ void lane_face(LaneShared<PH, G>& sh, int c, const double* phl, int dph,
+                                          const ParamsT<double>& p, int face, bool valid) {
+    constexpr int NF = PH::NF, H = (NF + 1) / 2, S = K == 0 ? 1 : G::BX;
+    const bool right = threadIdx.x & 1;
+    const int b = right ? c + S : c;
+    const double h = right ? -0.25 * phl[dph] : 0.25 * phl[0];
+    double Q[NF], U[NF], F[NF], Fo[H], lo, hi;
+#pragma unroll
+    for (int k = 0; k < NF; ++k) {
+        const double* w = sh.W + k * G::NBOX + b;
+        Q[k] = f64::face_value(w[-S], w[0], w[S], h);
+    }
+    PH::template face<double, K>(Q, p.sigma_lim, p.k_ws, U, F, lo, hi);
+    f64::pair_flux<NF>(U, F, lo, hi, right, p.flux, Fo);
+    if (!valid) return;
+#pragma unroll
+    for (int k = 0; k < H; ++k)
+        if (!right) sh.F[k * (G::NFX + G::NFY) + face] = Fo[k];
+        else if (H + k < NF) sh.F[(H + k) * (G::NFX + G::NFY) + face] = Fo[k];
+}
+
+template <class PH, class G>
+__device__ __forceinline__ void stage_f64_lanes(const Stage2DArgs& a) {
+    constexpr int NF = PH::NF, NFACE = G::NFX + G::NFY;
+    __shared__ LaneShared<PH, G> sh;
+    const int tid = threadIdx.x;
+    if (tid == 0) {
+        double tt;
+        sh.sdt[0] = step_dt(a.clk, a.slot, a.cfl, a.t_end, a.dt_fixed, tt);
+        sh.sdt[1] = tt;
+    }
+    if (tid == 32)
+        sh.sdt[2] = f64::tau_factor(a.rp.model, a.rp.tau_ref, a.rp.rho_ref, a.rp.T_ref);
+    const ParamsT<double> p = make_params<double>(a.sp, a.rp);
+    const Grid2D& g = a.g;
+    const int i0 = blockIdx.x * G::TX, j0 = blockIdx.y * G::TY;
+    for (int c = tid; c < G::NBOX; c += G::NT) {
+        double Q[NF];
+        load_prim_f64<PH>(a, i0 + c % G::BX - 2, j0 + c / G::BX - 2, Q);
+#pragma unroll
+        for (int k = 0; k < NF; ++k) sh.W[k * G::NBOX + c] = Q[k];
+    }
+    __syncthreads();
+    const double dt = sh.sdt[0], t = sh.sdt[1];
+    if (a.final_stage && blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) advance_clock(a, dt, t);
+    if (!(dt > 0.0)) return;
+    for (int n = tid; n < G::NPX + G::NPY; n += G::NT) {
+        const bool x = n < G::NPX;                   // x limiters, then y limiters
+        const int m = x ? n : n - G::NPX, wd = x ? G::TX + 2 : G::TX;
+        const int c = (m / wd + (x ? 2 : 1)) * G::BX + m % wd + (x ? 1 : 2);
+        sh.ph[n] = p.order == 2
+            ? f64::limiter<NF>(sh.W, c, x ? 1 : G::BX, G::NBOX, p.limiter) : 0.0;
+    }
+    __syncthreads();
+    if (tid < G::NSX) {                              // x faces: TY rows of TX + 1
+        const int f = min(tid >> 1, G::NFX - 1), fx = f % (G::TX + 1), fy = f / (G::TX + 1);
+        lane_face<PH, G, 0>(sh, (fy + 2) * G::BX + fx + 1, sh.ph + fy * (G::TX + 2) + fx, 1, p, f,
+                            tid < 2 * G::NFX);
+    } else if (tid < G::NSX + (2 * G::NFY + 31) / 32 * 32) {     // y faces: TY + 1 rows of TX
+        const int f = min((tid - G::NSX) >> 1, G::NFY - 1), fx = f % G::TX, fy = f / G::TX;
+        lane_face<PH, G, 1>(sh, (fy + 1) * G::BX + fx + 2, sh.ph + G::NPX + f, G::TX, p,
+                            G::NFX + f, tid - G::NSX < 2 * G::NFY);
+    }
+    __syncthreads();
+    double r = 0.0;
+    if (tid < G::TX * G::TY) {
+        const int cx = tid % G::TX, cy = tid / G::TX, gi = i0 + cx, gj = j0 + cy;
+        double Qc[NF], L[NF];
+#pragma unroll
+        for (int k = 0; k < NF; ++k) Qc[k] = sh.W[k * G::NBOX + (cy + 2) * G::BX + cx + 2];
+        cell_source<PH>(p, sh.sdt[2], Qc, L);
+        const double* fx = sh.F + cy * (G::TX + 1) + cx;
+        const double* fy = sh.F + G::NFX + cy * G::TX + cx;
+#pragma unroll
+        for (int k = 0; k < NF; ++k) {
+            L[k] -= (fx[k * NFACE + 1] - fx[k * NFACE]) * g.idx;
+            L[k] -= (fy[k * NFACE + G::TX] - fy[k * NFACE]) * g.idy;
+        }
+        if (gi < g.nx && gj < g.ny) r = update_cell<PH>(a, p, dt, gi, gj, L);
+    }
+    if (a.final_stage) block_max_atomic<G::NT>(r, &a.clk->rate[(a.slot + 1) % 3], sh.red);
+}
+
+using Lane5 = LaneGeo<5, 5, 128>;
+using Lane7 = LaneGeo<7, 8, 256>;
+#define MXE_LANES(NAME, PH, G)                                                           \
+    extern "C" __global__ void __launch_bounds__(G::NT) NAME(const Stage2DArgs a) {      \
+        stage_f64_lanes<PH, G>(a);                                                       \
+    }
+MXE_LANES(mxe_stage14_2d_f64_t5, PhysGeneral, Lane5)
+MXE_LANES(mxe_stage14_2d_f64_planar_t5, PhysPlanar, Lane5)
+MXE_LANES(mxe_stage14_2d_f64_t7, PhysGeneral, Lane7)
+MXE_LANES(mxe_stage14_2d_f64_planar_t7, PhysPlanar, Lane7)
+#undef MXE_LANES
+
+F64Tile f64_tile_kernel(bool planar, int tx) {
+    if (tx == Lane5::TX)
+        return {planar ? mxe_stage14_2d_f64_planar_t5 : mxe_stage14_2d_f64_t5, Lane5::TX,
+                Lane5::TY, Lane5::NT, 0};
+    if (tx == Lane7::TX)
+        return {planar ? mxe_stage14_2d_f64_planar_t7 : mxe_stage14_2d_f64_t7, Lane7::TX,
+                Lane7::TY, Lane7::NT, 0};
+    return {planar ? mxe_stage14_2d_f64_planar : mxe_stage14_2d_f64, TX, TY, NT2,
+            planar ? smem_f64<NP>() : smem_f64<14>()};
 }
 
 // Initial CFL rate of the current state into slot `slot` of the clock.

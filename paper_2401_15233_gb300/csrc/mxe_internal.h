@@ -65,6 +65,13 @@ struct Stage2DArgs {
     int resync;                     // mixed final stage: W^{n+1} = prim(U^{n+1}) in FP64
 };
 
+// One tile variant of the FP64 2D stage kernel
+struct F64Tile {
+    void (*kern)(Stage2DArgs);
+    int tx, ty, threads;
+    size_t smem;
+};
+
 // ---- 1D tubes ----
 struct TubeDesc {
     long long off;                  // element offset of the tube's field 0

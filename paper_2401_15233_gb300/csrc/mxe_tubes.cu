@@ -54,31 +54,6 @@ __device__ __forceinline__ void load_prim_1d(const TubeArgs& a, const double* U,
     PH::cons2prim_rn(Uc, Q);
 }
 
-// Face flux from the two states of a face held by adjacent lanes (left in the
-// even lane): the lanes exchange half of their conserved states and fluxes,
-// and each forms half of the fields, the even lane [0, H), the odd lane [H, NF).
-template <int NF>
-__device__ __forceinline__ void pair_flux(const double* U, const double* F, double lo, double hi,
-                                          bool right, int flux, double* Fo) {
-    constexpr int H = (NF + 1) / 2;
-    const double plo = __shfl_xor_sync(0xffffffffu, lo, 1);
-    const double phi = __shfl_xor_sync(0xffffffffu, hi, 1);
-    double UL[H], FL[H], UR[H], FR[H];
-#pragma unroll
-    for (int k = 0; k < H; ++k) {
-        const int k1 = H + k < NF ? H + k : NF - 1;
-        const double pu = __shfl_xor_sync(0xffffffffu, right ? U[k] : U[k1], 1);
-        const double pf = __shfl_xor_sync(0xffffffffu, right ? F[k] : F[k1], 1);
-        const double ou = right ? U[k1] : U[k], of = right ? F[k1] : F[k];
-        UL[k] = right ? pu : ou;
-        FL[k] = right ? pf : of;
-        UR[k] = right ? ou : pu;
-        FR[k] = right ? of : pf;
-    }
-    f64::riemann<H>(UL, FL, right ? plo : lo, right ? phi : hi, UR, FR, right ? lo : plo,
-                    right ? hi : phi, flux, Fo);
-}
-
 template <class PH, int C>
 struct TubeShared {
     double W[PH::NF * (C + 4)];          // primitives of the chunk and its halo
@@ -124,7 +99,7 @@ __device__ __forceinline__ double tube_stage(const TubeArgs& a, const ParamsT<do
                 Q[k] = f64::face_value(w[-1], w[0], w[1], h);
             }
             PH::template face<double, 0>(Q, p.sigma_lim, p.k_ws, U, F, lo, hi);
-            pair_flux<NF>(U, F, lo, hi, right, p.flux, Fo);
+            f64::pair_flux<NF>(U, F, lo, hi, right, p.flux, Fo);
             if ((tid >> 1) <= m) {
 #pragma unroll
                 for (int k = 0; k < H; ++k)

@@ -9,17 +9,17 @@
 //   mxe_adj_prims   primitives of U_in (FP64, oracle-order rounding)
 //   mxe_adj_faces   two lanes per face, one per face state: recompute the
 //                   reconstruction and the face state once (intermediates
-//                   kept), exchange the primal outputs with the partner lane,
-//                   reverse HLL / Rusanov, the face evaluation and the MUSCL
-//                   + shared limiter; write the primitive adjoint
-//                   contributions to the four stencil cells f-2 .. f+1
+//                   kept), reverse HLL / Rusanov together with the partner
+//                   lane, then the face evaluation and the MUSCL + shared
+//                   limiter; write the primitive adjoint contributions to
+//                   the four stencil cells f-2 .. f+1
 //   mxe_adj_cells   one thread per cell: gather the contributions of the
 //                   eight faces that touch it (and of ghost cells that copy
 //                   it), reverse the BGK source and the primitive recovery
 //   mxe_adj_ghosts  contributions to Dirichlet ghost cells -> adjoint of the
 //                   imposed primitive states
 // Branches follow the primal (see mxe_adjoint.cuh).
-#include "mxe_adjoint.cuh"
+#include "mxe_adj64.cuh"
 #include "mxe_internal.h"
 #include "mxe_policy.cuh"
 
@@ -77,30 +77,48 @@ __device__ __forceinline__ const double* ghost_of(const Grid2D& g, int side, int
     return nullptr;
 }
 
-// primitive state at stencil position (i, j) (one of them may be outside)
-__device__ __forceinline__ void stencil_prim(const AdjArgs& a, int i, int j, double* Q) {
+// Primitive state at stencil position (i, j) (one of them may be outside): a
+// ghost state, or the cell it copies.
+struct PrimCell {
+    const double* p;
+    long long fs;                // 0: a ghost state (14 fields)
+    __device__ __forceinline__ double operator()(int k) const {
+        return fs ? __ldg(p + k * fs) : p[planar_field(k)];
+    }
+};
+__device__ __forceinline__ PrimCell stencil_cell(const AdjArgs& a, int i, int j) {
     const Grid2D& g = a.g;
     int slot;
     if (i < 0 || i >= g.nx) {
         const double* gs = ghost_of(g, i < 0 ? 0 : 1, j, slot);
-        if (gs) {
-#pragma unroll
-            for (int k = 0; k < NP; ++k) Q[k] = gs[planar_field(k)];
-            return;
-        }
+        if (gs) return PrimCell{gs, 0};
         i = g.side[0].type == 1 ? ((i % g.nx) + g.nx) % g.nx : (i < 0 ? 0 : g.nx - 1);
     } else if (j < 0 || j >= g.ny) {
         const double* gs = ghost_of(g, j < 0 ? 2 : 3, i, slot);
-        if (gs) {
-#pragma unroll
-            for (int k = 0; k < NP; ++k) Q[k] = gs[planar_field(k)];
-            return;
-        }
+        if (gs) return PrimCell{gs, 0};
         j = g.side[2].type == 1 ? ((j % g.ny) + g.ny) % g.ny : (j < 0 ? 0 : g.ny - 1);
     }
-    const double* p = a.P + (long long)j * g.pitch + i;
+    return PrimCell{a.P + (long long)j * g.pitch + i, g.fstride};
+}
+__device__ __forceinline__ void stencil_prim(const AdjArgs& a, int i, int j, double* Q) {
+    const PrimCell c = stencil_cell(a, i, j);
 #pragma unroll
-    for (int k = 0; k < NP; ++k) Q[k] = p[k * g.fstride];
+    for (int k = 0; k < NP; ++k) Q[k] = c(k);
+}
+// the cells c - 1, c, c + 1 of line t along K
+struct Stencil {
+    PrimCell c[3];
+    __device__ __forceinline__ double operator()(int m, int k) const {
+        return (m < 0 ? c[0] : m > 0 ? c[2] : c[1])(k);
+    }
+};
+template <int K>
+__device__ __forceinline__ Stencil stencil(const AdjArgs& a, int c, int t) {
+    Stencil s;
+#pragma unroll
+    for (int m = 0; m < 3; ++m)
+        s.c[m] = K == 0 ? stencil_cell(a, c - 1 + m, t) : stencil_cell(a, t, c - 1 + m);
+    return s;
 }
 
 extern "C" __global__ void mxe_adj_prims(const AdjArgs a) {
@@ -158,14 +176,10 @@ extern "C" __global__ void mxe_adj_limiters(const AdjArgs a) {
     } else {
         return;
     }
-    double qm[NP], q0[NP], qp[NP];
-    stencil_prim(a, K == 0 ? i - 1 : i, K == 0 ? j : j - 1, qm);
-    stencil_prim(a, i, j, q0);
-    stencil_prim(a, K == 0 ? i + 1 : i, K == 0 ? j : j + 1, qp);
-    adj::PhiAdj<double> ph{1.0, 0.0, 0.0, -1};
-    if (a.p.order == 2) ph = adj::phi_adj<double, NP>(qm, q0, qp, a.p.limiter);
-    else ph.phi = 0.0;
-    if (a.frozen_phi) ph.ks = -1;
+    adj::PhiAdj<double> ph{0.0, 0.0, 0.0, -1};
+    if (a.p.order == 2)
+        ph = f64::phi_adj_at(K == 0 ? stencil<0>(a, i, j) : stencil<1>(a, j, i), a.p.limiter,
+                             a.frozen_phi);
     float* L = K == 0 ? a.LX : a.LY;
     const float v[4] = {(float)ph.phi, (float)ph.ddm, (float)ph.ddp, (float)ph.ks};
 #pragma unroll
@@ -274,110 +288,93 @@ __device__ __forceinline__ float shfl1(float v, unsigned m = 0xffffffffu) {
 // stencil f-1..f+1).  f in [0, n_K] on line t (row j for x-faces, column i
 // for y-faces).  Threads past the last face compute the last face (the
 // shuffles need the whole warp) and write nothing.
-template <int K, class T>
+template <int K>
 __device__ __forceinline__ void adj_face_side(const AdjArgs& a, int f, int t, bool valid) {
     const Grid2D& g = a.g;
     const ParamsT<double>& p = a.p;
     const int nK = K == 0 ? g.nx : g.ny;
     const bool isL = (threadIdx.x & 1) == 0;
-    const int c0 = isL ? f - 1 : f;                      // own cell
-    // reconstruction and limiter in FP64 (differences of nearby states); the
-    // face state itself in T.  The stencil is loaded again for the
-    // reconstruction reverse rather than kept live through the face state.
-    auto load_stencil = [&](double (*Qs)[NP]) {
-#pragma unroll
-        for (int m = 0; m < 3; ++m) {
-            if (K == 0) stencil_prim(a, c0 - 1 + m, t, Qs[m]);
-            else stencil_prim(a, t, c0 - 1 + m, Qs[m]);
-        }
-    };
-    adj::PhiAdj<double> ph{0.0, 0.0, 0.0, -1};
-    const double hs = isL ? 0.5 : -0.5;
-    T Qf[NP];
-    {
-        double Qs[3][NP];
-        load_stencil(Qs);
-        if (p.order == 2) ph = adj::phi_adj<double, NP>(Qs[0], Qs[1], Qs[2], p.limiter);
-        if (a.frozen_phi) ph.ks = -1;
-#pragma unroll
-        for (int k = 0; k < NP; ++k)
-            Qf[k] = (T)muscl_face(Qs[0][k], Qs[1][k], Qs[2][k], ph.phi, hs);
-    }
-    // adjoint of the face flux: L_l -= F idx, L_r += F idx
-    const double idx = K == 0 ? g.idx : g.idy;
-    // The reverse is linear in the flux adjoint: it runs on Fb scaled by a
-    // power of two (so that FP32 cannot overflow) and the result is scaled
+    const double hs = isL ? 0.25 : -0.25;
+    // adjoint of the face flux: L_l -= F idx, L_r += F idx.  The reverse is
+    // linear in it: it runs on Fb scaled by a power of two (so that no
+    // intermediate leaves the range of a double) and the result is scaled
     // back.  A face whose flux adjoint is zero contributes nothing.
-    double Fbd[NP];
+    double Fb[NP];
+    unsigned top = 0;                                    // high word of the largest |Fb|
+    unsigned low = 0;
     {
         const int l = f - 1, r = f;
         const long long ol = K == 0 ? (long long)t * g.pitch + l : (long long)l * g.pitch + t;
         const long long orr = K == 0 ? (long long)t * g.pitch + r : (long long)r * g.pitch + t;
+        const double w = a.coef * (K == 0 ? g.idx : g.idy);
 #pragma unroll
         for (int k = 0; k < NP; ++k) {
             const long long fo = planar_field(k) * g.fstride;
             const double vl = l >= 0 ? a.V[ol + fo] : 0.0;
             const double vr = r < nK ? a.V[orr + fo] : 0.0;
-            Fbd[k] = ((vr - vl) * a.coef) * idx;
+            Fb[k] = (vr - vl) * w;
+            top = max(top, f64::hi32(Fb[k]) & 0x7fffffffu);
+            low |= f64::lo32(Fb[k]);
         }
     }
-    double fmax = 0.0;
+    const bool live = (top | low) != 0u;                 // same in both lanes of the face
+    double Qb[NP];
 #pragma unroll
-    for (int k = 0; k < NP; ++k) fmax = fmax > fabs(Fbd[k]) ? fmax : fabs(Fbd[k]);
-    const bool live = fmax > 0.0;                       // same in both lanes of the face
-    const unsigned mask = __ballot_sync(0xffffffffu, live);
-    int ex = 0;
-    if (live) frexp(fmax, &ex);
-    const double scale = ldexp(1.0, ex);
-    T Fb[NP];
-#pragma unroll
-    for (int k = 0; k < NP; ++k) Fb[k] = (T)(Fbd[k] / scale);
-    T Qb[NP];
-#pragma unroll
-    for (int k = 0; k < NP; ++k) Qb[k] = T(0);
-    auto outadj = [&](const T* U, const T* F, T lmin, T lmax, T* Ub, T* Fob, T& lminb,
-                      T& lmaxb) {
-        T Up[NP], Fp[NP];
+    for (int k = 0; k < NP; ++k) Qb[k] = 0.0;
+    adj::PhiAdj<double> ph{0.0, 0.0, 0.0, -1};
+    if (__any_sync(0xffffffffu, live)) {
+        int ex = (int)(top >> 20) - 1023;                // subnormal: -1023; Inf, NaN: no scaling
+        if (ex > 1023) ex = 0;
+        double Qf[NP];
+        const Stencil s = stencil<K>(a, isL ? f - 1 : f, t);
+        if (p.order == 2) ph = f64::phi_adj_at(s, p.limiter, a.frozen_phi);
 #pragma unroll
         for (int k = 0; k < NP; ++k) {
-            Up[k] = shfl1(U[k], mask);
-            Fp[k] = shfl1(F[k], mask);
+            Qf[k] = f64::face_value(s(-1, k), s(0, k), s(1, k), hs * ph.phi);
+            Fb[k] = f64::scale2(Fb[k], -ex);
         }
-        const T lminp = shfl1(lmin, mask), lmaxp = shfl1(lmax, mask);
-        if (isL)
-            riemann_bwd_side<K, T>(p, true, U, F, lmin, lmax, Up, Fp, lminp, lmaxp, Fb, Ub, Fob,
-                                lminb, lmaxb);
-        else
-            riemann_bwd_side<K, T>(p, false, Up, Fp, lminp, lmaxp, U, F, lmin, lmax, Fb, Ub, Fob,
-                                lminb, lmaxb);
-    };
-    if (live) adj::face_side_adj<T, K>(Qf, (T)p.sigma_lim, (T)p.k_ws, outadj, Qb);
-    // reconstruction reverse -> own stencil (bm, b0, bp)
-    double Qbd[NP], bm[NP], b0[NP], bp[NP];
+        f64::face_adj_p<K>(Qf, p.sigma_lim, p.k_ws, p.flux, Fb, live, Qb);
 #pragma unroll
-    for (int k = 0; k < NP; ++k) {
-        Qbd[k] = (double)Qb[k] * scale;
-        bm[k] = b0[k] = bp[k] = 0.0;
+        for (int k = 0; k < NP; ++k) Qb[k] = f64::scale2(Qb[k], ex);
     }
-    if (p.order == 2) {
-        double Qs[3][NP];
-        load_stencil(Qs);
-        adj::muscl_bwd<double, NP>(Qs[0], Qs[1], Qs[2], ph, hs, Qbd, bm, b0, bp);
+    // reverse of the face value q0 + h (qp - qm), h = +-phi / 4 (zero slope,
+    // and derivative, where the three cells are equal) -> own stencil (bm, b0,
+    // bp); the stencil is loaded again rather than kept live through the face
+    // state
+    double bp[NP], dm = 0.0, dp = 0.0;
+    if (p.order == 2 && live) {
+        const double h = hs * ph.phi;
+        const Stencil s = stencil<K>(a, isL ? f - 1 : f, t);
+        double phib = 0.0;
+#pragma unroll
+        for (int k = 0; k < NP; ++k) {
+            const double qm = s(-1, k), q0 = s(0, k), qp = s(1, k);
+            const bool flat = qm == q0 && q0 == qp;
+            bp[k] = flat ? 0.0 : h * Qb[k];
+            if (ph.ks >= 0) phib = fma(qp - qm, Qb[k], phib);
+        }
+        dm = hs * phib * ph.ddm;
+        dp = hs * phib * ph.ddp;
     } else {
 #pragma unroll
-        for (int k = 0; k < NP; ++k) b0[k] = Qbd[k];
+        for (int k = 0; k < NP; ++k) bp[k] = 0.0;
     }
     // slots of the face: 0 = f-2, 1 = f-1, 2 = f, 3 = f+1.  Left state: bm,
     // b0, bp -> slots 0, 1, 2; right state: slots 1, 2, 3.  Exchange the
     // overlap so that each lane writes two slots.
+    const int s0 = isL ? 0 : 2;
 #pragma unroll
     for (int k = 0; k < NP; ++k) {
-        const double send = isL ? bp[k] : bm[k];
-        const double recv = shfl1(send);
+        double m = -bp[k], c = Qb[k], q = bp[k];
+        if (k == ph.ks) {
+            m -= dm;
+            c += dm - dp;
+            q += dp;
+        }
+        const double recv = shfl1(isL ? q : m);
         if (!valid) continue;
-        const double lo = isL ? bm[k] : b0[k] + recv;   // slot 0 (L) or 2 (R)
-        const double hi = isL ? b0[k] + recv : bp[k];   // slot 1 (L) or 3 (R)
-        const int s0 = isL ? 0 : 2;
+        const double lo = isL ? m : c + recv;            // slot 0 (L) or 2 (R)
+        const double hi = isL ? c + recv : q;            // slot 1 (L) or 3 (R)
         if (K == 0) {
             a.Cx[cx_index(g, s0, k, t, f)] = lo;
             a.Cx[cx_index(g, s0 + 1, k, t, f)] = hi;
@@ -507,27 +504,34 @@ __device__ __forceinline__ void adj_face_side_f32(const AdjArgs& a, int f, int t
     }
 }
 
-// 128 threads = 64 faces of one line (x) or 64 columns of one face row (y)
-template <class T>
-__device__ __forceinline__ void faces_x(const AdjArgs& a) {
+// FP64 reverse (exact linearisation): x and y faces side by side in one
+// launch, 32 faces a block whatever their line.
+constexpr int NTA = 64;
+extern "C" __global__ void __launch_bounds__(NTA) mxe_adj_faces(const AdjArgs a, int nbx) {
+    const Grid2D& g = a.g;
+    if ((int)blockIdx.x < nbx) {
+        const int n = (g.nx + 1) * g.ny, id = blockIdx.x * (NTA / 2) + (threadIdx.x >> 1);
+        const int f = min(id, n - 1);
+        adj_face_side<0>(a, f % (g.nx + 1), f / (g.nx + 1), id < n);
+    } else {
+        const int n = g.nx * (g.ny + 1);
+        const int id = (blockIdx.x - nbx) * (NTA / 2) + (threadIdx.x >> 1), f = min(id, n - 1);
+        adj_face_side<1>(a, f / g.nx, f % g.nx, id < n);
+    }
+}
+// FP32 reverse (the face states recomputed and reversed in FP32 from per-cell
+// FP32 data): 128 threads = 64 faces of one line (x) or 64 columns of one face
+// row (y)
+extern "C" __global__ void __launch_bounds__(128) mxe_adj_faces_x_f32(const AdjArgs a) {
     const int f = blockIdx.x * 64 + (threadIdx.x >> 1), j = blockIdx.y;
     const bool valid = f <= a.g.nx;
-    if (sizeof(T) == 4) adj_face_side_f32<0>(a, valid ? f : a.g.nx, j, valid);
-    else adj_face_side<0, T>(a, valid ? f : a.g.nx, j, valid);
+    adj_face_side_f32<0>(a, valid ? f : a.g.nx, j, valid);
 }
-template <class T>
-__device__ __forceinline__ void faces_y(const AdjArgs& a) {
+extern "C" __global__ void __launch_bounds__(128) mxe_adj_faces_y_f32(const AdjArgs a) {
     const int i = blockIdx.x * 64 + (threadIdx.x >> 1), f = blockIdx.y;
     const bool valid = i < a.g.nx;
-    if (sizeof(T) == 4) adj_face_side_f32<1>(a, f, valid ? i : a.g.nx - 1, valid);
-    else adj_face_side<1, T>(a, f, valid ? i : a.g.nx - 1, valid);
+    adj_face_side_f32<1>(a, f, valid ? i : a.g.nx - 1, valid);
 }
-// FP64 reverse (exact linearisation) and FP32 reverse (the face states
-// recomputed and reversed in FP32 from per-cell FP32 data)
-extern "C" __global__ void __launch_bounds__(128) mxe_adj_faces_x(const AdjArgs a) { faces_x<double>(a); }
-extern "C" __global__ void __launch_bounds__(128) mxe_adj_faces_y(const AdjArgs a) { faces_y<double>(a); }
-extern "C" __global__ void __launch_bounds__(128) mxe_adj_faces_x_f32(const AdjArgs a) { faces_x<float>(a); }
-extern "C" __global__ void __launch_bounds__(128) mxe_adj_faces_y_f32(const AdjArgs a) { faces_y<float>(a); }
 
 // Sum of the x-face contributions to stencil position (v, j): slot s of face
 // f targets cell f - 2 + s.
@@ -612,12 +616,14 @@ extern "C" __global__ void __launch_bounds__(128) mxe_adj_cells(const AdjArgs a)
             double W[NP];
 #pragma unroll
             for (int k = 0; k < NP; ++k) W[k] = a.coef * a.V[o + planar_field(k) * g.fstride];
-            taub = adj::source_p_bwd(a.p.tau_model, a.p.tau_ref, a.p.rho_ref, a.p.T_ref, Q, W, Qb);
+            const double it = f64::inv_tau(
+                a.p.tau_model,
+                f64::tau_factor(a.p.tau_model, a.p.tau_ref, a.p.rho_ref, a.p.T_ref), Q[0],
+                PhysPlanar::pressure64(Q));
+            taub = f64::source_rev_p(a.p.tau_model, it, a.p.tau_ref, Q, W, Qb);
         }
         double Ub[NP];
-#pragma unroll
-        for (int k = 0; k < NP; ++k) Ub[k] = 0.0;
-        adj::cons2prim_p_bwd(Q, Qb, Ub);
+        f64::cons2prim_rev_p(Q, Qb, Ub);
 #pragma unroll
         for (int k = 0; k < 14; ++k) {
             const long long ok = o + k * g.fstride;
@@ -727,8 +733,9 @@ cudaError_t adj_stage(const double* U, const double* V, double coef, const doubl
         mxe_adj_faces_x_f32<<<dim3((g.nx + 1 + 63) / 64, g.ny), 128, 0, st>>>(a);
         mxe_adj_faces_y_f32<<<dim3((g.nx + 63) / 64, g.ny + 1), 128, 0, st>>>(a);
     } else {
-        mxe_adj_faces_x<<<dim3((g.nx + 1 + 63) / 64, g.ny), 128, 0, st>>>(a);
-        mxe_adj_faces_y<<<dim3((g.nx + 63) / 64, g.ny + 1), 128, 0, st>>>(a);
+        const int nbx = ((g.nx + 1) * g.ny + NTA / 2 - 1) / (NTA / 2);
+        const int nby = (g.nx * (g.ny + 1) + NTA / 2 - 1) / (NTA / 2);
+        mxe_adj_faces<<<nbx + nby, NTA, 0, st>>>(a, nbx);
     }
     mxe_adj_ghosts<<<(4 * (g.nx + g.ny) + 127) / 128, 128, 0, st>>>(a);
     mxe_adj_cells<<<cg, 128, 0, st>>>(a);

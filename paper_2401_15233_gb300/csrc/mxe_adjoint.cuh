@@ -1,8 +1,8 @@
 // mxe_adjoint.cuh -- hand-written reverse mode (discrete adjoint) of the
-// planar 14-moment point physics in FP64: primitive recovery, the
-// interpolative closure (Sec. 2.4), the K-flux, the wave-speed fit
-// (Sec. 5), the BGK source with its local relaxation time, and the HLL /
-// Rusanov face flux (Sec. 3.1).
+// planar 14-moment face state, as the FP32 reverse runs it (FP64, the BGK
+// source and the primitive recovery: mxe_adj64.cuh): the interpolative
+// closure (Sec. 2.4), the K-flux, the wave-speed fit (Sec. 5) and the MUSCL
+// face value.
 //
 // Every *_bwd function recomputes the primal intermediates it needs with the
 // forward formulas of mxe_planar.cuh, then propagates adjoints in reverse
@@ -280,15 +280,6 @@ __device__ __forceinline__ void lam_p_rev(const LamP<T>& L, T sb, T lpb, T lmb,
         gb.qy += qdb;
         gb.qx += qperpb * sgn;
     }
-}
-
-// Reverse of lam_p<K> (recomputing its intermediates).
-template <class T, int K>
-__device__ __forceinline__ void lam_p_bwd(const DimlessP<T>& g, T sb, T lpb,
-                                          T lmb, DimlessBar<T>& gb, T& sbb) {
-    LamP<T> L;
-    lam_p_fwd<T, K>(g, sb, L);
-    lam_p_rev<T, K>(L, sb, lpb, lmb, gb, sbb);
 }
 
 // Intermediates of closure_p<K> (recomputed for the reverse sweep).
@@ -653,42 +644,6 @@ __device__ __forceinline__ void prim2cons_p_bwd(const T* Q, const T* Ub, T* Qb) 
     Qb[7] += qxb; Qb[8] += qyb; Qb[9] += Ub[9];
 }
 
-// Reverse of face_eval_p<K>: adjoints of (U, F, lmin, lmax) of one face
-// state -> Qb (added).
-template <class T, int K>
-__device__ __forceinline__ void face_eval_p_bwd(const T* Q, T sl, T kw,
-                                                const T* Ubar_in, const T* Fb,
-                                                T lminb, T lmaxb, T* Qb) {
-    DimlessP<T> g;
-    dimless_p(Q, g);
-    const T sb = clamp_sigma(g.sig, sl);
-    CloP<T> c;
-    T QK[4], RK[2], SK;
-    closure_p_fwd<T, K>(Q, g, sb, c, QK, RK, SK);
-    T U[NP];
-    prim2cons_p(Q, U);
-    T lp, lm;
-    lam_p<T, K>(g, sb, lp, lm);
-    DimlessBar<T> gb;
-    gb.zero();
-    T sbb = T(0.0);
-    // lmax = u_K + k lp sq, lmin = u_K + k lm sq
-    Qb[1 + K] += lmaxb + lminb;
-    gb.sq += kw * (lmaxb * lp + lminb * lm);
-    const T lpb = lmaxb * kw * g.sq, lmb = lminb * kw * g.sq;
-    // flux
-    T Ub[NP];
-#pragma unroll
-    for (int n = 0; n < NP; ++n) Ub[n] = Ubar_in[n];
-    T QKb[4] = {T(0.0), T(0.0), T(0.0), T(0.0)}, RKb[2] = {T(0.0), T(0.0)}, SKb = T(0.0);
-    flux_p_bwd<T, K>(Q, U, QK, RK, Fb, Qb, Ub, QKb, RKb, SKb);
-    prim2cons_p_bwd(Q, Ub, Qb);
-    closure_p_bwd<T, K>(Q, g, sb, c, QKb, RKb, SKb, gb, sbb, Qb);
-    lam_p_bwd<T, K>(g, sb, lpb, lmb, gb, sbb);
-    if (!(g.sig < sl) && !(g.sig > T(1.0))) gb.sig += sbb;
-    dimless_p_bwd(Q, g, gb, Qb);
-}
-
 // One face state evaluated once and reversed: the primal outputs (U, F,
 // lmin, lmax) are handed to `outadj`, which returns their adjoints (the
 // numerical-flux reverse needs both states of the face); the reverse then
@@ -726,130 +681,6 @@ __device__ __forceinline__ void face_side_adj(const T* Q, T sl, T kw,
     dimless_p_bwd(Q, g, gb, Qb);
 }
 
-// Reverse of source_p with the local relaxation time tau_p: W = adjoint of
-// the source vector C -> Qb; returns the adjoint of tau_ref.
-template <class T>
-__device__ __forceinline__ T source_p_bwd(int model, T tau_ref, T rho_ref,
-                                               T T_ref, const T* Q, const T* W,
-                                               T* Qb) {
-    const T rho = Q[0], ux = Q[1], uy = Q[2];
-    const T Pxx = Q[3], Pxy = Q[4], Pyy = Q[5], Pzz = Q[6];
-    const T qx = Q[7], qy = Q[8], R = Q[9];
-    const T tau = tau_p(model, tau_ref, rho_ref, T_ref, Q);
-    const T p = (Pxx + Pyy + Pzz) / T(3.0);
-    const T Pux = Pxx * ux + Pxy * uy, Puy = Pxy * ux + Pyy * uy;
-    const T uPu = ux * Pux + uy * Puy, uq = ux * qx + uy * qy, u2 = ux * ux + uy * uy;
-    // C_k = -N_k / tau
-    const T N[10] = {T(0.0), T(0.0), T(0.0), Pxx - p, Pxy, Pyy - p, Pzz - p,
-                          T(2.0) * Pux + qx - T(2.0) * ux * p, T(2.0) * Puy + qy - T(2.0) * uy * p,
-                          (T(4.0) * uPu + T(4.0) * uq + R) - (T(4.0) * u2 * p + T(15.0) * p * p / rho)};
-    T WN = T(0.0);
-#pragma unroll
-    for (int k = 3; k < NP; ++k) WN += W[k] * N[k];
-    const T itau = T(1.0) / tau;
-    const T taub = WN * itau * itau;
-    T n[NP];
-#pragma unroll
-    for (int k = 0; k < NP; ++k) n[k] = -W[k] * itau;
-    T rhob = T(0.0), uxb = T(0.0), uyb = T(0.0), pb = T(0.0), u2b = T(0.0);
-    T Pxxb = n[3], Pxyb = n[4], Pyyb = n[5], Pzzb = n[6];
-    pb -= n[3] + n[5] + n[6];
-    T qxb = n[7], qyb = n[8], Rb = n[9];
-    const T uPub = T(4.0) * n[9], uqb = T(4.0) * n[9];
-    u2b -= T(4.0) * p * n[9];
-    pb -= (T(4.0) * u2 + T(30.0) * p / rho) * n[9];
-    rhob += T(15.0) * p * p / (rho * rho) * n[9];
-    T Puxb = T(2.0) * n[7], Puyb = T(2.0) * n[8];
-    uxb -= T(2.0) * p * n[7];
-    uyb -= T(2.0) * p * n[8];
-    pb -= T(2.0) * ux * n[7] + T(2.0) * uy * n[8];
-    uxb += uqb * qx + uPub * Pux;
-    uyb += uqb * qy + uPub * Puy;
-    qxb += uqb * ux;
-    qyb += uqb * uy;
-    Puxb += uPub * ux;
-    Puyb += uPub * uy;
-    Pxyb += Puyb * ux + Puxb * uy;
-    Pyyb += Puyb * uy;
-    Pxxb += Puxb * ux;
-    uxb += Puyb * Pxy + Puxb * Pxx;
-    uyb += Puyb * Pyy + Puxb * Pxy;
-    uxb += T(2.0) * ux * u2b;
-    uyb += T(2.0) * uy * u2b;
-    T tau_refb;
-    if (model == 1) {
-        tau_refb = taub;
-    } else {
-        // tau = tau_ref (rho_ref / rho) sqrt(T_ref / T), T = tr P / (3 rho)
-        const T Tt = (Pxx + Pyy + Pzz) / (T(3.0) * rho);
-        const T Tb = -taub * tau / (T(2.0) * Tt);
-        rhob += -taub * tau / rho - Tb * Tt / rho;
-        const T trb = Tb / (T(3.0) * rho);
-        Pxxb += trb; Pyyb += trb; Pzzb += trb;
-        tau_refb = taub * tau / tau_ref;
-    }
-    Pxxb += pb / T(3.0); Pyyb += pb / T(3.0); Pzzb += pb / T(3.0);
-    Qb[0] += rhob; Qb[1] += uxb; Qb[2] += uyb;
-    Qb[3] += Pxxb; Qb[4] += Pxyb; Qb[5] += Pyyb; Qb[6] += Pzzb;
-    Qb[7] += qxb; Qb[8] += qyb; Qb[9] += Rb;
-    return tau_refb;
-}
-
-// Reverse of the planar primitive recovery Q = prim(U): Qb -> Ub (added).
-template <class T>
-__device__ __forceinline__ void cons2prim_p_bwd(const T* Q, const T* Qbar, T* Ub) {
-    const T rho = Q[0], ux = Q[1], uy = Q[2];
-    const T Pxx = Q[3], Pxy = Q[4], Pyy = Q[5], Pzz = Q[6];
-    const T qx = Q[7], qy = Q[8];
-    const T u2 = ux * ux + uy * uy, trP = Pxx + Pyy + Pzz;
-    T rhob = Qbar[0], uxb = Qbar[1], uyb = Qbar[2];
-    T Pxxb = Qbar[3], Pxyb = Qbar[4], Pyyb = Qbar[5], Pzzb = Qbar[6];
-    T qxb = Qbar[7], qyb = Qbar[8];
-    const T Rb = Qbar[9];
-    // R = U9 - rho u2^2 - 2 u2 trP - 4 uPu - 4 uq
-    Ub[9] += Rb;
-    rhob -= Rb * u2 * u2;
-    T u2b = -Rb * (T(2.0) * rho * u2 + T(2.0) * trP);
-    T trPb = -T(2.0) * u2 * Rb;
-    const T uPub = -T(4.0) * Rb, uqb = -T(4.0) * Rb;
-    uxb += uqb * qx;
-    qxb += uqb * ux;
-    uyb += uqb * qy;
-    qyb += uqb * uy;
-    uxb += uPub * (T(2.0) * ux * Pxx + T(2.0) * uy * Pxy);
-    uyb += uPub * (T(2.0) * ux * Pxy + T(2.0) * uy * Pyy);
-    Pxxb += uPub * ux * ux;
-    Pxyb += T(2.0) * uPub * ux * uy;
-    Pyyb += uPub * uy * uy;
-    // q_i = U_i - rho u_i u2 - u_i trP - 2 (P u)_i
-    Ub[7] += qxb;
-    Ub[8] += qyb;
-    rhob -= qxb * ux * u2 + qyb * uy * u2;
-    uxb -= qxb * (rho * u2 + trP + T(2.0) * Pxx) + T(2.0) * qyb * Pxy;
-    uyb -= qyb * (rho * u2 + trP + T(2.0) * Pyy) + T(2.0) * qxb * Pxy;
-    u2b -= qxb * rho * ux + qyb * rho * uy;
-    trPb -= qxb * ux + qyb * uy;
-    Pxxb -= T(2.0) * qxb * ux;
-    Pxyb -= T(2.0) * qxb * uy + T(2.0) * qyb * ux;
-    Pyyb -= T(2.0) * qyb * uy;
-    Pxxb += trPb; Pyyb += trPb; Pzzb += trPb;
-    uxb += T(2.0) * ux * u2b;
-    uyb += T(2.0) * uy * u2b;
-    // P_ij = U_ij - rho u_i u_j
-    Ub[6] += Pzzb;
-    Ub[5] += Pyyb;
-    Ub[4] += Pxyb;
-    Ub[3] += Pxxb;
-    rhob -= Pyyb * uy * uy + Pxyb * ux * uy + Pxxb * ux * ux;
-    uyb -= T(2.0) * rho * uy * Pyyb + rho * ux * Pxyb;
-    uxb -= rho * uy * Pxyb + T(2.0) * rho * ux * Pxxb;
-    // u_i = U_i / rho
-    Ub[2] += uyb / rho;
-    Ub[1] += uxb / rho;
-    rhob -= (uyb * uy + uxb * ux) / rho;
-    Ub[0] += rhob;
-}
-
 // Shared limiter with its selected field and the partial derivatives of
 // phi_{k*} with respect to dm and dp (zero when no field sets phi).
 template <class T>
@@ -857,55 +688,6 @@ struct PhiAdj {
     T phi, ddm, ddp;
     int ks;
 };
-
-// Shared limiter from the stencil differences dm = q0 - qm, dp = qp - q0.
-// A flat field (the flat test against the centre cell fr) has phi_k = 1 and
-// never sets phi.
-template <class T, int NF>
-__device__ __forceinline__ PhiAdj<T> phi_adj_d(const T* dm, const T* dp, int lim,
-                                               const FlatRef<T>& fr) {
-    PhiAdj<T> r{T(1.0), T(0.0), T(0.0), -1};
-#pragma unroll
-    for (int k = 0; k < NF; ++k) {
-        const T pk = phi_field(dm[k], dp[k], lim);
-        if (pk < r.phi && !field_flat<NF>(fr, k, abs_max(dm[k], dp[k]))) {
-            r.phi = pk;
-            r.ks = k;
-            if (mul_rn(dm[k], dp[k]) > T(0.0)) {
-                if (lim == 1) {
-                    const T s = dm[k] * dm[k] + dp[k] * dp[k];
-                    r.ddm = T(2.0) * dp[k] * (dp[k] * dp[k] - dm[k] * dm[k]) / (s * s);
-                    r.ddp = T(2.0) * dm[k] * (dm[k] * dm[k] - dp[k] * dp[k]) / (s * s);
-                } else {
-                    const T am = fabs(dm[k]), ap = fabs(dp[k]), s = am + ap;
-                    const T sm = dm[k] > T(0.0) ? T(1.0) : T(-1.0);
-                    const T sp = dp[k] > T(0.0) ? T(1.0) : T(-1.0);
-                    if (am < ap) {
-                        r.ddm = sm * T(2.0) * ap / (s * s);
-                        r.ddp = -sp * T(2.0) * am / (s * s);
-                    } else {
-                        r.ddp = sp * T(2.0) * am / (s * s);
-                        r.ddm = -sm * T(2.0) * ap / (s * s);
-                    }
-                }
-            } else {
-                r.ddm = r.ddp = T(0.0);      // constant branch
-            }
-        }
-    }
-    return r;
-}
-
-template <class T, int NF>
-__device__ __forceinline__ PhiAdj<T> phi_adj(const T* qm, const T* q0, const T* qp, int lim) {
-    T dm[NF], dp[NF];
-#pragma unroll
-    for (int k = 0; k < NF; ++k) {
-        dm[k] = q0[k] - qm[k];
-        dp[k] = qp[k] - q0[k];
-    }
-    return phi_adj_d<T, NF>(dm, dp, lim, flat_ref<NF>(q0, 1));
-}
 
 // Reverse of the MUSCL face value qf = q0 + hs (phi cen), cen = (dm + dp)/2,
 // phi = phi_{k*}(dm, dp), dm = q0 - qm, dp = qp - q0: adjoint qfb ->
@@ -937,19 +719,6 @@ __device__ __forceinline__ void muscl_bwd_d(const T* dm, const T* dp, const PhiA
                 bp[k] += dpb;
             }
     }
-}
-
-template <class T, int NF>
-__device__ __forceinline__ void muscl_bwd(const T* qm, const T* q0, const T* qp,
-                                          const PhiAdj<T>& ph, T hs, const T* qfb, T* bm, T* b0,
-                                          T* bp) {
-    T dm[NF], dp[NF];
-#pragma unroll
-    for (int k = 0; k < NF; ++k) {
-        dm[k] = q0[k] - qm[k];
-        dp[k] = qp[k] - q0[k];
-    }
-    muscl_bwd_d<T, NF>(dm, dp, ph, hs, qfb, bm, b0, bp);
 }
 
 }  // namespace adj

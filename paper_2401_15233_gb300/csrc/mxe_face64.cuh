@@ -538,10 +538,19 @@ __device__ __forceinline__ PhiScreen phi_screen(double dm, double dp) {
     return o;
 }
 
-template <int NF>
-__device__ __forceinline__ double limiter(const double* W, int c, int stride, int fs, int lim) {
-    const double* w0 = W + c;
-    const FlatRef<double> fr = flat_ref<NF>(w0, fs);
+// at(m, k): field k of the stencil cell m = -1, 0, 1; ks: the field that sets
+// phi where its derivative there is not zero (else -1).
+template <int NF, class At>
+__device__ __forceinline__ double limiter_at(const At& at, int lim, int& ks) {
+    ks = -1;
+    FlatRef<double> fr;
+    {
+        constexpr int p1 = NF == 5 ? 2 : NF == 10 ? 3 : 4, p2 = NF == 10 ? 5 : 7,
+                      p3 = NF == 10 ? 6 : 9;
+        fr.rho = at(0, 0);
+        fr.s = at(0, p1);
+        if (NF != 5) fr.s = add_rn(add_rn(fr.s, at(0, p2)), at(0, p3));
+    }
     // flat tolerances T x natural scale in FP32 (p = s or s / 3); a class whose
     // tolerance leaves FP32's range is left to the exact test (thr = -1)
     float thr[5];
@@ -560,8 +569,7 @@ __device__ __forceinline__ double limiter(const double* W, int c, int stride, in
     bool zero = false;
 #pragma unroll
     for (int k = 0; k < NF; ++k) {
-        const double* w = w0 + k * fs;
-        const PhiScreen s = phi_screen(w[0] - w[-stride], w[stride] - w[0]);
+        const PhiScreen s = phi_screen(at(0, k) - at(-1, k), at(1, k) - at(0, k));
         const float t = thr[flat_class<NF>(k)];
         const bool known = t > 0.0f && s.mx < 1e37f;
         const bool flat = known && s.mx < 0.9999f * t, rough = known && s.mx > 1.0001f * t;
@@ -582,12 +590,22 @@ __device__ __forceinline__ double limiter(const double* W, int c, int stride, in
     while (cand) {
         const int k = __ffs((int)cand) - 1;
         cand &= cand - 1u;
-        const double* w = w0 + k * fs;
-        const double dm = w[0] - w[-stride], dp = w[stride] - w[0];
+        const double dm = at(0, k) - at(-1, k), dp = at(1, k) - at(0, k);
         const double pk = phi_field(dm, dp, lim);
-        if (lt(pk, phi) && !field_flat_at<NF>(fr, k, max_(abs_(dm), abs_(dp)))) phi = pk;
+        if (lt(pk, phi) && !field_flat_at<NF>(fr, k, max_(abs_(dm), abs_(dp)))) {
+            phi = pk;
+            ks = k;
+        }
     }
+    if (phi == 0.0) ks = -1;
     return phi;
+}
+// the cell c of fields fs apart, neighbours at +- stride
+template <int NF>
+__device__ __forceinline__ double limiter(const double* W, int c, int stride, int fs, int lim) {
+    int ks;
+    const double* w = W + c;
+    return limiter_at<NF>([=](int m, int k) { return w[k * fs + m * stride]; }, lim, ks);
 }
 
 // MUSCL face value Q0 + sgn/2 phi (Qp - Qm)/2, h = sgn phi / 4

@@ -51,6 +51,7 @@ extern "C" __global__ void mxe_rate14_2d_mixed_planar(const float* W, Grid2D g,
                                                       DevClock* clk, int slot);
 size_t stage14_2d_mixed_smem(bool planar, int blocks_per_sm);
 size_t stage14_2d_mixed_x2_smem();
+int stage14_2d_mixed_x2_threads();
 int stage14_2d_mixed_x2_tile_x();
 int stage14_2d_mixed_x2_tile_y();
 const void* tubes_mixed_kernel(bool planar, int nt);
@@ -932,7 +933,8 @@ static mxe_status launch_2d_step(mxe_ctx* c, double t_end, double dt_fixed,
             }
             const int tx = stage14_2d_mixed_x2_tile_x(), ty = stage14_2d_mixed_x2_tile_y();
             dim3 gp((c->g.nx + tx - 1) / tx, (c->g.ny + ty - 1) / ty);
-            mxe_stage14_2d_mixed_planar_x2<<<gp, 256, stage14_2d_mixed_x2_smem(), c->stream>>>(
+            mxe_stage14_2d_mixed_planar_x2<<<gp, stage14_2d_mixed_x2_threads(),
+                                             stage14_2d_mixed_x2_smem(), c->stream>>>(
                 a, fparams(c), c->mp);
         };
         a.Ubase = c->U;

@@ -23,6 +23,7 @@
 // planar (ten-moment) state.
 #include "mxe_internal.h"
 #include "mxe_mixed_x2.cuh"
+#include "mxe_rate32.cuh"
 
 namespace mxe {
 
@@ -186,9 +187,9 @@ __device__ __forceinline__ void block_max_atomic_m(float r, unsigned long long* 
     if (lane == 0) red[wid] = r;
     __syncthreads();
     if (wid == 0) {
-        r = lane < (NTm / 32) ? red[lane] : 0.0f;
+        r = lane < (int)(blockDim.x >> 5) ? red[lane] : 0.0f;
 #pragma unroll
-        for (int o = 4; o > 0; o >>= 1) r = fmaxf(r, __shfl_xor_sync(0xffffffffu, r, o));
+        for (int o = 8; o > 0; o >>= 1) r = fmaxf(r, __shfl_xor_sync(0xffffffffu, r, o));
         if (lane == 0)
             atomicMax(dst, (unsigned long long)__double_as_longlong((double)r));
     }
@@ -459,19 +460,33 @@ mxe_stage14_2d_mixed_planar_b3(const Stage2DArgs a, const ParamsT<float> p,
 }
 
 // ---------------------------------------------------------------------------
-// Packed planar stage (the default for planar states).  A block of NTP
+// Packed planar stage (the default for planar states).  A block of 320
 // threads owns a TX x TY tile; every thread evaluates up to two x faces and
 // two y faces as packed pairs of face states, the limiters of about two
 // cells (both directions of an interior cell in one evaluation), and
-// updates up to two cells.  The tile is 31 x 15: a row of 32 x faces is one
+// updates up to two cells.  The tile is 31 x 18: a row of 32 x faces is one
 // warp (no shared-memory bank conflicts in the face phase), the owned cells
 // of a warp sit in one or two rows (124-byte segments of each field in
-// global memory), and against the 15 x 16 tile of the scalar kernels the
-// halo cells loaded, the limiters evaluated and the faces computed twice
-// per owned cell, and the per-block fixed work, are about halved.
-template <int TX_, int TY_>
+// global memory), and few halo cells are loaded and limited.
+//
+// What bounds it is instruction issue, so registers go before occupancy: two
+// blocks of ten warps an SM leave 96 registers a thread, at which the face
+// evaluation hardly spills.  4096 x 4096 RK2 step:
+//   31 x 15, 256 threads, 3 blocks, 80 registers  3.91 ms (3.79 with the wave
+//                                                 speeds last)
+//   31 x 15, 256 threads, 2 blocks, 128           3.50
+//   31 x 23, 256 threads, 2 blocks, 128           3.50
+//   31 x 11, 192 threads, 3 blocks, 96            3.42
+//   31 x 19, 320 threads, 2 blocks, 96            3.36
+//   31 x  7, 128 threads, 4 blocks, 128           3.81
+//   31 x  9, 160 threads, 4 blocks, 96            3.84
+//   31 x 11, 192 threads, 4 blocks, 80            4.21
+// 31 x 18 leaves no limiter for a third pass over the threads but 16 and fits
+// 1024 x 1024 in whole waves (3.45 ms and 243 us with the accurate CFL rates;
+// 261 us before).
+template <int TX_, int TY_, int NT_>
 struct TileGeo {
-    static constexpr int TX = TX_, TY = TY_;
+    static constexpr int TX = TX_, TY = TY_, NT = NT_;
     static constexpr int BX = TX + 4, BY = TY + 4, NBOX = BX * BY;
     static constexpr int NC = TX * TY;             // owned cells
     static constexpr int NFX = (TX + 1) * TY;      // x faces
@@ -482,16 +497,28 @@ struct TileGeo {
     // columns (x only) and the halo rows (y only)
     static constexpr int NLIM = NC + 2 * TY + 2 * TX;
 };
-using TileP = TileGeo<31, 15>;
-constexpr int NTP = 256;
-static_assert(TileP::NFX <= 2 * NTP && TileP::NFY <= 2 * NTP && TileP::NC <= 2 * NTP,
-              "two faces per direction and two cells per thread");
+using TileP = TileGeo<31, 18, 320>;
 
 // shared memory of the packed stage: stencil box, x and y face fluxes,
 // limiters, reduction scratch
 template <class G>
 constexpr size_t smem_mixed_x2() {
-    return sizeof(float) * (NP * G::NBOX + NP * G::NFX + NP * G::NFY + G::NPX + G::NPY + 8);
+    return sizeof(float) * (NP * G::NBOX + NP * G::NFX + NP * G::NFY + G::NPX + G::NPY + G::NT / 32);
+}
+
+// CFL rate of the cell whose conserved state starts at U (see mxe_rate32.cuh)
+template <class PH>
+__device__ __noinline__ float cell_rate(const double* U, long long fstride, float sigma_lim,
+                                        float k_ws, float idx, float idy) {
+    double Uc[PH::NF], Q[PH::NF];
+    float W[PH::NF];
+#pragma unroll
+    for (int k = 0; k < PH::NF; ++k) Uc[k] = U[PH::ufield(k) * fstride];
+    PH::cons2prim_fast(Uc, Q);
+#pragma unroll
+    for (int k = 0; k < PH::NF; ++k) W[k] = (float)Q[k];
+    const float r = rn::rate<PH::NF>(W, sigma_lim, k_ws, idx, idy);
+    return r >= 0.0f ? r : __int_as_float(0x7f800000);             // NaN -> inf
 }
 
 template <class G>
@@ -505,9 +532,9 @@ __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const Param
     float* Fy = Fx + NF * G::NFX;                    // [NF][TY+1][TX]
     float* phx = Fy + NF * G::NFY;                   // [TY][TX+2]
     float* phy = phx + G::NPX;                       // [TY+2][TX]
-    float* red = phy + G::NPY;                       // [8]
+    float* red = phy + G::NPY;                       // [NT / 32]
     __shared__ double sdt[2];
-    __shared__ float scdt;
+    __shared__ float scdt, srate;
     __shared__ unsigned cnt;
 
     const int tid = threadIdx.x;
@@ -540,7 +567,7 @@ __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const Param
     // final stage: the owned cells' U^n and W^n are needed only after the
     // face fluxes; start moving them into L2 now
     if (a.final_stage) {
-        for (int c = tid; c < G::NC; c += NTP) {
+        for (int c = tid; c < G::NC; c += G::NT) {
             const int gi = i0 + c % G::TX, gj = j0 + c / G::TX;
             if (gi < g.nx && gj < g.ny) {
                 const long long o = (long long)gj * g.pitch + gi;
@@ -555,14 +582,14 @@ __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const Param
     const bool interior = i0 >= 2 && j0 >= 2 && i0 + G::TX + 2 <= g.nx && j0 + G::TY + 2 <= g.ny;
     if (interior) {      // the whole box inside the grid: asynchronous copies, no ghost cells
         const float* src = a.Win + (long long)(j0 - 2) * g.pitch + (i0 - 2);
-        for (int c = tid; c < G::NBOX; c += NTP) {
+        for (int c = tid; c < G::NBOX; c += G::NT) {
             const float* s0 = src + (long long)(c / G::BX) * g.pitch + c % G::BX;
 #pragma unroll
             for (int k = 0; k < NF; ++k) cp_async4(W + k * G::NBOX + c, s0 + k * g.fstride);
         }
         asm volatile("cp.async.commit_group;\n" ::);
     } else {
-        for (int c = tid; c < G::NBOX; c += NTP) {
+        for (int c = tid; c < G::NBOX; c += G::NT) {
             const int bx = c % G::BX, by = c / G::BX;
             float Q[NF];
             load_prim_f32<PH>(a, i0 + bx - 2, j0 + by - 2, Q);
@@ -572,7 +599,7 @@ __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const Param
     }
     asm volatile("cp.async.wait_group 0;\n" ::);
     __syncthreads();
-    for (int n = tid; n < G::NLIM; n += NTP) {
+    for (int n = tid; n < G::NLIM; n += G::NT) {
         if (n < G::NC) {                   // owned cell: both directions
             const int bx = 2 + n % G::TX, by = 2 + n / G::TX;
             float2 v = make_float2(0.0f, 0.0f);
@@ -598,7 +625,7 @@ __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const Param
     const double sl64 = a.sp.sigma_lim, kw64 = a.sp.k_ws;
     unsigned nflag = 0;
 #pragma unroll 1
-    for (int f = tid; f < G::NFX; f += NTP) {       // x faces: TY rows of TX + 1
+    for (int f = tid; f < G::NFX; f += G::NT) {       // x faces: TY rows of TX + 1
         const int fx = f % (G::TX + 1), fy = f / (G::TX + 1);
         float F[NF];
         face_flux_x2<0, G::NBOX>(W, (fy + 2) * G::BX + fx + 1, 1, phx[fy * (G::TX + 2) + fx],
@@ -607,7 +634,7 @@ __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const Param
         for (int k = 0; k < NF; ++k) Fx[k * G::NFX + f] = F[k];
     }
 #pragma unroll 1
-    for (int f = tid; f < G::NFY; f += NTP) {       // y faces: TY + 1 rows of TX
+    for (int f = tid; f < G::NFY; f += G::NT) {       // y faces: TY + 1 rows of TX
         const int fx = f % G::TX, fy = f / G::TX;
         float F[NF];
         face_flux_x2<1, G::NBOX>(W, (fy + 1) * G::BX + fx + 2, G::BX, phy[fy * G::TX + fx],
@@ -615,13 +642,22 @@ __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const Param
 #pragma unroll
         for (int k = 0; k < NF; ++k) Fy[k * G::NFY + f] = F[k];
     }
+    // cells with a smaller approximate rate are not evaluated again: those below
+    // what other blocks have found (that only grows), or 1 % below the last
+    // step's maximum
+    if (a.final_stage && tid == 0) {
+        const volatile unsigned long long* rt = a.clk->rate;
+        srate = fmaxf((float)__longlong_as_double((long long)rt[(a.slot + 1) % 3]) * (1.0f - 0x1p-15f),
+                      (float)__longlong_as_double((long long)rt[a.slot]) * 0.99f);
+    }
     __syncthreads();
 
     float r = 0.0f;
+    long long orate = 0;         // the cell of r
     const float cdt = scdt;
     const bool implicit = p.tau_model != 0 && p.src_implicit;
 #pragma unroll 1
-    for (int c = tid; c < G::NC; c += NTP) {
+    for (int c = tid; c < G::NC; c += G::NT) {
         const int cx = c % G::TX, cy = c / G::TX;
         const int gi = i0 + cx, gj = j0 + cy;
         if (gi >= g.nx || gj >= g.ny) continue;
@@ -698,9 +734,14 @@ __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const Param
             x2::rates_x2(Wn, p.sigma_lim, p.k_ws, ax, ay);
             float rc = ax * a.idxf + ay * a.idyf;
             if (!(rc >= 0.0f)) rc = __int_as_float(0x7f800000);     // NaN -> inf
-            r = fmaxf(r, rc);
+            if (rc >= r) {
+                r = rc;
+                orate = o;
+            }
         }
     }
+    if (a.final_stage && r >= srate && r > 0.0f)
+        r = cell_rate<PH>(a.Uout + orate, g.fstride, p.sigma_lim, p.k_ws, a.idxf, a.idyf);
     unsigned wf = __reduce_add_sync(0xffffffffu, nflag);
     if ((tid & 31) == 0 && wf) atomicAdd(&cnt, wf);
     if (a.final_stage) block_max_atomic_m(r, &a.clk->rate[(a.slot + 1) % 3], red);
@@ -711,13 +752,14 @@ __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const Param
     }
 }
 
-// planar state, packed face-state pairs, 15 x 32 tile, three blocks per SM
-extern "C" __global__ void __launch_bounds__(NTP, 3)
+// planar state, packed face-state pairs, two blocks per SM
+extern "C" __global__ void __launch_bounds__(TileP::NT, 2)
 mxe_stage14_2d_mixed_planar_x2(const Stage2DArgs a, const ParamsT<float> p,
                                const MixedPolicy mp) {
     stage_mixed_x2<TileP>(a, p, mp);
 }
 size_t stage14_2d_mixed_x2_smem() { return smem_mixed_x2<TileP>(); }
+int stage14_2d_mixed_x2_threads() { return TileP::NT; }
 int stage14_2d_mixed_x2_tile_x() { return TileP::TX; }
 int stage14_2d_mixed_x2_tile_y() { return TileP::TY; }
 
@@ -760,9 +802,7 @@ __device__ __forceinline__ void rate_mixed(const float* W, const Grid2D& g, cons
         float Q[PH::NF];
 #pragma unroll
         for (int k = 0; k < PH::NF; ++k) Q[k] = W[o + k * g.fstride];
-        float ax, ay;
-        PH::rates(Q, p.sigma_lim, p.k_ws, ax, ay);
-        r = ax * idxf + ay * idyf;
+        r = rn::rate<PH::NF>(Q, p.sigma_lim, p.k_ws, idxf, idyf);
         if (!(r >= 0.0f)) r = __int_as_float(0x7f800000);
     }
     block_max_atomic_m(r, &clk->rate[slot], red);

@@ -105,36 +105,18 @@ __device__ __forceinline__ void face_flux_x2(const float* W, int cl, int stride,
     using namespace x2;
     constexpr int NF = NP;
     v2 Q[NF];
-    const v2 hp = make_float2(0.25f * phl, -0.25f * phr);
+    auto reconstruct = [&]() {
+        const v2 hp = make_float2(0.25f * phl, -0.25f * phr);
 #pragma unroll
-    for (int k = 0; k < NF; ++k) {
-        const float* w = W + k * NBOX + cl;
-        const float wm = w[-stride], w0 = w[0], w1 = w[stride], w2 = w[2 * stride];
-        Q[k] = fma(hp, sub(make_float2(w1, w2), make_float2(wm, w0)), make_float2(w0, w1));
-    }
-    v2 U[NF], Fv[NF], lmin, lmax, sig, det;
-    face_eval_x2<K>(Q, p.sigma_lim, p.k_ws, U, Fv, lmin, lmax, sig, det);
-    if (p.flux == 1) {
-        float s = fmaxf(fmaxf(fabsf(lmin.x), fabsf(lmax.x)), fmaxf(fabsf(lmin.y), fabsf(lmax.y)));
-#pragma unroll
-        for (int k = 0; k < NF; ++k)
-            F[k] = 0.5f * (Fv[k].x + Fv[k].y) - 0.5f * s * (U[k].y - U[k].x);
-    } else {
-        float SL = fminf(lmin.x, lmin.y), SR = fmaxf(lmax.x, lmax.y);
-        if (SL >= 0.0f) {
-#pragma unroll
-            for (int k = 0; k < NF; ++k) F[k] = Fv[k].x;
-        } else if (SR <= 0.0f) {
-#pragma unroll
-            for (int k = 0; k < NF; ++k) F[k] = Fv[k].y;
-        } else {
-            float inv = 1.0f / (SR - SL);
-            float cl_ = SR * inv, cr_ = -SL * inv, cu = SL * SR * inv;
-#pragma unroll
-            for (int k = 0; k < NF; ++k)
-                F[k] = cl_ * Fv[k].x + cr_ * Fv[k].y + cu * (U[k].y - U[k].x);
+        for (int k = 0; k < NF; ++k) {
+            const float* w = W + k * NBOX + cl;
+            const float wm = w[-stride], w0 = w[0], w1 = w[stride], w2 = w[2 * stride];
+            Q[k] = fma(hp, sub(make_float2(w1, w2), make_float2(wm, w0)), make_float2(w0, w1));
         }
-    }
+    };
+    reconstruct();
+    v2 sig, det;
+    face_eval_x2<K>(Q, p.sigma_lim, p.k_ws, p.flux, F, sig, det);
     if (mp.sig_lo > 0.0f || mp.sig_hi < 1.0f || mp.det_min > 0.0f) {
         const bool fx = (sig.x >= p.sigma_lim && sig.x < mp.sig_lo) || sig.x > mp.sig_hi ||
                         det.x < mp.det_min || !(sig.x == sig.x);
@@ -142,6 +124,8 @@ __device__ __forceinline__ void face_flux_x2(const float* W, int cl, int stride,
                         det.y < mp.det_min || !(sig.y == sig.y);
         nflag += (fx ? 1u : 0u) + (fy ? 1u : 0u);
         if (__any_sync(__activemask(), fx || fy) && (fx || fy)) {
+            asm volatile("" ::: "memory");   // form the states again rather than keep them live
+            reconstruct();
             FacePairIn<NF> in;
 #pragma unroll
             for (int k = 0; k < NF; ++k) {

@@ -53,38 +53,36 @@ struct DimX2 {
 
 // sigma = [A + sqrt(A^2 + X)] / (4 T), rationalised for A < 0.
 __device__ __forceinline__ v2 sigma_root_x2(v2 A, v2 X, v2 T2) {
-    v2 rt = sqrt_(fma(A, A, X));
-    v2 fT = mul(T2, S(4.0f));
-    v2 s1 = add(A, rt);                // A >= 0
-    v2 dn = mul(fT, sub(rt, A));       // A < 0
-    return div_(make_float2(A.x >= 0.0f ? s1.x : X.x, A.y >= 0.0f ? s1.y : X.y),
+    const v2 s = add(sqrt_(fma(A, A, X)), abs_(A));
+    const v2 fT = mul(T2, S(4.0f)), dn = mul(fT, s);
+    return div_(make_float2(A.x >= 0.0f ? s.x : X.x, A.y >= 0.0f ? s.y : X.y),
                 make_float2(A.x >= 0.0f ? fT.x : dn.x, A.y >= 0.0f ? fT.y : dn.y));
 }
 
 __device__ __forceinline__ void dimless_x2(const v2* Q, DimX2& g) {
-    v2 rho = Q[0];
+    const v2 rho = Q[0];
     g.tr = add(add(Q[3], Q[5]), Q[6]);
     g.p = mul(g.tr, S(1.0f / 3.0f));
-    v2 ip = rcp(g.p), ir = rcp(rho);
-    g.th = mul(g.p, ir);
-    v2 rsq = rsqrt_(g.th);
+    const v2 ip = rcp(g.p);
+    g.th = mul(g.p, rcp(rho));
+    const v2 rsq = rsqrt_(g.th);
     g.sq = mul(g.th, rsq);
-    v2 isc3 = mul(ip, rsq);                           // 1 / (rho th sqrt th)
+    const v2 isc3 = mul(ip, rsq);                     // 1 / (rho th sqrt th)
     g.a = mul(Q[3], ip); g.b = mul(Q[4], ip); g.d = mul(Q[5], ip); g.f = mul(Q[6], ip);
     g.qx = mul(Q[7], isc3); g.qy = mul(Q[8], isc3);
-    v2 nRs = mul(mul(Q[9], neg(rho)), mul(ip, ip));   // -R / (rho th^2)
+    const v2 nip = neg(ip);
+    const v2 nRs = mul(mul(Q[9], rho), mul(ip, nip)); // -R / (rho th^2)
     g.trPs = add(add(g.a, g.d), g.f);
     g.bb = mul(g.b, g.b);
     g.T2 = fma(g.a, g.a, fma(g.d, g.d, fma(g.f, g.f, add(g.bb, g.bb))));
-    v2 det2 = fma(g.a, g.d, neg(g.bb));
-    v2 i2 = rcp(det2);
-    v2 ia = mul(g.d, i2), ib = mul(neg(g.b), i2), id = mul(g.a, i2);
+    const v2 det2 = sub(mul(g.a, g.d), g.bb);
+    const v2 i2 = rcp(det2), nb = neg(g.b);
     g.det = mul(det2, g.f);
-    g.yx = fma(ia, g.qx, mul(ib, g.qy));
-    g.yy = fma(ib, g.qx, mul(id, g.qy));
-    v2 qPq = fma(g.qx, g.yx, mul(g.qy, g.yy));
-    v2 A = fma(g.trPs, g.trPs, fma(g.T2, S(2.0f), nRs));
-    v2 X = mul(mul(g.T2, S(8.0f)), qPq);
+    g.yx = mul(fma(g.d, g.qx, mul(nb, g.qy)), i2);
+    g.yy = mul(fma(g.a, g.qy, mul(nb, g.qx)), i2);
+    const v2 qPq = fma(g.qx, g.yx, mul(g.qy, g.yy));
+    const v2 A = fma(g.trPs, g.trPs, fma(g.T2, S(2.0f), nRs));
+    const v2 X = mul(mul(g.T2, S(8.0f)), qPq);
     g.sig = sigma_root_x2(A, X, g.T2);
 }
 
@@ -92,151 +90,40 @@ __device__ __forceinline__ v2 clamp_sigma_x2(v2 s, float slim) {
     return make_float2(fminf(fmaxf(s.x, slim), 1.0f), fminf(fmaxf(s.y, slim), 1.0f));
 }
 
-// Closure slice along K (dimensional): QK = (Q_KKK, Q_KKO, Q_KOO, Q_Kzz),
-// RK = (R_KKjj, R_OKjj), SK = S_Kiijj (see closure_p).
-template <int K>
-__device__ __forceinline__ void closure_x2(const DimX2& g, v2 sb, v2 isb, v2 ssb, v2* QK, v2* RK,
-                                           v2& SK) {
-    const v2 a = g.a, b = g.b, d = g.d, f = g.f;
-    v2 P2xx = fma(a, a, g.bb), P2xy = mul(b, add(a, d)), P2yy = fma(d, d, g.bb), P2zz = mul(f, f);
-    v2 P3xx = fma(P2xx, a, mul(P2xy, b)), P3xy = fma(P2xx, b, mul(P2xy, d));
-    v2 P3yy = fma(P2xy, b, mul(P2yy, d));
-    v2 trP3 = fma(P2zz, f, add(P3xx, P3yy));
-    v2 T2x2 = add(g.T2, g.T2);
-    v2 Bxx = fma(a, T2x2, mul(P3xx, S(4.0f)));
-    v2 Bxy = fma(b, T2x2, mul(P3xy, S(4.0f)));
-    v2 Byy = fma(d, T2x2, mul(P3yy, S(4.0f)));
-    v2 nBxy = neg(Bxy);
-    v2 iB = rcp(fma(Bxy, nBxy, mul(Bxx, Byy)));
-    v2 vx = mul(fma(Byy, g.qx, mul(nBxy, g.qy)), iB);
-    v2 vy = mul(fma(Bxx, g.qy, mul(nBxy, g.qx)), iB);
-    v2 wx = fma(a, vx, mul(b, vy)), wy = fma(b, vx, mul(d, vy));
-    const v2 wK = K == 0 ? wx : wy, wO = K == 0 ? wy : wx;
-    const v2 vK = K == 0 ? vx : vy, vO = K == 0 ? vy : vx;
-    const v2 yK = K == 0 ? g.yx : g.yy, yO = K == 0 ? g.yy : g.yx;
-    const v2 P2KK = K == 0 ? P2xx : P2yy, P2OO = K == 0 ? P2yy : P2xx;
-    const v2 P3KK = K == 0 ? P3xx : P3yy, P3KO = P3xy;
-    const v2 PKK = K == 0 ? a : d;
-    const v2 qK = K == 0 ? g.qx : g.qy;
-    v2 w2K = add(wK, wK), w2O = add(wO, wO);
-    v2 QKKK = mul(mul(wK, P2KK), S(6.0f));
-    v2 QKKO = mul(fma(w2K, P2xy, mul(wO, P2KK)), S(2.0f));
-    v2 QKOO = mul(fma(wK, P2OO, mul(w2O, P2xy)), S(2.0f));
-    v2 QKzz = mul(w2K, P2zz);
-    v2 omsb2 = fma(sb, S(-2.0f), S(2.0f));           // 2 (1 - sigma)
-    v2 t1 = fma(QKKK, yK, mul(QKKO, yO));
-    v2 t2 = fma(QKKO, yK, mul(QKOO, yO));
-    v2 RKK = fma(t1, isb, fma(omsb2, P2KK, mul(PKK, g.trPs)));
-    v2 ROK = fma(t2, isb, fma(omsb2, P2xy, mul(b, g.trPs)));
-    v2 yQy = fma(yK, t1, mul(yO, t2));
-    v2 t = g.trPs, tt = mul(t, t);
-    v2 c1 = fma(add(t, t), sub(tt, g.T2), mul(trP3, S(12.0f)));
-    v2 c2 = fma(g.T2, S(14.0f), mul(tt, S(-6.0f)));
-    v2 c3 = mul(t, S(20.0f));
-    v2 P4KK = fma(P2KK, P2KK, mul(P2xy, P2xy));
-    v2 P4KO = mul(P2xy, add(P2xx, P2yy));
-    v2 mKK = fma(c1, PKK, fma(c2, P2KK, fma(c3, P3KK, mul(P4KK, S(20.0f)))));
-    v2 mKO = fma(c1, b, fma(c2, P2xy, fma(c3, P3KO, mul(P4KO, S(20.0f)))));
-    v2 Wq = fma(mKK, vK, mul(mKO, vO));
-    v2 Ss = fma(yQy, mul(isb, isb), fma(add(ssb, ssb), mul(t, qK), mul(sub(S(1.0f), ssb), Wq)));
-    v2 sc3 = mul(g.p, g.sq), sc4 = mul(g.p, g.th);
-    v2 sc5 = mul(sc4, g.sq);
-    QK[0] = mul(QKKK, sc3); QK[1] = mul(QKKO, sc3); QK[2] = mul(QKOO, sc3); QK[3] = mul(QKzz, sc3);
-    RK[0] = mul(RKK, sc4); RK[1] = mul(ROK, sc4);
-    SK = mul(Ss, sc5);
-}
-
-// Conserved face state of the compact primitives; also returns |u|^2, P u.
-__device__ __forceinline__ void prim2cons_x2(const v2* Q, v2 trP, v2* U, v2& u2, v2& Pux,
-                                             v2& Puy) {
-    v2 rho = Q[0], ux = Q[1], uy = Q[2];
-    v2 Pxx = Q[3], Pxy = Q[4], Pyy = Q[5];
-    u2 = fma(ux, ux, mul(uy, uy));
-    Pux = fma(Pxx, ux, mul(Pxy, uy));
-    Puy = fma(Pxy, ux, mul(Pyy, uy));
-    v2 uPu = fma(ux, Pux, mul(uy, Puy));
-    v2 uq = fma(ux, Q[7], mul(uy, Q[8]));
-    v2 e = fma(rho, u2, trP);
-    U[0] = rho;
-    U[1] = mul(rho, ux); U[2] = mul(rho, uy);
-    U[3] = fma(U[1], ux, Pxx); U[4] = fma(U[1], uy, Pxy); U[5] = fma(U[2], uy, Pyy);
-    U[6] = Q[6];
-    U[7] = fma(ux, e, fma(Pux, S(2.0f), Q[7]));
-    U[8] = fma(uy, e, fma(Puy, S(2.0f), Q[8]));
-    U[9] = fma(mul(rho, u2), u2, fma(add(u2, u2), trP, fma(add(uPu, uq), S(4.0f), Q[9])));
-}
-
-// K-flux of the compact system, u_K U + central part (see flux_p).
-template <int K>
-__device__ __forceinline__ void flux_x2(const v2* Q, const v2* U, v2 u2, v2 Pux, v2 Puy,
-                                        const v2* QK, const v2* RK, v2 SK, v2* F) {
-    const v2 ux = Q[1], uy = Q[2];
-    const v2 uK = K == 0 ? ux : uy, uO = K == 0 ? uy : ux;
-    const v2 Pxy = Q[4];
-    const v2 PxK = K == 0 ? Q[3] : Pxy, PyK = K == 0 ? Pxy : Q[5];
-    const v2 qK = Q[7 + K];
-    const v2 PuK = K == 0 ? Pux : Puy;
-    v2 QuK = fma(QK[0], uK, mul(QK[1], uO));
-    v2 QuO = fma(QK[1], uK, mul(QK[2], uO));
-    const v2 QxxK = K == 0 ? QK[0] : QK[2];
-    const v2 QxyK = QK[1];
-    const v2 QyyK = K == 0 ? QK[2] : QK[0];
-    F[0] = mul(uK, U[0]);
-    F[1] = fma(uK, U[1], PxK);
-    F[2] = fma(uK, U[2], PyK);
-    F[3] = fma(uK, U[3], fma(add(ux, ux), PxK, QxxK));
-    F[4] = fma(uK, U[4], fma(ux, PyK, fma(uy, PxK, QxyK)));
-    F[5] = fma(uK, U[5], fma(add(uy, uy), PyK, QyyK));
-    F[6] = fma(uK, U[6], QK[3]);
-    v2 gK = fma(PuK, S(2.0f), qK);
-    const v2 QuX = K == 0 ? QuK : QuO, QuY = K == 0 ? QuO : QuK;
-    const v2 RxK = K == 0 ? RK[0] : RK[1], RyK = K == 0 ? RK[1] : RK[0];
-    F[7] = fma(uK, U[7], fma(ux, gK, fma(u2, PxK, fma(QuX, S(2.0f), RxK))));
-    F[8] = fma(uK, U[8], fma(uy, gK, fma(u2, PyK, fma(QuY, S(2.0f), RyK))));
-    v2 uQu = fma(uK, QuK, mul(uO, QuO));
-    v2 uR = fma(uK, RK[0], mul(uO, RK[1]));
-    F[9] = fma(uK, U[9], fma(u2, fma(PuK, S(4.0f), add(qK, qK)), fma(add(uQu, uR), S(4.0f), SK)));
-}
-
-// zeta + sqrt(zeta^2 + D0), discriminant clamped at 0, rationalised for zeta < 0.
-__device__ __forceinline__ float hyp1(float z, float D0, float D, float rt) {
-    return z >= 0.0f ? z + rt : (D > 0.0f ? __fdividef(D0, rt - z) : z);
+// zeta + sqrt(zeta^2 + D0), discriminant D clamped at 0, rationalised to
+// D0 / (sqrt(D) - zeta) for zeta < 0, where a clamped discriminant makes the
+// quotient smaller than zeta, the value it stands for.
+__device__ __forceinline__ float hyp1(float z, float D0, float s) {
+    const float q = fmaxf(__fdividef(D0, s), z);
+    return z >= 0.0f ? s : q;
 }
 __device__ __forceinline__ v2 hyp_x2(v2 z, v2 D0) {
-    v2 D = fma(z, z, D0);
-    v2 rt = sqrt_(make_float2(fmaxf(D.x, 0.0f), fmaxf(D.y, 0.0f)));
-    return make_float2(hyp1(z.x, D0.x, D.x, rt.x), hyp1(z.y, D0.y, D.y, rt.y));
+    const v2 D = fma(z, z, D0);
+    const v2 s = add(sqrt_(make_float2(fmaxf(D.x, 0.0f), fmaxf(D.y, 0.0f))), abs_(z));
+    return make_float2(hyp1(z.x, D0.x, s.x), hyp1(z.y, D0.y, s.y));
 }
 
 // Eq. (14mom-approx-ws-equations) for two (P*_kk, q*_k, |q*_perp|) triples
-// at once: the dimensionless lambda*_max (lp) and lambda*_min (lm).
+// at once: the magnitudes of the dimensionless lambda*_max (lp) and
+// -lambda*_min (lm).
 __device__ __forceinline__ void lam_core_x2(v2 Pkk, v2 qd, v2 qperp, v2 sb, v2 isb, v2 ssb,
                                             v2& lp, v2& lm) {
-    v2 l2 = lg2(Pkk);
-    v2 Pkk2 = mul(Pkk, Pkk);
-    v2 a = mul(ex2(fma(Pkk2, S(-LOG2E), mul(l2, S(1.1f)))), S(1.4f));
-    v2 b = mul(mul(Pkk, S(0.9f)), ex2(mul(ex2(mul(l2, S(1.4f))), S(-0.5f * LOG2E))));
-    v2 C = sqrt_(mul(fma(sb, S(-3.0f), S(3.0f)), Pkk));
-    v2 E = mul(C, S(0.8f));
+    const v2 l2 = lg2(Pkk);
+    const v2 Pkk2 = mul(Pkk, Pkk);
+    const v2 a = ex2(fma(Pkk2, S(-LOG2E), mul(l2, S(1.1f))));
+    const v2 b = ex2(mul(ex2(mul(l2, S(1.4f))), S(-0.5f * LOG2E)));
+    const v2 pre = fma(mul(mul(Pkk, S(0.45f)), b), isb, mul(a, S(0.7f)));
+    const v2 E = mul(sqrt_(mul(fma(sb, S(-3.0f), S(3.0f)), Pkk)), S(0.8f));
     // B = 5 - 4 r + sqrt(2 (5 - 3 r)(1 - r)), Y = (sqrt B - E)^2, r = sqrt(sigma)
-    v2 B = add(fma(ssb, S(-4.0f), S(5.0f)),
-               sqrt_(mul(mul(fma(ssb, S(-3.0f), S(5.0f)), sub(S(1.0f), ssb)), S(2.0f))));
-    v2 dd = sub(sqrt_(B), E);
-    v2 Y = mul(dd, dd);
-    v2 al = mul(qperp, fma(Pkk2, S(0.6f), fma(Pkk, S(-0.38f), S(0.35f))));
-    v2 base = fma(mul(sb, sb), mul(Y, S(4.0f)), mul(mul(qperp, qperp), S(0.1f)));
-    v2 pre = mul(fma(a, sb, b), mul(isb, S(0.5f)));
-    v2 zp = add(qd, al), zm = sub(al, qd);
-    v2 m08 = mul(mul(sb, C), S(-0.8f));
-    lp = fma(pre, hyp_x2(zp, fma(zp, m08, base)), E);
-    lm = neg(fma(pre, hyp_x2(zm, fma(zm, m08, base)), E));
-}
-
-// The same along K for two face states, q_perp = |q*_O|.
-template <int K>
-__device__ __forceinline__ void lam_x2(const DimX2& g, v2 sb, v2 isb, v2 ssb, v2& lp, v2& lm) {
-    lam_core_x2(K == 0 ? g.a : g.d, K == 0 ? g.qx : g.qy, abs_(K == 0 ? g.qy : g.qx), sb, isb,
-                ssb, lp, lm);
+    const v2 B = add(fma(ssb, S(-4.0f), S(5.0f)),
+                     sqrt_(mul(fma(ssb, S(-6.0f), S(10.0f)), sub(S(1.0f), ssb))));
+    const v2 sd = mul(sub(sqrt_(B), E), add(sb, sb));
+    const v2 al = mul(qperp, fma(Pkk, fma(Pkk, S(0.6f), S(-0.38f)), S(0.35f)));
+    const v2 base = fma(sd, sd, mul(mul(qperp, S(0.1f)), qperp));
+    const v2 zp = add(qd, al), zm = sub(al, qd);
+    const v2 msE = mul(mul(sb, S(-1.0f)), E);
+    lp = fma(pre, hyp_x2(zp, fma(zp, msE, base)), E);
+    lm = fma(pre, hyp_x2(zm, fma(zm, msE, base)), E);
 }
 
 // CFL rates max(|lambda_min|, |lambda_max|) of one cell state in x and y
@@ -251,34 +138,148 @@ __device__ __forceinline__ void rates_x2(const float* Q, float sigma_lim, float 
                 make_float2(fabsf(g.qy), fabsf(g.qx)), S(sb), S(1.0f / sb), S(sqrtf(sb)), lp, lm);
     const v2 u = make_float2(Q[1], Q[2]);
     const v2 ks = S(k_ws * g.sq);
-    const v2 hi = fma(lp, ks, u), lo = fma(lm, ks, u);
+    const v2 hi = fma(lp, ks, u), lo = fma(lm, neg(ks), u);
     ax = fmaxf(fabsf(lo.x), fabsf(hi.x));
     ay = fmaxf(fabsf(lo.y), fabsf(hi.y));
 }
 
-// Both face states of a face: conserved U, K-flux F, wave speeds, and the
-// raw sigma and det P* (the conditioning the mixed policy checks).
+// Weights of the numerical flux of a face with wave speeds (lmin, lmax) of
+// its two states: F = l F_L + r F_R + u (U_R - U_L) (HLL with Davis speeds,
+// or Rusanov).
+struct FluxWeights {
+    float l, r, u;
+};
+__device__ __forceinline__ FluxWeights flux_weights(v2 lmin, v2 lmax, int flux) {
+    FluxWeights w;
+    if (flux == 1) {
+        const float s = fmaxf(fmaxf(fabsf(lmin.x), fabsf(lmax.x)),
+                              fmaxf(fabsf(lmin.y), fabsf(lmax.y)));
+        w.l = w.r = 0.5f;
+        w.u = -0.5f * s;
+        return w;
+    }
+    const float SL = fminf(lmin.x, lmin.y), SR = fmaxf(lmax.x, lmax.y);
+    const float inv = 1.0f / (SR - SL);
+    w.l = SR * inv;
+    w.r = -SL * inv;
+    w.u = SL * w.l;
+    if (SL >= 0.0f) {
+        w.l = 1.0f;
+        w.r = w.u = 0.0f;
+    } else if (SR <= 0.0f) {
+        w.r = 1.0f;
+        w.l = w.u = 0.0f;
+    }
+    return w;
+}
+__device__ __forceinline__ float weigh(const FluxWeights& w, v2 F, v2 U) {
+    return fmaf(w.u, U.y - U.x, fmaf(w.l, F.x, w.r * F.y));
+}
+
+// Numerical flux Fn along K of a face with the states Q (left in lane x, right
+// in lane y), and the raw sigma and det P* of both (the conditioning that the
+// mixed policy checks).  The wave speeds need the dimensionless state alone,
+// so they come first: each field's U and K-flux then goes into Fn as it is
+// formed, and no U or F of the pair stays in registers.
+// closure slice: QK = (Q_KKK, Q_KKO, Q_KOO, Q_Kzz), RK = (R_KKjj, R_OKjj),
+// SK = S_Kiijj (see closure_p); conserved state and flux: prim2cons_p, flux_p.
 template <int K>
-__device__ __forceinline__ void face_eval_x2(const v2* Q, float sigma_lim, float k_ws, v2* U,
-                                             v2* F, v2& lmin, v2& lmax, v2& sig, v2& det) {
+__device__ __forceinline__ void face_eval_x2(const v2* Q, float sigma_lim, float k_ws, int flux,
+                                             float* Fn, v2& sig, v2& det) {
     DimX2 g;
     dimless_x2(Q, g);
-    v2 sb = clamp_sigma_x2(g.sig, sigma_lim);
-    v2 rsb = rsqrt_(sb);
-    v2 isb = mul(rsb, rsb), ssb = mul(sb, rsb);       // 1/sigma, sqrt(sigma)
-    v2 QK[4], RK[2], SK;
-    closure_x2<K>(g, sb, isb, ssb, QK, RK, SK);
-    v2 u2, Pux, Puy;
-    prim2cons_x2(Q, g.tr, U, u2, Pux, Puy);
-    flux_x2<K>(Q, U, u2, Pux, Puy, QK, RK, SK, F);
-    v2 lp, lm;
-    lam_x2<K>(g, sb, isb, ssb, lp, lm);
-    const v2 uK = Q[1 + K];
-    v2 ks = mul(g.sq, S(k_ws));
-    lmax = fma(lp, ks, uK);
-    lmin = fma(lm, ks, uK);
     sig = g.sig;
     det = g.det;
+    const v2 sb = clamp_sigma_x2(g.sig, sigma_lim);
+    const v2 rsb = rsqrt_(sb);
+    const v2 isb = mul(rsb, rsb), ssb = mul(sb, rsb);  // 1/sigma, sqrt(sigma)
+    const v2 ux = Q[1], uy = Q[2], uK = K == 0 ? ux : uy, uO = K == 0 ? uy : ux;
+    FluxWeights w;
+    {
+        v2 lp, lm;
+        lam_core_x2(K == 0 ? g.a : g.d, K == 0 ? g.qx : g.qy, abs_(K == 0 ? g.qy : g.qx), sb,
+                    isb, ssb, lp, lm);
+        const v2 ks = mul(g.sq, S(k_ws));
+        w = flux_weights(fma(lm, neg(ks), uK), fma(lp, ks, uK), flux);
+    }
+    // second moments and the pressure work need Q_K.. of the closure, with
+    // v = B^-1 q* (scaled by 4: B/4 = (T2/2) P* + P*^3), w = P* v
+    const v2 a = g.a, b = g.b, d = g.d, f = g.f, t = g.trPs;
+    const v2 P2xx = fma(a, a, g.bb), P2xy = mul(b, add(a, d)), P2yy = fma(d, d, g.bb);
+    const v2 P2zz = mul(f, f);
+    const v2 P3xx = fma(P2xx, a, mul(P2xy, b)), P3xy = fma(P2xx, b, mul(P2xy, d));
+    const v2 P3yy = fma(P2xy, b, mul(P2yy, d));
+    const v2 h2 = mul(g.T2, S(0.5f));
+    const v2 Bxx = fma(h2, a, P3xx), Bxy = fma(h2, b, P3xy), Byy = fma(h2, d, P3yy);
+    const v2 nBxy = neg(Bxy);
+    const v2 iB = rcp(fma(Bxy, nBxy, mul(Bxx, Byy)));
+    const v2 vx = mul(fma(Byy, g.qx, mul(nBxy, g.qy)), iB);
+    const v2 vy = mul(fma(Bxx, g.qy, mul(nBxy, g.qx)), iB);
+    const v2 P2KK = K == 0 ? P2xx : P2yy, P2OO = K == 0 ? P2yy : P2xx;
+    const v2 P3KK = K == 0 ? P3xx : P3yy;
+    const v2 PKK = K == 0 ? a : d;
+    const v2 yK = K == 0 ? g.yx : g.yy, yO = K == 0 ? g.yy : g.yx;
+    v2 QK[4], RKK, ROK, SK;
+    {
+        const v2 wx = fma(a, vx, mul(b, vy)), wy = fma(b, vx, mul(d, vy));
+        const v2 wK = mul(K == 0 ? wx : wy, S(0.5f)), wO = mul(K == 0 ? wy : wx, S(0.5f));
+        const v2 P2xyd = add(P2xy, P2xy);
+        QK[0] = mul(mul(wK, P2KK), S(3.0f));
+        QK[1] = fma(wK, P2xyd, mul(wO, P2KK));
+        QK[2] = fma(wK, P2OO, mul(wO, P2xyd));
+        QK[3] = mul(wK, P2zz);
+        const v2 t1 = fma(QK[0], yK, mul(QK[1], yO)), t2 = fma(QK[1], yK, mul(QK[2], yO));
+        const v2 om2 = fma(sb, S(-2.0f), S(2.0f));     // 2 (1 - sigma)
+        RKK = fma(t1, isb, fma(om2, P2KK, mul(PKK, t)));
+        ROK = fma(t2, isb, fma(om2, P2xy, mul(b, t)));
+        const v2 yQy = fma(yK, t1, mul(yO, t2));
+        // row K of the W bracket over 4, against v
+        const v2 tt = mul(t, t), trP3 = fma(P2zz, f, add(P3xx, P3yy));
+        const v2 c1 = fma(trP3, S(3.0f), mul(mul(t, S(0.5f)), sub(tt, g.T2)));
+        const v2 c2 = fma(g.T2, S(3.5f), mul(tt, S(-1.5f)));
+        const v2 c3 = mul(t, S(5.0f));
+        const v2 P4KK = fma(P2KK, P2KK, mul(P2xy, P2xy)), P4KO = mul(P2xy, add(P2xx, P2yy));
+        const v2 mKK = fma(c1, PKK, fma(c2, P2KK, fma(c3, P3KK, mul(P4KK, S(5.0f)))));
+        const v2 mKO = fma(c1, b, fma(c2, P2xy, fma(c3, P3xy, mul(P4KO, S(5.0f)))));
+        const v2 Wq = fma(mKK, K == 0 ? vx : vy, mul(mKO, K == 0 ? vy : vx));
+        const v2 Ss = fma(yQy, mul(isb, isb),
+                          fma(add(ssb, ssb), mul(t, K == 0 ? g.qx : g.qy),
+                              mul(sub(S(1.0f), ssb), Wq)));
+        const v2 sc3 = mul(g.p, g.sq), sc4 = mul(g.p, g.th);
+#pragma unroll
+        for (int n = 0; n < 4; ++n) QK[n] = mul(QK[n], sc3);
+        RKK = mul(RKK, sc4);
+        ROK = mul(ROK, sc4);
+        SK = mul(Ss, mul(sc4, g.sq));
+    }
+    // conserved state and flux u_K U + central part, field by field
+    const v2 rho = Q[0], Pxy = Q[4], PxK = K == 0 ? Q[3] : Pxy, PyK = K == 0 ? Pxy : Q[5];
+    const v2 mx = mul(rho, ux), my = mul(rho, uy);
+    Fn[0] = weigh(w, K == 0 ? mx : my, rho);
+    Fn[1] = weigh(w, fma(uK, mx, PxK), mx);
+    Fn[2] = weigh(w, fma(uK, my, PyK), my);
+    {
+        const v2 U3 = fma(mx, ux, Q[3]), U4 = fma(mx, uy, Pxy), U5 = fma(my, uy, Q[5]);
+        Fn[3] = weigh(w, fma(uK, U3, fma(add(ux, ux), PxK, K == 0 ? QK[0] : QK[2])), U3);
+        Fn[4] = weigh(w, fma(uK, U4, fma(ux, PyK, fma(uy, PxK, QK[1]))), U4);
+        Fn[5] = weigh(w, fma(uK, U5, fma(add(uy, uy), PyK, K == 0 ? QK[2] : QK[0])), U5);
+        Fn[6] = weigh(w, fma(uK, Q[6], QK[3]), Q[6]);
+    }
+    const v2 u2 = fma(ux, ux, mul(uy, uy)), ru2 = mul(rho, u2), e = add(ru2, g.tr);
+    const v2 Pux = fma(Q[3], ux, mul(Pxy, uy)), Puy = fma(Pxy, ux, mul(Q[5], uy));
+    const v2 QuK = fma(QK[0], uK, mul(QK[1], uO)), QuO = fma(QK[1], uK, mul(QK[2], uO));
+    const v2 gK = fma(K == 0 ? Pux : Puy, S(2.0f), Q[7 + K]);
+    {
+        const v2 U7 = fma(ux, e, fma(Pux, S(2.0f), Q[7])), U8 = fma(uy, e, fma(Puy, S(2.0f), Q[8]));
+        Fn[7] = weigh(w, fma(uK, U7, fma(ux, gK, fma(u2, PxK, fma(K == 0 ? QuK : QuO, S(2.0f),
+                                                                 K == 0 ? RKK : ROK)))), U7);
+        Fn[8] = weigh(w, fma(uK, U8, fma(uy, gK, fma(u2, PyK, fma(K == 0 ? QuO : QuK, S(2.0f),
+                                                                 K == 0 ? ROK : RKK)))), U8);
+    }
+    const v2 uPq = fma(ux, add(Pux, Q[7]), mul(uy, add(Puy, Q[8])));
+    const v2 U9 = fma(u2, fma(g.tr, S(2.0f), ru2), fma(uPq, S(4.0f), Q[9]));
+    const v2 uQR = fma(uK, add(QuK, RKK), mul(uO, add(QuO, ROK)));
+    Fn[9] = weigh(w, fma(uK, U9, fma(add(u2, u2), gK, fma(uQR, S(4.0f), SK))), U9);
 }
 
 }  // namespace x2

@@ -39,9 +39,6 @@ extern "C" __global__ void mxe_stage14_2d_mixed_b3(const Stage2DArgs a, const Pa
 extern "C" __global__ void mxe_stage14_2d_mixed_planar_b3(const Stage2DArgs a,
                                                           const ParamsT<float> p,
                                                           const MixedPolicy mp);
-extern "C" __global__ void mxe_stage14_2d_mixed_planar_x2(const Stage2DArgs a,
-                                                          const ParamsT<float> p,
-                                                          const MixedPolicy mp);
 extern "C" __global__ void mxe_resync14_2d(const double* U, float* W, Grid2D g);
 extern "C" __global__ void mxe_resync14_2d_planar(const double* U, float* W, Grid2D g);
 extern "C" __global__ void mxe_rate14_2d_mixed(const float* W, Grid2D g, ParamsT<float> p,
@@ -50,10 +47,7 @@ extern "C" __global__ void mxe_rate14_2d_mixed_planar(const float* W, Grid2D g,
                                                       ParamsT<float> p, float idxf, float idyf,
                                                       DevClock* clk, int slot);
 size_t stage14_2d_mixed_smem(bool planar, int blocks_per_sm);
-size_t stage14_2d_mixed_x2_smem();
-int stage14_2d_mixed_x2_threads();
-int stage14_2d_mixed_x2_tile_x();
-int stage14_2d_mixed_x2_tile_y();
+MixedTile mixed_tile_kernel(int n);
 const void* tubes_mixed_kernel(bool planar, int nt);
 cudaError_t adj_stage(const double* U, const double* V, double coef, const double* b1,
                       const double* b2, double* out, double* P, double* Cx, double* Cy,
@@ -481,10 +475,10 @@ extern "C" mxe_status mxe_create(const mxe_config* cfg, mxe_ctx** out) {
             e = cudaFuncSetAttribute(mxe_stage14_2d_mixed_planar_b3,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)stage14_2d_mixed_smem(true, 3));
-        if (e == cudaSuccess && c->mixed)
-            e = cudaFuncSetAttribute(mxe_stage14_2d_mixed_planar_x2,
+        for (int n = 0; n < 3 && e == cudaSuccess && c->mixed; ++n)
+            e = cudaFuncSetAttribute(mixed_tile_kernel(n).kern,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)stage14_2d_mixed_x2_smem());
+                                     (int)mixed_tile_kernel(n).smem);
         if (e == cudaSuccess && c->mixed)
             e = cudaFuncSetAttribute(mxe_stage14_2d_mixed_b3,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -895,6 +889,25 @@ static F64Tile f64_tile(const mxe_ctx* c, bool pl) {
     return best;
 }
 
+// Tile of the packed mixed stage.  Time of an RK2 step on GB300 (152 SMs), us:
+//            48 x 48  130 x 130  200 x 200  300 x 300  400 x 400  512 x 512  1024 x 1024
+//   31 x 18     35        35         35         43         44         76         224
+//   31 x  7     22        22         26         36         51         80         273
+//   15 x  7     18        21         29         41         67        103         386
+// (one tile before: 33 on 48 x 48, 262 on 1024 x 1024).  Small grids pay for the
+// passes of one block, then for each block; TileP's come two to an SM, in waves.
+static MixedTile mixed_tile(const mxe_ctx* c) {
+    auto blocks = [&](int n) {
+        const MixedTile f = mixed_tile_kernel(n);
+        return (double)((c->g.nx + f.tx - 1) / f.tx) * ((c->g.ny + f.ty - 1) / f.ty) * 152.0 /
+               c->nsm;
+    };
+    const double b = blocks(0), p = b <= 152.0 ? 35.0 : 9.0 + 34.5 * std::ceil(b / 304.0);
+    const double m = std::max(22.3, 14.0 + 0.0523 * blocks(1));
+    const double s = std::max(20.0, 11.0 + 0.0365 * blocks(2));
+    return mixed_tile_kernel(p <= m && p <= s ? 0 : m <= s ? 1 : 2);
+}
+
 // One step of a 2D grid.  ustar (FP64 RK2 only, optional): where stage 1
 // writes U* (default: the context's stage buffer).
 static mxe_status launch_2d_step(mxe_ctx* c, double t_end, double dt_fixed,
@@ -926,16 +939,17 @@ static mxe_status launch_2d_step(mxe_ctx* c, double t_end, double dt_fixed,
                              : (b3 ? mxe_stage14_2d_mixed_b3 : mxe_stage14_2d_mixed);
         const size_t smem = stage14_2d_mixed_smem(pl, c->stage_occ);
         // packed planar stage: its own kernel and tile
+        const MixedTile tl = mixed_tile(c);
+        const dim3 gp((c->g.nx + tl.tx - 1) / tl.tx, (c->g.ny + tl.ty - 1) / tl.ty);
         auto launch = [&]() {
             if (!packed) {
                 kern<<<grid, 256, smem, c->stream>>>(a, fparams(c), c->mp);
                 return;
             }
-            const int tx = stage14_2d_mixed_x2_tile_x(), ty = stage14_2d_mixed_x2_tile_y();
-            dim3 gp((c->g.nx + tx - 1) / tx, (c->g.ny + ty - 1) / ty);
-            mxe_stage14_2d_mixed_planar_x2<<<gp, stage14_2d_mixed_x2_threads(),
-                                             stage14_2d_mixed_x2_smem(), c->stream>>>(
-                a, fparams(c), c->mp);
+            ParamsT<float> p = fparams(c);
+            MixedPolicy mp = c->mp;
+            void* args[] = {&a, &p, &mp};
+            cudaLaunchKernel(tl.kern, gp, dim3(tl.threads), args, tl.smem, c->stream);
         };
         a.Ubase = c->U;
         a.Uout = c->U;

@@ -70,6 +70,14 @@ __device__ __forceinline__ float narrow(double x) {
     return __uint_as_float((h & 0x80000000u) | f);
 }
 
+// (float)x, rounded to nearest, by integer operations in FP32's normal range
+__device__ __forceinline__ float to_f32(double x) {
+    const unsigned e = (hi32(x) >> 20) & 0x7ffu;
+    if (e - 898u > 250u) return (float)x;
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    return narrow(__longlong_as_double((long long)(b + 0x0fffffffull + ((b >> 29) & 1ull))));
+}
+
 // ---------------------------------------------------------------- 1/x, 1/sqrt(x)
 __device__ __forceinline__ float rcp32(float x) {
     float r;

@@ -496,8 +496,16 @@ struct TileGeo {
     // limiter work items: the owned cells (both directions), then the halo
     // columns (x only) and the halo rows (y only)
     static constexpr int NLIM = NC + 2 * TY + 2 * TX;
+    // y faces start on the warp after the last x face where all fit in one pass
+    static constexpr int NFXW = (NFX + 31) / 32 * 32;
+    static constexpr int YOFF = NFXW + NFY <= NT ? NFXW : 0;
 };
 using TileP = TileGeo<31, 18, 320>;
+// Smaller tiles for grids of few TileP tiles, which would leave SMs idle; x
+// and y faces of the smallest one are evaluated side by side by different
+// warps.  mixed_tile() in mxe_capi.cu chooses and has the times.
+using TileM = TileGeo<31, 7, 256>;
+using TileS = TileGeo<15, 7, 256>;
 
 // shared memory of the packed stage: stencil box, x and y face fluxes,
 // limiters, reduction scratch
@@ -516,7 +524,7 @@ __device__ __noinline__ float cell_rate(const double* U, long long fstride, floa
     for (int k = 0; k < PH::NF; ++k) Uc[k] = U[PH::ufield(k) * fstride];
     PH::cons2prim_fast(Uc, Q);
 #pragma unroll
-    for (int k = 0; k < PH::NF; ++k) W[k] = (float)Q[k];
+    for (int k = 0; k < PH::NF; ++k) W[k] = f64::to_f32(Q[k]);
     const float r = rn::rate<PH::NF>(W, sigma_lim, k_ws, idx, idy);
     return r >= 0.0f ? r : __int_as_float(0x7f800000);             // NaN -> inf
 }
@@ -634,7 +642,8 @@ __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const Param
         for (int k = 0; k < NF; ++k) Fx[k * G::NFX + f] = F[k];
     }
 #pragma unroll 1
-    for (int f = tid; f < G::NFY; f += G::NT) {       // y faces: TY + 1 rows of TX
+    for (int f = tid - G::YOFF; f < G::NFY; f += G::NT) {       // y faces: TY + 1 rows of TX
+        if (G::YOFF > 0 && f < 0) break;
         const int fx = f % G::TX, fy = f / G::TX;
         float F[NF];
         face_flux_x2<1, G::NBOX>(W, (fy + 1) * G::BX + fx + 2, G::BX, phy[fy * G::TX + fx],
@@ -753,15 +762,27 @@ __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const Param
 }
 
 // planar state, packed face-state pairs, two blocks per SM
-extern "C" __global__ void __launch_bounds__(TileP::NT, 2)
-mxe_stage14_2d_mixed_planar_x2(const Stage2DArgs a, const ParamsT<float> p,
-                               const MixedPolicy mp) {
-    stage_mixed_x2<TileP>(a, p, mp);
+#define MXE_X2(NAME, G)                                                                   \
+    extern "C" __global__ void __launch_bounds__(G::NT, 2)                                \
+    NAME(const Stage2DArgs a, const ParamsT<float> p, const MixedPolicy mp) {             \
+        stage_mixed_x2<G>(a, p, mp);                                                      \
+    }
+MXE_X2(mxe_stage14_2d_mixed_planar_x2, TileP)
+MXE_X2(mxe_stage14_2d_mixed_planar_x2_m, TileM)
+MXE_X2(mxe_stage14_2d_mixed_planar_x2_s, TileS)
+#undef MXE_X2
+
+// 0: TileP, 1: TileM, 2: TileS
+MixedTile mixed_tile_kernel(int n) {
+    if (n == 2)
+        return {(const void*)mxe_stage14_2d_mixed_planar_x2_s, TileS::TX, TileS::TY, TileS::NT,
+                smem_mixed_x2<TileS>()};
+    if (n == 1)
+        return {(const void*)mxe_stage14_2d_mixed_planar_x2_m, TileM::TX, TileM::TY, TileM::NT,
+                smem_mixed_x2<TileM>()};
+    return {(const void*)mxe_stage14_2d_mixed_planar_x2, TileP::TX, TileP::TY, TileP::NT,
+            smem_mixed_x2<TileP>()};
 }
-size_t stage14_2d_mixed_x2_smem() { return smem_mixed_x2<TileP>(); }
-int stage14_2d_mixed_x2_threads() { return TileP::NT; }
-int stage14_2d_mixed_x2_tile_x() { return TileP::TX; }
-int stage14_2d_mixed_x2_tile_y() { return TileP::TY; }
 
 size_t stage14_2d_mixed_smem(bool planar, int blocks_per_sm) {
     if (!planar) return smem_mixed<14, false>();      // both general variants
@@ -780,7 +801,7 @@ __device__ __forceinline__ void resync(const double* U, float* W, const Grid2D& 
     for (int k = 0; k < PH::NF; ++k) Uc[k] = U[o + PH::ufield(k) * g.fstride];
     PH::cons2prim_fast(Uc, Q);
 #pragma unroll
-    for (int k = 0; k < PH::NF; ++k) W[o + k * g.fstride] = (float)Q[k];
+    for (int k = 0; k < PH::NF; ++k) W[o + k * g.fstride] = f64::to_f32(Q[k]);
 }
 extern "C" __global__ void mxe_resync14_2d(const double* U, float* W, Grid2D g) {
     resync<PhysGeneral>(U, W, g);

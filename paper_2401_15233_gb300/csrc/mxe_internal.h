@@ -72,6 +72,14 @@ struct F64Tile {
     size_t smem;
 };
 
+// One tile variant of the packed mixed 2D stage kernel, whose parameters are
+// (Stage2DArgs, ParamsT<float>, MixedPolicy)
+struct MixedTile {
+    const void* kern;
+    int tx, ty, threads;
+    size_t smem;
+};
+
 // ---- 1D tubes ----
 struct TubeDesc {
     long long off;                  // element offset of the tube's field 0

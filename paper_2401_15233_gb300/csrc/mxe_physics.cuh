@@ -302,7 +302,9 @@ __device__ __forceinline__ void prim2cons14(const T* Q, T* U) {
 template <class T>
 __device__ __forceinline__ void cons2prim14(const T* U, T* Q) {
     T rho = U[0];
-    T ir = T(1) / rho;
+    T ir;
+    if constexpr (sizeof(T) == 8) ir = f64::rcp(rho);
+    else ir = T(1) / rho;
     T ux = U[1] * ir, uy = U[2] * ir, uz = U[3] * ir;
     T Pxx = U[4] - rho * ux * ux, Pxy = U[5] - rho * ux * uy, Pxz = U[6] - rho * ux * uz;
     T Pyy = U[7] - rho * uy * uy, Pyz = U[8] - rho * uy * uz, Pzz = U[9] - rho * uz * uz;

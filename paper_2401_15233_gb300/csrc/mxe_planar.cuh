@@ -48,7 +48,9 @@ __device__ __forceinline__ void prim2cons_p(const T* Q, T* U) {
 template <class T>
 __device__ __forceinline__ void cons2prim_p(const T* U, T* Q) {
     T rho = U[0];
-    T ir = T(1) / rho;
+    T ir;
+    if constexpr (sizeof(T) == 8) ir = f64::rcp(rho);
+    else ir = T(1) / rho;
     T ux = U[1] * ir, uy = U[2] * ir;
     T Pxx = U[3] - U[1] * ux, Pxy = U[4] - U[1] * uy, Pyy = U[5] - U[2] * uy, Pzz = U[6];
     T u2 = ux * ux + uy * uy;

@@ -208,8 +208,10 @@ mxe_status mxe_step_dt(mxe_ctx *ctx, int n, const double *dts);
 mxe_status mxe_set_mixed_policy(mxe_ctx *ctx, double sigma_lo, double sigma_hi,
                                 double det_min, int resync_every);
 
-/* 2D MXE_MIXED only: launch shape of the fused stage kernels (planar
- * ten-field and general fourteen-field).  blocks_per_sm = 3 (default): at
+/* 2D MXE_MIXED only: launch shape of the fused stage kernels with scalar face
+ * states (planar ten-field and general fourteen-field; packed face states,
+ * mxe_set_face_packing, need 3 here and choose their own tile and shape).
+ * blocks_per_sm = 3 (default): at
  * most 80 registers per thread, three blocks per SM, the final stage's own
  * cells prefetched into L2; 2: up to 128 registers per thread, two blocks per
  * SM (planar: the final stage prefetches its own cells' U^n and W^n into
@@ -218,7 +220,7 @@ mxe_status mxe_set_mixed_policy(mxe_ctx *ctx, double sigma_lo, double sigma_hi,
  * context. */
 mxe_status mxe_set_stage_occupancy(mxe_ctx *ctx, int blocks_per_sm);
 
-/* 2D MXE_MIXED only, planar states at three blocks per SM: how the two face
+/* 2D MXE_MIXED only, while the stage occupancy is 3: how the two face
  * states of a face are evaluated (closure Eqs. closure-14mom-Qijk/Rijkk/
  * Sijjkk, wave speeds Eq. 14mom-approx-ws-equations, Sec. 3.1 flux).
  * packed = 1 (default): as one pair in packed FP32 (f32x2) arithmetic, the

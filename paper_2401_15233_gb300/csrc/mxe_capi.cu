@@ -47,8 +47,8 @@ extern "C" __global__ void mxe_rate14_2d_mixed_planar(const float* W, Grid2D g,
                                                       ParamsT<float> p, float idxf, float idyf,
                                                       DevClock* clk, int slot);
 size_t stage14_2d_mixed_smem(bool planar, int blocks_per_sm);
-MixedTile mixed_tile_kernel(int n);
-const void* tubes_mixed_kernel(bool planar, int nt);
+MixedTile mixed_tile_kernel(bool planar, bool rus, int n);
+const void* tubes_mixed_kernel(bool planar, int nt, bool rus);
 cudaError_t adj_stage(const double* U, const double* V, double coef, const double* b1,
                       const double* b2, double* out, double* P, double* Cx, double* Cy,
                       double* gbar, double* taubar, const Grid2D& g, const ParamsT<double>& p,
@@ -343,7 +343,7 @@ static mxe_status team_plans(mxe_ctx* c) {
         for (int ch : {31, 63}) {
             int v = 0;
             CK(c->mixed ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                              &v, tubes_mixed_kernel(pl, 128), 128, tubes_mixed_smem(pl, 128))
+                              &v, tubes_mixed_kernel(pl, 128, c->sp.flux == MXE_FLUX_RUSANOV), 128, tubes_mixed_smem(pl, 128))
                         : cudaOccupancyMaxActiveBlocksPerMultiprocessor(
                               &v, tubes_f64_kernel(c->nf, pl, ch), tubes_threads(), 0));
             per = std::min(per, v);
@@ -396,7 +396,7 @@ static mxe_status tubes_setup(mxe_ctx* c) {
     CK(cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, dev));
     for (int pl = 0; pl < 2; ++pl)
         for (int nt = 128; nt <= 256; nt *= 2)
-            CK(cudaFuncSetAttribute(tubes_mixed_kernel(pl, nt),
+            CK(cudaFuncSetAttribute(tubes_mixed_kernel(pl, nt, c->sp.flux == MXE_FLUX_RUSANOV),
                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)tubes_mixed_smem(pl, nt)));
     return team_plans(c);
@@ -475,10 +475,11 @@ extern "C" mxe_status mxe_create(const mxe_config* cfg, mxe_ctx** out) {
             e = cudaFuncSetAttribute(mxe_stage14_2d_mixed_planar_b3,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)stage14_2d_mixed_smem(true, 3));
-        for (int n = 0; n < 3 && e == cudaSuccess && c->mixed; ++n)
-            e = cudaFuncSetAttribute(mixed_tile_kernel(n).kern,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)mixed_tile_kernel(n).smem);
+        for (int n = 0; n < 12 && e == cudaSuccess && c->mixed; ++n) {
+            const MixedTile f = mixed_tile_kernel(n & 1, n & 2, n >> 2);
+            e = cudaFuncSetAttribute(f.kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)f.smem);
+        }
         if (e == cudaSuccess && c->mixed)
             e = cudaFuncSetAttribute(mxe_stage14_2d_mixed_b3,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -894,18 +895,28 @@ static F64Tile f64_tile(const mxe_ctx* c, bool pl) {
 //   31 x 18     35        35         35         43         44         76         224
 //   31 x  7     22        22         26         36         51         80         273
 //   15 x  7     18        21         29         41         67        103         386
-// (one tile before: 33 on 48 x 48, 262 on 1024 x 1024).  Small grids pay for the
-// passes of one block, then for each block; TileP's come two to an SM, in waves.
-static MixedTile mixed_tile(const mxe_ctx* c) {
+// (one tile before: 33 on 48 x 48, 262 on 1024 x 1024); general states:
+//   31 x 15     39        40         40         52         74         93         330
+//   31 x  7     27        27         33         45         67        107         374
+//   15 x  7     22        25         33         52         89        138         540
+// (scalar faces before: 35 on 48 x 48, 92 on 400 x 400).  Small grids pay for the
+// passes of one block, then for each block; the large tiles come two to an SM,
+// in waves.
+static MixedTile mixed_tile(const mxe_ctx* c, bool pl) {
+    const bool rus = c->sp.flux == MXE_FLUX_RUSANOV;
     auto blocks = [&](int n) {
-        const MixedTile f = mixed_tile_kernel(n);
+        const MixedTile f = mixed_tile_kernel(pl, rus, n);
         return (double)((c->g.nx + f.tx - 1) / f.tx) * ((c->g.ny + f.ty - 1) / f.ty) * 152.0 /
                c->nsm;
     };
-    const double b = blocks(0), p = b <= 152.0 ? 35.0 : 9.0 + 34.5 * std::ceil(b / 304.0);
-    const double m = std::max(22.3, 14.0 + 0.0523 * blocks(1));
-    const double s = std::max(20.0, 11.0 + 0.0365 * blocks(2));
-    return mixed_tile_kernel(p <= m && p <= s ? 0 : m <= s ? 1 : 2);
+    // us: large tile alone, offset and wave; small tiles alone, offset and block
+    static const double t[2][9] = {{39.5, 8.0, 43.0, 27.0, 18.0, 0.0705, 22.5, 14.0, 0.0465},
+                                   {35.0, 9.0, 34.5, 22.3, 14.0, 0.0523, 20.0, 11.0, 0.0365}};
+    const double* w = t[pl];
+    const double b = blocks(0), p = b <= 152.0 ? w[0] : w[1] + w[2] * std::ceil(b / 304.0);
+    const double m = std::max(w[3], w[4] + w[5] * blocks(1));
+    const double s = std::max(w[6], w[7] + w[8] * blocks(2));
+    return mixed_tile_kernel(pl, rus, p <= m && p <= s ? 0 : m <= s ? 1 : 2);
 }
 
 // One step of a 2D grid.  ustar (FP64 RK2 only, optional): where stage 1
@@ -934,12 +945,12 @@ static mxe_status launch_2d_step(mxe_ctx* c, double t_end, double dt_fixed,
         // three blocks per SM (L2 prefetch) or two (planar: with the final
         // stage's shared-memory prefetch); the same kernel for both stages
         const bool b3 = c->stage_occ == 3;
-        const bool packed = pl && b3 && c->face_packed;
+        const bool packed = b3 && c->face_packed;
         const auto kern = pl ? (b3 ? mxe_stage14_2d_mixed_planar_b3 : mxe_stage14_2d_mixed_planar)
                              : (b3 ? mxe_stage14_2d_mixed_b3 : mxe_stage14_2d_mixed);
         const size_t smem = stage14_2d_mixed_smem(pl, c->stage_occ);
-        // packed planar stage: its own kernel and tile
-        const MixedTile tl = mixed_tile(c);
+        // packed stage: its own kernel and tile
+        const MixedTile tl = mixed_tile(c, pl);
         const dim3 gp((c->g.nx + tl.tx - 1) / tl.tx, (c->g.ny + tl.ty - 1) / tl.ty);
         auto launch = [&]() {
             if (!packed) {
@@ -1142,7 +1153,7 @@ static void tube_fill_split(const mxe_ctx* c, TubeLaunch* L, const std::vector<d
 static mxe_status tube_launch_shape(mxe_ctx* c, int nt, int cl, TubeLaunch* L,
                                     const std::vector<double>* est = nullptr) {
     const bool pl = tubes_planar(c);
-    L->kern = tubes_mixed_kernel(pl, nt);
+    L->kern = tubes_mixed_kernel(pl, nt, c->sp.flux == MXE_FLUX_RUSANOV);
     L->smem = tubes_mixed_smem(pl, nt);
     L->nt = nt;
     L->cl = cl;
@@ -1182,7 +1193,7 @@ static mxe_status tube_launch(mxe_ctx* c, bool to_time, TubeLaunch* L,
     if (c->shape_set || c->team_ctas[k] == 0)
         return tube_launch_shape(c, c->tune_nt, c->tune_cl, L, est);
     const bool pl = tubes_planar(c);
-    L->kern = tubes_mixed_kernel(pl, 128);
+    L->kern = tubes_mixed_kernel(pl, 128, c->sp.flux == MXE_FLUX_RUSANOV);
     L->smem = tubes_mixed_smem(pl, 128);
     L->nt = 128;
     L->cl = 1;

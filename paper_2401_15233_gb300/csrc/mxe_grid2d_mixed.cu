@@ -460,7 +460,7 @@ mxe_stage14_2d_mixed_planar_b3(const Stage2DArgs a, const ParamsT<float> p,
 }
 
 // ---------------------------------------------------------------------------
-// Packed planar stage (the default for planar states).  A block of 320
+// Packed stage (the default).  Planar states: a block of 320
 // threads owns a TX x TY tile; every thread evaluates up to two x faces and
 // two y faces as packed pairs of face states, the limiters of about two
 // cells (both directions of an interior cell in one evaluation), and
@@ -501,6 +501,9 @@ struct TileGeo {
     static constexpr int YOFF = NFXW + NFY <= NT ? NFXW : 0;
 };
 using TileP = TileGeo<31, 18, 320>;
+// General states: 14 fields of the box and of the fluxes fill 96 KB, and the
+// face evaluation wants 128 registers.
+using TileG = TileGeo<31, 15, 256>;
 // Smaller tiles for grids of few TileP tiles, which would leave SMs idle; x
 // and y faces of the smallest one are evaluated side by side by different
 // warps.  mixed_tile() in mxe_capi.cu chooses and has the times.
@@ -509,9 +512,9 @@ using TileS = TileGeo<15, 7, 256>;
 
 // shared memory of the packed stage: stencil box, x and y face fluxes,
 // limiters, reduction scratch
-template <class G>
+template <class G, int NF>
 constexpr size_t smem_mixed_x2() {
-    return sizeof(float) * (NP * G::NBOX + NP * G::NFX + NP * G::NFY + G::NPX + G::NPY + G::NT / 32);
+    return sizeof(float) * (NF * (G::NBOX + G::NFX + G::NFY) + G::NPX + G::NPY + G::NT / 32);
 }
 
 // CFL rate of the cell whose conserved state starts at U (see mxe_rate32.cuh)
@@ -529,11 +532,10 @@ __device__ __noinline__ float cell_rate(const double* U, long long fstride, floa
     return r >= 0.0f ? r : __int_as_float(0x7f800000);             // NaN -> inf
 }
 
-template <class G>
+template <class PH, class G, bool RUS>
 __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const ParamsT<float>& p,
                                                const MixedPolicy& mp) {
-    using PH = PhysPlanar;
-    constexpr int NF = NP;
+    constexpr int NF = PH::NF;
     extern __shared__ __align__(16) double smd[];
     float* W = (float*)smd;                          // [NF][BY][BX]
     float* Fx = W + NF * G::NBOX;                    // [NF][TY][TX+1]
@@ -636,7 +638,7 @@ __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const Param
     for (int f = tid; f < G::NFX; f += G::NT) {       // x faces: TY rows of TX + 1
         const int fx = f % (G::TX + 1), fy = f / (G::TX + 1);
         float F[NF];
-        face_flux_x2<0, G::NBOX>(W, (fy + 2) * G::BX + fx + 1, 1, phx[fy * (G::TX + 2) + fx],
+        face_flux_x2<PH, 0, G::NBOX, RUS>(W, (fy + 2) * G::BX + fx + 1, 1, phx[fy * (G::TX + 2) + fx],
                                  phx[fy * (G::TX + 2) + fx + 1], p, mp, sl64, kw64, F, nflag);
 #pragma unroll
         for (int k = 0; k < NF; ++k) Fx[k * G::NFX + f] = F[k];
@@ -646,7 +648,7 @@ __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const Param
         if (G::YOFF > 0 && f < 0) break;
         const int fx = f % G::TX, fy = f / G::TX;
         float F[NF];
-        face_flux_x2<1, G::NBOX>(W, (fy + 1) * G::BX + fx + 2, G::BX, phy[fy * G::TX + fx],
+        face_flux_x2<PH, 1, G::NBOX, RUS>(W, (fy + 1) * G::BX + fx + 2, G::BX, phy[fy * G::TX + fx],
                                  phy[(fy + 1) * G::TX + fx], p, mp, sl64, kw64, F, nflag);
 #pragma unroll
         for (int k = 0; k < NF; ++k) Fy[k * G::NFY + f] = F[k];
@@ -740,7 +742,8 @@ __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const Param
             if (PH::nonpositive(Wn)) atomicOr(&a.clk->status, ST_NONPOSITIVE);
             if (bad) atomicOr(&a.clk->status, ST_NONFINITE);
             float ax, ay;
-            x2::rates_x2(Wn, p.sigma_lim, p.k_ws, ax, ay);
+            if constexpr (NF == NP) x2::rates_x2(Wn, p.sigma_lim, p.k_ws, ax, ay);
+            else x2::rates14_x2(Wn, p.sigma_lim, p.k_ws, ax, ay);
             float rc = ax * a.idxf + ay * a.idyf;
             if (!(rc >= 0.0f)) rc = __int_as_float(0x7f800000);     // NaN -> inf
             if (rc >= r) {
@@ -761,27 +764,41 @@ __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const Param
     }
 }
 
-// planar state, packed face-state pairs, two blocks per SM
-#define MXE_X2(NAME, G)                                                                   \
+// packed face-state pairs, two blocks per SM
+#define MXE_X2(NAME, PH, G, RUS)                                                             \
     extern "C" __global__ void __launch_bounds__(G::NT, 2)                                \
     NAME(const Stage2DArgs a, const ParamsT<float> p, const MixedPolicy mp) {             \
-        stage_mixed_x2<G>(a, p, mp);                                                      \
+        stage_mixed_x2<PH, G, RUS>(a, p, mp);                                                  \
     }
-MXE_X2(mxe_stage14_2d_mixed_planar_x2, TileP)
-MXE_X2(mxe_stage14_2d_mixed_planar_x2_m, TileM)
-MXE_X2(mxe_stage14_2d_mixed_planar_x2_s, TileS)
+MXE_X2(mxe_stage14_2d_mixed_planar_x2, PhysPlanar, TileP, false)
+MXE_X2(mxe_stage14_2d_mixed_planar_x2_rus, PhysPlanar, TileP, true)
+MXE_X2(mxe_stage14_2d_mixed_planar_x2_m, PhysPlanar, TileM, false)
+MXE_X2(mxe_stage14_2d_mixed_planar_x2_m_rus, PhysPlanar, TileM, true)
+MXE_X2(mxe_stage14_2d_mixed_planar_x2_s, PhysPlanar, TileS, false)
+MXE_X2(mxe_stage14_2d_mixed_planar_x2_s_rus, PhysPlanar, TileS, true)
+MXE_X2(mxe_stage14_2d_mixed_x2, PhysGeneral, TileG, false)
+MXE_X2(mxe_stage14_2d_mixed_x2_rus, PhysGeneral, TileG, true)
+MXE_X2(mxe_stage14_2d_mixed_x2_m, PhysGeneral, TileM, false)
+MXE_X2(mxe_stage14_2d_mixed_x2_m_rus, PhysGeneral, TileM, true)
+MXE_X2(mxe_stage14_2d_mixed_x2_s, PhysGeneral, TileS, false)
+MXE_X2(mxe_stage14_2d_mixed_x2_s_rus, PhysGeneral, TileS, true)
 #undef MXE_X2
 
-// 0: TileP, 1: TileM, 2: TileS
-MixedTile mixed_tile_kernel(int n) {
-    if (n == 2)
-        return {(const void*)mxe_stage14_2d_mixed_planar_x2_s, TileS::TX, TileS::TY, TileS::NT,
-                smem_mixed_x2<TileS>()};
-    if (n == 1)
-        return {(const void*)mxe_stage14_2d_mixed_planar_x2_m, TileM::TX, TileM::TY, TileM::NT,
-                smem_mixed_x2<TileM>()};
-    return {(const void*)mxe_stage14_2d_mixed_planar_x2, TileP::TX, TileP::TY, TileP::NT,
-            smem_mixed_x2<TileP>()};
+template <class PH, class G>
+static MixedTile tile_of(void (*kern)(const Stage2DArgs, const ParamsT<float>, const MixedPolicy)) {
+    return {(const void*)kern, G::TX, G::TY, G::NT, smem_mixed_x2<G, PH::NF>()};
+}
+// n = 0: TileP or TileG, 1: TileM, 2: TileS
+MixedTile mixed_tile_kernel(bool planar, bool rus, int n) {
+#define MXE_TILE(NAME, PH, G) tile_of<PH, G>(rus ? NAME##_rus : NAME)
+    if (planar)
+        return n == 2   ? MXE_TILE(mxe_stage14_2d_mixed_planar_x2_s, PhysPlanar, TileS)
+               : n == 1 ? MXE_TILE(mxe_stage14_2d_mixed_planar_x2_m, PhysPlanar, TileM)
+                        : MXE_TILE(mxe_stage14_2d_mixed_planar_x2, PhysPlanar, TileP);
+    return n == 2   ? MXE_TILE(mxe_stage14_2d_mixed_x2_s, PhysGeneral, TileS)
+           : n == 1 ? MXE_TILE(mxe_stage14_2d_mixed_x2_m, PhysGeneral, TileM)
+                    : MXE_TILE(mxe_stage14_2d_mixed_x2, PhysGeneral, TileG);
+#undef MXE_TILE
 }
 
 size_t stage14_2d_mixed_smem(bool planar, int blocks_per_sm) {

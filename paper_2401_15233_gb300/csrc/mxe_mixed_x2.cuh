@@ -5,7 +5,7 @@
 // conversion of the accumulator's increments.
 #pragma once
 #include "mxe_mixed.cuh"
-#include "mxe_planar_x2.cuh"
+#include "mxe_general_x2.cuh"
 
 namespace mxe {
 
@@ -60,18 +60,18 @@ template <int NF>
 struct FaceFluxOut {
     float f[NF];
 };
-template <int K>
-__device__ __noinline__ FaceFluxOut<NP> face_flux_fp64(FacePairIn<NP> in, double sl, double kw,
-                                                       int flux) {
-    constexpr int NF = NP;
+template <class PH, int K>
+__device__ __noinline__ FaceFluxOut<PH::NF> face_flux_fp64(FacePairIn<PH::NF> in, double sl,
+                                                           double kw, int flux) {
+    constexpr int NF = PH::NF;
     double QL[NF], QR[NF], UL[NF], UR[NF], FL[NF], FR[NF], lminL, lmaxL, lminR, lmaxR;
 #pragma unroll
     for (int k = 0; k < NF; ++k) {
         QL[k] = (double)in.q[k];
         QR[k] = (double)in.q[NF + k];
     }
-    PhysPlanar::face<double, K>(QL, sl, kw, UL, FL, lminL, lmaxL);
-    PhysPlanar::face<double, K>(QR, sl, kw, UR, FR, lminR, lmaxR);
+    PH::template face<double, K>(QL, sl, kw, UL, FL, lminL, lmaxL);
+    PH::template face<double, K>(QR, sl, kw, UR, FR, lminR, lmaxR);
     FaceFluxOut<NF> r;
     if (flux == 1) {
         double sp = fmax(fmax(fabs(lminL), fabs(lmaxL)), fmax(fabs(lminR), fabs(lmaxR)));
@@ -92,18 +92,19 @@ __device__ __noinline__ FaceFluxOut<NP> face_flux_fp64(FacePairIn<NP> in, double
 }
 
 // Both face states of the face between box cells cl and cl + stride along K
-// (planar state), evaluated as one packed FP32 pair (left state in lane x,
+// evaluated as one packed FP32 pair (left state in lane x,
 // right in lane y): the reconstruction shares the four stencil cells, and
 // no face state is staged in shared memory.  A face with an ill-conditioned
 // closure in either state (the policy of face_state_m) takes its flux from
-// face_flux_fp64 instead.
-template <int K, int NBOX>
+// face_flux_fp64 instead.  RUS: the flux, Rusanov or HLL (a kernel of each: with
+// both in one, HLL stages spilled ten times as much and took 18 % longer).
+template <class PH, int K, int NBOX, bool RUS>
 __device__ __forceinline__ void face_flux_x2(const float* W, int cl, int stride, float phl,
                                              float phr, const ParamsT<float>& p,
                                              const MixedPolicy& mp, double sl64, double kw64,
                                              float* F, unsigned& nflag) {
     using namespace x2;
-    constexpr int NF = NP;
+    constexpr int NF = PH::NF;
     v2 Q[NF];
     auto reconstruct = [&]() {
         const v2 hp = make_float2(0.25f * phl, -0.25f * phr);
@@ -116,7 +117,17 @@ __device__ __forceinline__ void face_flux_x2(const float* W, int cl, int stride,
     };
     reconstruct();
     v2 sig, det;
-    face_eval_x2<K>(Q, p.sigma_lim, p.k_ws, p.flux, F, sig, det);
+    float D[NF];             // the jumps Q_R - Q_L (Rusanov)
+    if (RUS) {
+#pragma unroll
+        for (int k = 0; k < NF; ++k) {
+            const float* w = W + k * NBOX + cl;
+            const float w0 = w[0], w1 = w[stride];
+            D[k] = (w1 - w0) - 0.25f * fmaf(phr, w[2 * stride] - w0, phl * (w1 - w[-stride]));
+        }
+    }
+    if constexpr (NF == NP) face_eval_x2<K, RUS>(Q, D, p.sigma_lim, p.k_ws, F, sig, det);
+    else face_eval14_x2<K, RUS>(Q, D, p.sigma_lim, p.k_ws, F, sig, det);
     if (mp.sig_lo > 0.0f || mp.sig_hi < 1.0f || mp.det_min > 0.0f) {
         const bool fx = (sig.x >= p.sigma_lim && sig.x < mp.sig_lo) || sig.x > mp.sig_hi ||
                         det.x < mp.det_min || !(sig.x == sig.x);
@@ -132,7 +143,7 @@ __device__ __forceinline__ void face_flux_x2(const float* W, int cl, int stride,
                 in.q[k] = Q[k].x;
                 in.q[NF + k] = Q[k].y;
             }
-            FaceFluxOut<NF> r = face_flux_fp64<K>(in, sl64, kw64, p.flux);
+            FaceFluxOut<NF> r = face_flux_fp64<PH, K>(in, sl64, kw64, p.flux);
 #pragma unroll
             for (int k = 0; k < NF; ++k) F[k] = r.f[k];
         }

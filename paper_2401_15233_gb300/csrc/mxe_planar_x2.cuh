@@ -149,9 +149,10 @@ __device__ __forceinline__ void rates_x2(const float* Q, float sigma_lim, float 
 struct FluxWeights {
     float l, r, u;
 };
-__device__ __forceinline__ FluxWeights flux_weights(v2 lmin, v2 lmax, int flux) {
+template <bool RUS>
+__device__ __forceinline__ FluxWeights flux_weights(v2 lmin, v2 lmax) {
     FluxWeights w;
-    if (flux == 1) {
+    if (RUS) {
         const float s = fmaxf(fmaxf(fabsf(lmin.x), fabsf(lmax.x)),
                               fmaxf(fabsf(lmin.y), fabsf(lmax.y)));
         w.l = w.r = 0.5f;
@@ -172,8 +173,14 @@ __device__ __forceinline__ FluxWeights flux_weights(v2 lmin, v2 lmax, int flux) 
     }
     return w;
 }
-__device__ __forceinline__ float weigh(const FluxWeights& w, v2 F, v2 U) {
-    return fmaf(w.u, U.y - U.x, fmaf(w.l, F.x, w.r * F.y));
+// one field's face flux from the pair's F and the jump dU = U_R - U_L
+__device__ __forceinline__ float weigh(const FluxWeights& w, v2 F, float dU) {
+    return fmaf(w.u, dU, fmaf(w.l, F.x, w.r * F.y));
+}
+__device__ __forceinline__ float jump(v2 U) { return U.y - U.x; }
+// the jump of a product x y from the jumps of its factors
+__device__ __forceinline__ float djump(v2 x, float dx, v2 y, float dy) {
+    return fmaf(x.y, dy, y.x * dx);
 }
 
 // Numerical flux Fn along K of a face with the states Q (left in lane x, right
@@ -181,11 +188,15 @@ __device__ __forceinline__ float weigh(const FluxWeights& w, v2 F, v2 U) {
 // mixed policy checks).  The wave speeds need the dimensionless state alone,
 // so they come first: each field's U and K-flux then goes into Fn as it is
 // formed, and no U or F of the pair stays in registers.
+// RUS: the jumps of the conserved moments are formed from those of the
+// primitives, D[k] = Q_R - Q_L, which come from the stencil's differences: Rusanov
+// weighs them with the largest speed (HLL, away from stagnation, with the
+// small one), and differences of rounded moments left 3 to 6 times HLL's error.
 // closure slice: QK = (Q_KKK, Q_KKO, Q_KOO, Q_Kzz), RK = (R_KKjj, R_OKjj),
 // SK = S_Kiijj (see closure_p); conserved state and flux: prim2cons_p, flux_p.
-template <int K>
-__device__ __forceinline__ void face_eval_x2(const v2* Q, float sigma_lim, float k_ws, int flux,
-                                             float* Fn, v2& sig, v2& det) {
+template <int K, bool RUS>
+__device__ __forceinline__ void face_eval_x2(const v2* Q, const float* D, float sigma_lim,
+                                             float k_ws, float* Fn, v2& sig, v2& det) {
     DimX2 g;
     dimless_x2(Q, g);
     sig = g.sig;
@@ -200,7 +211,7 @@ __device__ __forceinline__ void face_eval_x2(const v2* Q, float sigma_lim, float
         lam_core_x2(K == 0 ? g.a : g.d, K == 0 ? g.qx : g.qy, abs_(K == 0 ? g.qy : g.qx), sb,
                     isb, ssb, lp, lm);
         const v2 ks = mul(g.sq, S(k_ws));
-        w = flux_weights(fma(lm, neg(ks), uK), fma(lp, ks, uK), flux);
+        w = flux_weights<RUS>(fma(lm, neg(ks), uK), fma(lp, ks, uK));
     }
     // second moments and the pressure work need Q_K.. of the closure, with
     // v = B^-1 q* (scaled by 4: B/4 = (T2/2) P* + P*^3), w = P* v
@@ -255,31 +266,53 @@ __device__ __forceinline__ void face_eval_x2(const v2* Q, float sigma_lim, float
     // conserved state and flux u_K U + central part, field by field
     const v2 rho = Q[0], Pxy = Q[4], PxK = K == 0 ? Q[3] : Pxy, PyK = K == 0 ? Pxy : Q[5];
     const v2 mx = mul(rho, ux), my = mul(rho, uy);
-    Fn[0] = weigh(w, K == 0 ? mx : my, rho);
-    Fn[1] = weigh(w, fma(uK, mx, PxK), mx);
-    Fn[2] = weigh(w, fma(uK, my, PyK), my);
+    const float dmx = RUS ? djump(rho, D[0], ux, D[1]) : jump(mx);
+    const float dmy = RUS ? djump(rho, D[0], uy, D[2]) : jump(my);
+    Fn[0] = weigh(w, K == 0 ? mx : my, RUS ? D[0] : jump(rho));
+    Fn[1] = weigh(w, fma(uK, mx, PxK), dmx);
+    Fn[2] = weigh(w, fma(uK, my, PyK), dmy);
     {
         const v2 U3 = fma(mx, ux, Q[3]), U4 = fma(mx, uy, Pxy), U5 = fma(my, uy, Q[5]);
-        Fn[3] = weigh(w, fma(uK, U3, fma(add(ux, ux), PxK, K == 0 ? QK[0] : QK[2])), U3);
-        Fn[4] = weigh(w, fma(uK, U4, fma(ux, PyK, fma(uy, PxK, QK[1]))), U4);
-        Fn[5] = weigh(w, fma(uK, U5, fma(add(uy, uy), PyK, K == 0 ? QK[2] : QK[0])), U5);
-        Fn[6] = weigh(w, fma(uK, Q[6], QK[3]), Q[6]);
+        const float d3 = RUS ? djump(mx, dmx, ux, D[1]) + D[3] : jump(U3);
+        const float d4 = RUS ? djump(mx, dmx, uy, D[2]) + D[4] : jump(U4);
+        const float d5 = RUS ? djump(my, dmy, uy, D[2]) + D[5] : jump(U5);
+        Fn[3] = weigh(w, fma(uK, U3, fma(add(ux, ux), PxK, K == 0 ? QK[0] : QK[2])), d3);
+        Fn[4] = weigh(w, fma(uK, U4, fma(ux, PyK, fma(uy, PxK, QK[1]))), d4);
+        Fn[5] = weigh(w, fma(uK, U5, fma(add(uy, uy), PyK, K == 0 ? QK[2] : QK[0])), d5);
+        Fn[6] = weigh(w, fma(uK, Q[6], QK[3]), RUS ? D[6] : jump(Q[6]));
     }
     const v2 u2 = fma(ux, ux, mul(uy, uy)), ru2 = mul(rho, u2), e = add(ru2, g.tr);
     const v2 Pux = fma(Q[3], ux, mul(Pxy, uy)), Puy = fma(Pxy, ux, mul(Q[5], uy));
     const v2 QuK = fma(QK[0], uK, mul(QK[1], uO)), QuO = fma(QK[1], uK, mul(QK[2], uO));
     const v2 gK = fma(K == 0 ? Pux : Puy, S(2.0f), Q[7 + K]);
+    float du2 = 0.0f, dru2 = 0.0f, de = 0.0f, dPx = 0.0f, dPy = 0.0f;
+    if (RUS) {
+        du2 = fmaf(ux.x + ux.y, D[1], (uy.x + uy.y) * D[2]);
+        dru2 = djump(rho, D[0], u2, du2);
+        de = dru2 + (D[3] + D[5] + D[6]);
+        dPx = djump(Q[3], D[3], ux, D[1]) + djump(Pxy, D[4], uy, D[2]);
+        dPy = djump(Pxy, D[4], ux, D[1]) + djump(Q[5], D[5], uy, D[2]);
+    }
     {
         const v2 U7 = fma(ux, e, fma(Pux, S(2.0f), Q[7])), U8 = fma(uy, e, fma(Puy, S(2.0f), Q[8]));
+        const float d7 = RUS ? djump(ux, D[1], e, de) + fmaf(2.0f, dPx, D[7]) : jump(U7);
+        const float d8 = RUS ? djump(uy, D[2], e, de) + fmaf(2.0f, dPy, D[8]) : jump(U8);
         Fn[7] = weigh(w, fma(uK, U7, fma(ux, gK, fma(u2, PxK, fma(K == 0 ? QuK : QuO, S(2.0f),
-                                                                 K == 0 ? RKK : ROK)))), U7);
+                                                                 K == 0 ? RKK : ROK)))), d7);
         Fn[8] = weigh(w, fma(uK, U8, fma(uy, gK, fma(u2, PyK, fma(K == 0 ? QuO : QuK, S(2.0f),
-                                                                 K == 0 ? ROK : RKK)))), U8);
+                                                                 K == 0 ? ROK : RKK)))), d8);
     }
-    const v2 uPq = fma(ux, add(Pux, Q[7]), mul(uy, add(Puy, Q[8])));
-    const v2 U9 = fma(u2, fma(g.tr, S(2.0f), ru2), fma(uPq, S(4.0f), Q[9]));
+    const v2 Pqx = add(Pux, Q[7]), Pqy = add(Puy, Q[8]), e2 = fma(g.tr, S(2.0f), ru2);
+    const v2 uPq = fma(ux, Pqx, mul(uy, Pqy));
+    const v2 U9 = fma(u2, e2, fma(uPq, S(4.0f), Q[9]));
     const v2 uQR = fma(uK, add(QuK, RKK), mul(uO, add(QuO, ROK)));
-    Fn[9] = weigh(w, fma(uK, U9, fma(add(u2, u2), gK, fma(uQR, S(4.0f), SK))), U9);
+    float d9;
+    if (RUS)
+        d9 = djump(u2, du2, e2, fmaf(2.0f, D[3] + D[5] + D[6], dru2)) +
+             fmaf(4.0f, djump(ux, D[1], Pqx, dPx + D[7]) + djump(uy, D[2], Pqy, dPy + D[8]), D[9]);
+    else
+        d9 = jump(U9);
+    Fn[9] = weigh(w, fma(uK, U9, fma(add(u2, u2), gK, fma(uQR, S(4.0f), SK))), d9);
 }
 
 }  // namespace x2

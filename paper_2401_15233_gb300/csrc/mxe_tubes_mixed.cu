@@ -170,7 +170,7 @@ struct TubeView {
 //   !final:  Wout = prim(cons(W_own) + dU)  with W_own the stencil's cell
 //   final:   U += dU (FP64);  Wout = prim(U) by increment from Wbase (or in
 //            FP64 from the new U when `resync`);  returns the CFL rate max.
-template <class PH, int NT>
+template <class PH, int NT, bool RUS>
 __device__ float tube_stage_m(const TubeMixedArgs& a, const TubeView& v, const MixedPolicy& mp,
                               const float* Win, const float* Wbase, float* Wout, float cdt,
                               bool final, bool resync, unsigned rank, unsigned team, float* sm,
@@ -200,7 +200,7 @@ __device__ float tube_stage_m(const TubeMixedArgs& a, const TubeView& v, const M
         if (tid <= C) {                  // C + 1 faces
             float F[NF];
             if constexpr (NF == NP) {
-                face_flux_x2<0, BOX>(Wb, tid + 1, 1, ph[tid], ph[tid + 1], p, mp, a.sl64,
+                face_flux_x2<PH, 0, BOX, RUS>(Wb, tid + 1, 1, ph[tid], ph[tid + 1], p, mp, a.sl64,
                                      a.kw64, F, nflag);
             } else {
                 face_flux_1d<PH, NT, BOX>(Wb, tid + 1, ph[tid], ph[tid + 1], p, mp, a.sl64,
@@ -375,7 +375,7 @@ __device__ __forceinline__ bool team_reduce_grid(TubeSync* s, float r, unsigned 
 // threads; the same kernel, so that the stage is the same code and its result
 // the same to the bit); otherwise a cluster is a team and takes tubes from
 // the queue.
-template <class PH, int NT>
+template <class PH, int NT, bool RUS>
 __device__ void tubes_mixed_body(const TubeMixedArgs& a, const ParamsT<float>& p0,
                                  const MixedPolicy& mp) {
     constexpr int NF = PH::NF;
@@ -483,18 +483,18 @@ __device__ void tubes_mixed_body(const TubeMixedArgs& a, const ParamsT<float>& p
             unsigned status = 0;
             float rr;
             if (a.integrator == 1) {
-                tube_stage_m<PH, NT>(a, v, mp, Wc, nullptr, Wn, (float)(0.5 * dt), false, false,
+                tube_stage_m<PH, NT, RUS>(a, v, mp, Wc, nullptr, Wn, (float)(0.5 * dt), false, false,
                                      rank, team, sm, status, nflag);
                 if (grid) {
                     if (!(ok = team_barrier(sy, team, target))) break;
                 } else {
                     cl_sync();
                 }
-                rr = tube_stage_m<PH, NT>(a, v, mp, Wn, Wc, Wc, (float)dt, true, rs, rank, team,
+                rr = tube_stage_m<PH, NT, RUS>(a, v, mp, Wn, Wc, Wc, (float)dt, true, rs, rank, team,
                                           sm, status, nflag);
                 nface += 2u;
             } else {
-                rr = tube_stage_m<PH, NT>(a, v, mp, Wc, nullptr, Wn, (float)dt, true, rs, rank,
+                rr = tube_stage_m<PH, NT, RUS>(a, v, mp, Wc, nullptr, Wn, (float)dt, true, rs, rank,
                                           team, sm, status, nflag);
                 float* tmp = Wc;
                 Wc = Wn;
@@ -529,15 +529,17 @@ __device__ void tubes_mixed_body(const TubeMixedArgs& a, const ParamsT<float>& p
     }
 }
 
-#define MXE_TUBES_MIXED(NAME, PH, NT, MINB)                                                  \
+#define MXE_TUBES_MIXED(NAME, PH, NT, MINB, RUS)                                             \
     extern "C" __global__ void __launch_bounds__(NT, MINB)                                   \
         NAME(const TubeMixedArgs a, const ParamsT<float> p, const MixedPolicy mp) {          \
-        tubes_mixed_body<PH, NT>(a, p, mp);                                                  \
+        tubes_mixed_body<PH, NT, RUS>(a, p, mp);                                             \
     }
-MXE_TUBES_MIXED(mxe_tubes14_mixed_128, PhysGeneral, 128, 4)
-MXE_TUBES_MIXED(mxe_tubes14_mixed_256, PhysGeneral, 256, 2)
-MXE_TUBES_MIXED(mxe_tubes14_mixed_planar_128, PhysPlanar, 128, 4)
-MXE_TUBES_MIXED(mxe_tubes14_mixed_planar_256, PhysPlanar, 256, 2)
+MXE_TUBES_MIXED(mxe_tubes14_mixed_128, PhysGeneral, 128, 4, false)   // both fluxes
+MXE_TUBES_MIXED(mxe_tubes14_mixed_256, PhysGeneral, 256, 2, false)   // both fluxes
+MXE_TUBES_MIXED(mxe_tubes14_mixed_planar_128, PhysPlanar, 128, 4, false)
+MXE_TUBES_MIXED(mxe_tubes14_mixed_planar_128_rus, PhysPlanar, 128, 4, true)
+MXE_TUBES_MIXED(mxe_tubes14_mixed_planar_256, PhysPlanar, 256, 2, false)
+MXE_TUBES_MIXED(mxe_tubes14_mixed_planar_256_rus, PhysPlanar, 256, 2, true)
 #undef MXE_TUBES_MIXED
 
 // CFL rate max_cells |lambda|_max / dx of every tube's current state (one
@@ -593,7 +595,10 @@ void tube_rates(bool planar, const double* U, const TubeDesc* tubes, int ntubes,
 }
 
 // Kernel and dynamic shared memory of one block shape (nt = 128 or 256).
-const void* tubes_mixed_kernel(bool planar, int nt) {
+const void* tubes_mixed_kernel(bool planar, int nt, bool rus) {
+    if (planar && rus)
+        return nt == 256 ? (const void*)mxe_tubes14_mixed_planar_256_rus
+                         : (const void*)mxe_tubes14_mixed_planar_128_rus;
     if (planar) return nt == 256 ? (const void*)mxe_tubes14_mixed_planar_256
                                  : (const void*)mxe_tubes14_mixed_planar_128;
     return nt == 256 ? (const void*)mxe_tubes14_mixed_256 : (const void*)mxe_tubes14_mixed_128;

@@ -107,26 +107,6 @@ __device__ __forceinline__ float phi_box_m(const float* W, int c, int stride, in
     return phi;
 }
 
-// Shared limiter of box cell c in x (result .x) and y (.y): the stencil
-// centre and the flat-test reference are loaded once for both directions.
-template <int NF, int NBOX, int BX>
-__device__ __forceinline__ float2 phi_pair_m(const float* W, int c, int lim) {
-    using namespace x2;
-    const FlatRef<float> fr = flat_ref<NF>(W + c, NBOX);
-    float nx = 1.0f, xx = 1.0f, ny = 1.0f, xy = 1.0f;
-#pragma unroll
-    for (int k = 0; k < NF; ++k) {
-        const float* w = W + k * NBOX + c;
-        const float w0 = w[0];
-        // the x and y differences as the lanes of packed subtractions
-        const v2 dm = sub(S(w0), make_float2(w[-1], w[-BX]));
-        const v2 dp = sub(make_float2(w[1], w[BX]), S(w0));
-        phi_ratio_step<NF>(dm.x, dp.x, w0, fr, k, nx, xx);
-        phi_ratio_step<NF>(dm.y, dp.y, w0, fr, k, ny, xy);
-    }
-    return make_float2(phi_of_ratio(nx, xx, lim), phi_of_ratio(ny, xy, lim));
-}
-
 template <int NF>
 __device__ __forceinline__ void face_prims_m(const float* W, int c, int stride, float phi,
                                              float hs, float* Qf) {
@@ -364,7 +344,7 @@ __device__ __forceinline__ void stage_mixed(const Stage2DArgs& a, const ParamsT<
 #pragma unroll
         for (int k = 0; k < NF; ++k) Qc[k] = W[k * NBOXm + (cy + 2) * BXm + cx + 2];
         if (p.tau_model != 0 && !p.src_implicit) {
-            PH::source(Qc, PH::tau(p, Qc), L);
+            PH::source(Qc, p, L);
         } else {
 #pragma unroll
             for (int k = 0; k < NF; ++k) L[k] = 0.0f;
@@ -689,7 +669,7 @@ __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const Param
 #pragma unroll
         for (int k = 0; k < NF; ++k) Qc[k] = W[k * G::NBOX + cb];
         if (p.tau_model != 0 && !p.src_implicit) {
-            PH::source(Qc, PH::tau(p, Qc), L);
+            PH::source(Qc, p, L);
         } else {
 #pragma unroll
             for (int k = 0; k < NF; ++k) L[k] = 0.0f;

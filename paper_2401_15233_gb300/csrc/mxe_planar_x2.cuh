@@ -12,6 +12,7 @@
 // 14mom-approx-ws-equations), regrouped into fused multiply-adds; the
 // results agree with the scalar FP32 path to FP32 rounding.
 #pragma once
+#include "mxe_fast64.cuh"
 #include "mxe_planar.cuh"
 
 namespace mxe {
@@ -35,7 +36,7 @@ __device__ __forceinline__ v2 ex2(v2 a) { return make_float2(exp2f(a.x), exp2f(a
 __device__ __forceinline__ v2 lg2(v2 a) { return make_float2(__log2f(a.x), __log2f(a.y)); }
 __device__ __forceinline__ v2 abs_(v2 a) { return make_float2(fabsf(a.x), fabsf(a.y)); }
 __device__ __forceinline__ v2 div_(v2 a, v2 b) {
-    return make_float2(__fdividef(a.x, b.x), __fdividef(a.y, b.y));
+    return make_float2(a.x * f64::rcp32(b.x), a.y * f64::rcp32(b.y));
 }
 
 constexpr float LOG2E = 1.4426950408889634f;
@@ -94,7 +95,7 @@ __device__ __forceinline__ v2 clamp_sigma_x2(v2 s, float slim) {
 // D0 / (sqrt(D) - zeta) for zeta < 0, where a clamped discriminant makes the
 // quotient smaller than zeta, the value it stands for.
 __device__ __forceinline__ float hyp1(float z, float D0, float s) {
-    const float q = fmaxf(__fdividef(D0, s), z);
+    const float q = fmaxf(D0 * f64::rcp32(s), z);
     return z >= 0.0f ? s : q;
 }
 __device__ __forceinline__ v2 hyp_x2(v2 z, v2 D0) {

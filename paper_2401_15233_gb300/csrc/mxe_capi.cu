@@ -291,7 +291,7 @@ static mxe_status alloc_common(mxe_ctx* c) {
 //     steps x passes, is the longest (steps: equal, or proportional to 1/dx
 //     when the tubes march to a common time);
 //   * with more tubes than slots every tube has one CTA and nothing waits.
-// Mixed tubes have one chunk size (126).
+// Mixed CTAs have one size, four warps of 30 cells.
 // Measured on GB300 (152 SMs), per step, one CTA a tube before / teams now:
 //   5 moments, 1000 cells, first order Euler          288   ->  18.5 us
 //   14 moments, 4096 cells, MUSCL RK2, planar        8350   ->  64.7 us
@@ -352,7 +352,7 @@ static mxe_status team_plans(mxe_ctx* c) {
     if (c->mixed && c->ntubes > nsm) return MXE_OK;      // one CTA a tube fills the chip
     for (int k = 0; k < 2; ++k) {
         std::vector<TubeTeam> t;
-        team_plan(c, k == 1, per * nsm, c->mixed ? 126 : 31, c->mixed ? 126 : 63, t,
+        team_plan(c, k == 1, per * nsm, c->mixed ? 120 : 31, c->mixed ? 120 : 63, t,
                   &c->team_chunk[k], &c->team_coop[k]);
         c->team_ctas[k] = (int)t.size();
         CK(cudaMalloc(&c->team_d[k], sizeof(TubeTeam) * t.size()));
@@ -1144,7 +1144,7 @@ static void tube_fill_split(const mxe_ctx* c, TubeLaunch* L, const std::vector<d
         cells[q] = c->tdesc[c->order_h[q]].n;
         steps[q] = (*est)[c->order_h[q]];
     }
-    const int nA = plan_fill(n, cells.data(), steps.data(), L->nt - 2, L->cl, L->teams, L->fill,
+    const int nA = plan_fill(n, cells.data(), steps.data(), L->nt / 32 * 30, L->cl, L->teams, L->fill,
                              nullptr);
     L->nA = nA;
     L->fill = nA < n ? std::min(L->fill, n - nA) : 0;

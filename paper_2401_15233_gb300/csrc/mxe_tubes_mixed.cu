@@ -12,12 +12,15 @@
 // (a thread-block cluster of 1..8 CTAs) takes one tube at a time from a
 // device work queue whose order is longest-expected-work first, and marches
 // it to t_end on the tube's own clock.  Within a stage the team splits the
-// tube into chunks of NT-2 cells (chunk j belongs to CTA j mod team); a CTA
-// stages a chunk's primitives plus a 2-cell halo in shared memory, forms one
-// shared limiter per cell (NT of them: one per thread), evaluates one face
-// per thread (planar states: both face states as one packed FP32 pair) and
-// updates its cells.  Cluster barriers separate the stages; the team's CFL maximum and
-// status bits are combined in the shared memory of CTA 0 of the cluster
+// tube into chunks of 30 cells, one a warp at a time (chunk j belongs to CTA j
+// mod team); a warp stages a chunk's primitives plus a 2-cell halo in its own
+// shared memory, forms one shared limiter per cell (32 of them: one per
+// lane), evaluates one face per lane (planar states: both face states as one
+// packed FP32 pair) and updates its cells.  No block barrier stands inside a
+// stage: warps drift apart and hide one another's loads and arithmetic, which pays for
+// the 7 % of halo work that a chunk of 30 has over one of 254 (256 tubes of
+// 512 to 8192 cells, teams of 8 CTAs of 256 threads: 137 -> 131 us an RK2 step).
+// Cluster barriers separate the stages; the team's CFL maximum and status bits are combined in the shared memory of CTA 0 of the cluster
 // (distributed shared memory).
 //
 // While the block shape is left to the library and the tubes are few, a tube's
@@ -69,17 +72,21 @@ __device__ __forceinline__ unsigned cl_ld(unsigned addr) {
     return v;
 }
 
-// ---- shared-memory layout of one CTA -------------------------------------
+// ---- shared memory of one warp, and of the CTA's reductions --------------
+// A warp advances a chunk of C cells on its own: its lanes hold the C + 2
+// limiters, the C + 1 faces and the C cells.
+constexpr int TC = 30;
 template <int NF, int NT>
 struct TubeLayout {
-    static constexpr int C = NT - 2;              // cells per chunk (C + 2 limiters)
+    static constexpr int C = TC;
     static constexpr int BOX = C + 4;             // staged cells (chunk + 2 + 2)
-    static constexpr int FS = 2 * NF + 2;         // staged left face state
+    static constexpr int FS = NF == NP ? 0 : 2 * NF + 2;   // staged left face state (scalar faces)
     static constexpr int W_OFF = 0;               // [NF][BOX] primitives
-    static constexpr int F_OFF = W_OFF + NF * BOX;   // [NF][NT] face fluxes
-    static constexpr int L_OFF = F_OFF + NF * NT;    // [FS][NT] left face states
-    static constexpr int P_OFF = L_OFF + FS * NT;    // [C+2] limiters
-    static constexpr int R_OFF = P_OFF + C + 2;      // [NT/32] reduction scratch (rate)
+    static constexpr int F_OFF = W_OFF + NF * BOX;   // [NF][32] face fluxes
+    static constexpr int L_OFF = F_OFF + NF * 32;    // [FS][32] left face states
+    static constexpr int P_OFF = L_OFF + FS * 32;    // [32] limiters
+    static constexpr int WARP = P_OFF + 32;
+    static constexpr int R_OFF = WARP * (NT / 32);   // [NT/32] reduction scratch (rate)
     static constexpr int S_OFF = R_OFF + NT / 32;    // [NT/32] reduction scratch (status)
     static constexpr int TOTAL = S_OFF + NT / 32;
     static constexpr size_t bytes() { return sizeof(float) * TOTAL; }
@@ -105,9 +112,9 @@ __device__ __forceinline__ void load_w(const TubeMixedArgs& a, const float* Wt, 
     for (int k = 0; k < PH::NF; ++k) Q[k] = __ldcg(Wt + (long long)k * n + gi);
 }
 
-// Face flux of the face between box cells cl = tid+1 and cr = tid+2; the
-// left face state is staged in this thread's column of Ls.
-template <class PH, int NT, int BOX>
+// Face flux of the face between box cells cl and cl + 1; the left face state
+// is staged in this lane's column of Ls.
+template <class PH, int BOX>
 __device__ __forceinline__ void face_flux_1d(const float* W, int cl, float phl, float phr,
                                              const ParamsT<float>& p, const MixedPolicy& mp,
                                              double sl64, double kw64, float* Ls, float* F,
@@ -123,26 +130,26 @@ __device__ __forceinline__ void face_flux_1d(const float* W, int cl, float phl, 
     }
     nflag += face_state_m<PH, 0>(Qf, p, mp, sl64, kw64, Lv) ? 1u : 0u;
 #pragma unroll
-    for (int n = 0; n < FS; ++n) Ls[n * NT] = Lv[n];
+    for (int n = 0; n < FS; ++n) Ls[n * 32] = Lv[n];
 #pragma unroll
     for (int k = 0; k < NF; ++k) {
         const float* w = W + k * BOX + cr;
         Qf[k] = w[0] - (0.5f * phr) * (0.5f * (w[1] - w[-1]));
     }
     nflag += face_state_m<PH, 0>(Qf, p, mp, sl64, kw64, R) ? 1u : 0u;
-    float lminL = Ls[(2 * NF) * NT], lmaxL = Ls[(2 * NF + 1) * NT];
+    float lminL = Ls[(2 * NF) * 32], lmaxL = Ls[(2 * NF + 1) * 32];
     float lminR = R[2 * NF], lmaxR = R[2 * NF + 1];
     if (p.flux == 1) {
         float s = fmaxf(fmaxf(fabsf(lminL), fabsf(lmaxL)), fmaxf(fabsf(lminR), fabsf(lmaxR)));
 #pragma unroll
         for (int k = 0; k < NF; ++k)
-            F[k] = 0.5f * (Ls[(NF + k) * NT] + R[NF + k]) - 0.5f * s * (R[k] - Ls[k * NT]);
+            F[k] = 0.5f * (Ls[(NF + k) * 32] + R[NF + k]) - 0.5f * s * (R[k] - Ls[k * 32]);
         return;
     }
     float SL = fminf(lminL, lminR), SR = fmaxf(lmaxL, lmaxR);
     if (SL >= 0.0f) {
 #pragma unroll
-        for (int k = 0; k < NF; ++k) F[k] = Ls[(NF + k) * NT];
+        for (int k = 0; k < NF; ++k) F[k] = Ls[(NF + k) * 32];
     } else if (SR <= 0.0f) {
 #pragma unroll
         for (int k = 0; k < NF; ++k) F[k] = R[NF + k];
@@ -151,7 +158,7 @@ __device__ __forceinline__ void face_flux_1d(const float* W, int cl, float phl, 
         float cl_ = SR * inv, cr_ = -SL * inv, cu = SL * SR * inv;
 #pragma unroll
         for (int k = 0; k < NF; ++k)
-            F[k] = cl_ * Ls[(NF + k) * NT] + cr_ * R[NF + k] + cu * (R[k] - Ls[k * NT]);
+            F[k] = cl_ * Ls[(NF + k) * 32] + cr_ * R[NF + k] + cu * (R[k] - Ls[k * 32]);
     }
 }
 
@@ -165,7 +172,7 @@ struct TubeView {
     ParamsT<float> p;           // scheme + this tube's relaxation
 };
 
-// One stage over the chunks this CTA owns:
+// One stage over the chunks this warp owns (chunk j: CTA j mod team, then warp):
 //   L = L(Win);  dU = cdt L
 //   !final:  Wout = prim(cons(W_own) + dU)  with W_own the stencil's cell
 //   final:   U += dU (FP64);  Wout = prim(U) by increment from Wbase (or in
@@ -178,43 +185,43 @@ __device__ float tube_stage_m(const TubeMixedArgs& a, const TubeView& v, const M
     constexpr int NF = PH::NF;
     using LY = TubeLayout<NF, NT>;
     constexpr int C = LY::C, BOX = LY::BOX;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    sm += wid * LY::WARP;
     float* Wb = sm + LY::W_OFF;
     float* Fb = sm + LY::F_OFF;
     float* Ls = sm + LY::L_OFF;
     float* ph = sm + LY::P_OFF;
-    const int tid = threadIdx.x;
     const int n = v.n;
     const ParamsT<float>& p = v.p;
     float rmax = 0.0f;
-    for (int c0 = (int)rank * C; c0 < n; c0 += (int)team * C) {
-        for (int i = tid; i < BOX; i += NT) {
+    for (int c0 = (wid * (int)team + (int)rank) * C; c0 < n; c0 += (int)team * (NT / 32) * C) {
+        for (int i = lane; i < BOX; i += 32) {
             float Q[NF];
             load_w<PH>(a, Win, n, c0 - 2 + i, Q);
 #pragma unroll
             for (int k = 0; k < NF; ++k) Wb[k * BOX + i] = Q[k];
         }
-        __syncthreads();
-        for (int i = tid; i < C + 2; i += NT)
-            ph[i] = p.order == 2 ? phi_one_m<NF, BOX>(Wb, i + 1, 1, p.limiter) : 0.0f;
-        __syncthreads();
-        if (tid <= C) {                  // C + 1 faces
+        __syncwarp();
+        ph[lane] = p.order == 2 ? phi_one_m<NF, BOX>(Wb, lane + 1, 1, p.limiter) : 0.0f;
+        __syncwarp();
+        if (lane <= C) {                 // C + 1 faces
             float F[NF];
             if constexpr (NF == NP) {
-                face_flux_x2<PH, 0, BOX, RUS>(Wb, tid + 1, 1, ph[tid], ph[tid + 1], p, mp, a.sl64,
-                                     a.kw64, F, nflag);
+                face_flux_x2<PH, 0, BOX, RUS>(Wb, lane + 1, 1, ph[lane], ph[lane + 1], p, mp,
+                                              a.sl64, a.kw64, F, nflag);
             } else {
-                face_flux_1d<PH, NT, BOX>(Wb, tid + 1, ph[tid], ph[tid + 1], p, mp, a.sl64,
-                                          a.kw64, Ls + tid, F, nflag);
+                face_flux_1d<PH, BOX>(Wb, lane + 1, ph[lane], ph[lane + 1], p, mp, a.sl64,
+                                      a.kw64, Ls + lane, F, nflag);
             }
 #pragma unroll
-            for (int k = 0; k < NF; ++k) Fb[k * NT + tid] = F[k];
+            for (int k = 0; k < NF; ++k) Fb[k * 32 + lane] = F[k];
         }
-        __syncthreads();
-        const int i = c0 + tid;
-        if (tid < C && i < n) {
+        __syncwarp();
+        const int i = c0 + lane;
+        if (lane < C && i < n) {
             float Qc[NF], L[NF];
 #pragma unroll
-            for (int k = 0; k < NF; ++k) Qc[k] = Wb[k * BOX + tid + 2];
+            for (int k = 0; k < NF; ++k) Qc[k] = Wb[k * BOX + lane + 2];
             const bool implicit = p.tau_model != 0 && p.src_implicit;
             if (p.tau_model != 0 && !implicit) {
                 PH::source(Qc, p, L);
@@ -225,7 +232,7 @@ __device__ float tube_stage_m(const TubeMixedArgs& a, const TubeView& v, const M
             float dU[NF], Wn[NF];
 #pragma unroll
             for (int k = 0; k < NF; ++k) {
-                L[k] -= (Fb[k * NT + tid + 1] - Fb[k * NT + tid]) * v.idx;
+                L[k] -= (Fb[k * 32 + lane + 1] - Fb[k * 32 + lane]) * v.idx;
                 dU[k] = cdt * L[k];
             }
             if (!final) {
@@ -274,7 +281,7 @@ __device__ float tube_stage_m(const TubeMixedArgs& a, const TubeView& v, const M
 #pragma unroll
             for (int k = 0; k < NF; ++k) Wout[(long long)k * n + i] = Wn[k];
         }
-        __syncthreads();
+        __syncwarp();
     }
     return rmax;
 }
@@ -441,9 +448,10 @@ __device__ void tubes_mixed_body(const TubeMixedArgs& a, const ParamsT<float>& p
 
         // W = prim(U) in FP64, and the CFL rate of the current state
         float r = 0.0f;
-        for (int c0 = (int)rank * C; c0 < n; c0 += (int)team * C) {
-            const int i = c0 + tid;
-            if (tid < C && i < n) {
+        for (int c0 = ((tid >> 5) * (int)team + (int)rank) * C; c0 < n;
+             c0 += (int)team * (NT / 32) * C) {
+            const int i = c0 + (tid & 31);
+            if ((tid & 31) < C && i < n) {
                 double Uc[NF], Q[NF];
 #pragma unroll
                 for (int k = 0; k < NF; ++k) Uc[k] = v.U[(long long)PH::ufield(k) * n + i];
@@ -514,7 +522,7 @@ __device__ void tubes_mixed_body(const TubeMixedArgs& a, const ParamsT<float>& p
         __syncthreads();
         if (tid == 0) {
             unsigned nch = 0;
-            for (int c0 = (int)rank * C; c0 < n; c0 += (int)team * C) ++nch;
+            for (int j = (int)rank; j * C < n; j += (int)team) ++nch;
             atomicAdd(&ck->n_face, (unsigned long long)nface * nch * 2ull * (C + 1));
             if (s_cnt) atomicAdd(&ck->n_face64, (unsigned long long)s_cnt);
             if (!ok) atomicOr(&ck->status, ST_TIMEOUT);

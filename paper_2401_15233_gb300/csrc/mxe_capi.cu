@@ -67,7 +67,8 @@ extern "C" __global__ void mxe_k_validate(CellMap m, int nf, int kind, const dou
                                           unsigned long long* bad, unsigned* nonplanar,
                                           double* copy);
 extern "C" __global__ void mxe_k_setstate(CellMap m, int nf, int kind, const double* src,
-                                          double* U);
+                                          double* U,
+                                          float* W, int planar);
 extern "C" __global__ void mxe_k_getstate(CellMap m, int nf, int kind, const double* U,
                                           double* dst);
 extern "C" __global__ void mxe_k_ghost(int nf, int n, const double* in, double* out);
@@ -624,7 +625,8 @@ static void launch_resync(mxe_ctx* c, bool planar) {
 }
 
 // ---------------------------------------------------------------- clocks
-static mxe_status reset_clock(mxe_ctx* c) {
+// w_set: W already holds the state's primitives
+static mxe_status reset_clock(mxe_ctx* c, bool w_set) {
     if (c->tubes) {
         std::vector<TubeClock> z(c->ntubes);
         memset(z.data(), 0, sizeof(TubeClock) * c->ntubes);
@@ -640,7 +642,7 @@ static mxe_status reset_clock(mxe_ctx* c) {
     dim3 grid((c->g.nx + nt - 1) / nt, c->g.ny);
     bool pl = use_planar(c);
     if (c->mixed) {
-        launch_resync(c, pl);
+        if (!w_set) launch_resync(c, pl);
         if (pl)
             mxe_rate14_2d_mixed_planar<<<grid, nt, 0, c->stream>>>(c->W, c->g, fparams(c),
                                                                    (float)c->g.idx, (float)c->g.idy,
@@ -710,11 +712,16 @@ extern "C" mxe_status mxe_set_state(mxe_ctx* c, int kind, const double* soa, int
         return fail(c, code == 1 ? MXE_ENONFINITE : MXE_EUNREALIZABLE,
                     "input cell %llu: %s", idx, why);
     }
-    mxe_k_setstate<<<grid, 128, 0, c->stream>>>(m, c->nf, kind, src, c->U);
-    CK(cudaGetLastError());
     c->state_planar = (res[1] == 0ull);
+    const bool pl = c->tubes ? c->state_planar : use_planar(c);
+    // a mixed grid given its primitives keeps them as W
+    const bool w_set = c->mixed && !c->tubes && kind == MXE_PRIMITIVE;
+    mxe_k_setstate<<<grid, 128, 0, c->stream>>>(m, c->nf, kind, src, c->U, w_set ? c->W : nullptr,
+                                                pl);
+    CK(cudaGetLastError());
+    if (w_set) c->w_planar = pl;
     if (!c->tubes && c->Us) CK(cudaMemsetAsync(c->Us, 0, sizeof(double) * c->nelem, c->stream));
-    mxe_status s = reset_clock(c);
+    mxe_status s = reset_clock(c, w_set);
     if (s != MXE_OK) return s;
     c->have_state = true;
     return MXE_OK;

@@ -1,7 +1,9 @@
 // mxe_util.cu -- set-up and read-back kernels: primitive <-> conserved
 // conversion, state validation, ghost-state round trip, diagnostics.
 // Nothing here is on the time-stepping path.
+#include "mxe_fast64.cuh"
 #include "mxe_internal.h"
+#include "mxe_planar.cuh"
 
 namespace mxe {
 
@@ -40,50 +42,47 @@ __device__ __forceinline__ double raw_sigma(const double* Q, int nf) {
     return d.sig;
 }
 
-// sigma <= 1 (with 1e-9 of slack): decided in FP32 where FP32 clearly can
-// (sigma_32 <= 0.99 with every |Q| in [1e-30, 1e30] and det P* >= 1e-3, so
-// that the FP32 error of sigma is orders of magnitude below the 1e-2
-// margin), in FP64 otherwise.  FP64 here runs at 1/64 of the FP32 rate.
-__device__ __forceinline__ bool sigma_within_one(const double* Q, int nf) {
+// A state that is realizable by a clear margin, decided without the FP64 pipe
+// (2 operations a clock and SM here, against 128 in FP32): every |Q| 0 or
+// in [1e-30, 1e30], and in FP32 sigma <= 0.99 and, of P* = 3 P / tr P, the
+// diagonal element > 0, the leading minor > 1e-4 and det >= 1e-3 (a positive
+// definite P* of that determinant has a leading minor of at least det / 3; the FP32
+// errors are orders of magnitude below these margins).
+__device__ __forceinline__ bool clearly_realizable(const double* Q, int nf) {
     bool screen = true;
     float Qf[14];
     for (int k = 0; k < nf; ++k) {
-        double a = fabs(Q[k]);
-        screen &= (a == 0.0) || (a >= 1e-30 && a <= 1e30);
-        Qf[k] = (float)Q[k];
+        const unsigned e = (f64::hi32(Q[k]) >> 20) & 0x7ffu;
+        const bool zero = ((f64::hi32(Q[k]) & 0x7fffffffu) | f64::lo32(Q[k])) == 0u;
+        screen &= zero || (e >= 924u && e <= 1122u);         // 2^-99 .. 2^99
+        Qf[k] = f64::narrow(Q[k]);
     }
-    if (screen) {
-        float s32;
-        bool cond = true;
-        if (nf == 5) {
-            float th = Qf[2] / Qf[0];
-            s32 = sigma5(Qf[3] / (Qf[0] * th * sqrtf(th)), Qf[4] / (Qf[0] * th * th));
-        } else {
-            Dimless14<float> d;
-            dimless14(Qf, d);
-            s32 = d.sig;
-            cond = d.det >= 1e-3f;
-        }
-        if (cond && s32 <= 0.99f) return true;     // NaN falls through to FP64
+    if (!screen) return false;
+    if (nf == 5) {
+        const float th = Qf[2] / Qf[0];
+        return sigma5(Qf[3] / (Qf[0] * th * sqrtf(th)), Qf[4] / (Qf[0] * th * th)) <= 0.99f;
     }
-    return raw_sigma(Q, nf) <= 1.0 + 1e-9;
+    Dimless14<float> d;
+    dimless14(Qf, d);
+    return d.th > 0.0f && d.Ps[0] > 0.0f && d.Ps[0] * d.Ps[3] - d.Ps[1] * d.Ps[1] > 1e-4f && d.det >= 1e-3f &&
+           d.sig <= 0.99f;                                    // false for NaN
 }
 
 // 0 ok; 1 non-finite; 2 rho <= 0 or P not positive definite; 3 sigma > 1
+// (with 1e-9 of slack)
 __device__ __forceinline__ int check_prim(const double* Q, int nf) {
     for (int k = 0; k < nf; ++k)
-        if (!isfinite(Q[k])) return 1;
-    if (!(Q[0] > 0.0)) return 2;
-    if (nf == 5) {
-        if (!(Q[2] > 0.0)) return 2;
-    } else {
+        if (!f64::is_finite(Q[k])) return 1;
+    if (f64::le0(Q[0])) return 2;
+    if (nf == 5 && f64::le0(Q[2])) return 2;
+    if (clearly_realizable(Q, nf)) return 0;
+    if (nf == 14) {
         double a = Q[4], b = Q[5], c = Q[6], d = Q[7], e = Q[8], f = Q[9];
         double m2 = a * d - b * b;
         double det = a * (d * f - e * e) - b * (b * f - e * c) + c * (b * e - d * c);
         if (!(a > 0.0) || !(m2 > 0.0) || !(det > 0.0)) return 2;
     }
-    if (!sigma_within_one(Q, nf)) return 3;
-    return 0;
+    return raw_sigma(Q, nf) <= 1.0 + 1e-9 ? 0 : 3;
 }
 
 __device__ __forceinline__ void to_prim(const double* U, double* Q, int nf) {
@@ -122,7 +121,12 @@ __device__ __forceinline__ void validate_body(const CellMap& m, int kind, const 
         if (code) atomicMin(bad, ((unsigned long long)idx << 2) | (unsigned long long)code);
         // planar iff the z-odd moments (u_z, P_xz, P_yz, q_z) vanish; on the
         // conserved side they are rho u_z, E_xz, E_yz, H_z (same positions)
-        if (NF == 14) np = V[3] != 0.0 || V[6] != 0.0 || V[8] != 0.0 || V[12] != 0.0;
+        if (NF == 14) {
+            auto zero = [](double x) {
+                return ((f64::hi32(x) & 0x7fffffffu) | f64::lo32(x)) == 0u;
+            };
+            np = !(zero(V[3]) && zero(V[6]) && zero(V[8]) && zero(V[12]));
+        }
     }
     // one atomic per warp that saw a non-planar cell (blocks are whole warps)
     if (__any_sync(0xffffffffu, np) && (threadIdx.x & 31) == 0) atomicOr(nonplanar, 1u);
@@ -137,28 +141,54 @@ extern "C" __global__ void mxe_k_validate(CellMap m, int nf, int kind, const dou
     else validate_body<14>(m, kind, src, bad, nonplanar, copy);
 }
 
+// planar: the state has no z-odd moments (ten fields are converted).  W (may
+// be null): FP32 primitives of a mixed grid, NF fields or (planar) ten.
+// FP64-pipe bound: 4096 x 4096 cells of 14 moments, primitive in: 1.37 ms + 1.75 ms
+// for W from the conserved state; in one pass with ten fields and W from the
+// given primitives the two and the check fit the memory traffic
+// better: 4096 x 4096 set-up 6.0 -> 3.0 ms in all.
 template <int NF>
 __device__ __forceinline__ void setstate_body(const CellMap& m, int kind, const double* src,
-                                              double* U) {
+                                              double* U, float* Wp, bool planar) {
     long long dense, dfs, dev, fs, idx;
     if (!cell_of(m, dense, dfs, dev, fs, idx)) return;
-    double V[NF], W[NF];
+    if constexpr (NF == 14) {
+        if (kind == 0 && planar) {
+            double Q[NP], C[NP];
+#pragma unroll
+            for (int k = 0; k < NP; ++k) Q[k] = src[dense + planar_field(k) * dfs];
+            prim2cons_p(Q, C);
+#pragma unroll
+            for (int k = 0; k < NP; ++k) {
+                U[dev + planar_field(k) * fs] = C[k];
+                if (Wp) Wp[dev + k * fs] = f64::to_f32(Q[k]);
+            }
+            const int odd[4] = {3, 6, 8, 12};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) U[dev + odd[k] * fs] = 0.0;
+            return;
+        }
+    }
+    double V[NF], C[NF];
 #pragma unroll
     for (int k = 0; k < NF; ++k) V[k] = src[dense + k * dfs];
     if (kind == 0) {
-        to_cons(V, W, NF);
+        to_cons(V, C, NF);
+#pragma unroll
+        for (int k = 0; k < NF; ++k)
+            if (Wp) Wp[dev + k * fs] = f64::to_f32(V[k]);
     } else {
 #pragma unroll
-        for (int k = 0; k < NF; ++k) W[k] = V[k];
+        for (int k = 0; k < NF; ++k) C[k] = V[k];
     }
 #pragma unroll
-    for (int k = 0; k < NF; ++k) U[dev + k * fs] = W[k];
+    for (int k = 0; k < NF; ++k) U[dev + k * fs] = C[k];
 }
 
 extern "C" __global__ void mxe_k_setstate(CellMap m, int nf, int kind, const double* src,
-                                          double* U) {
-    if (nf == 5) setstate_body<5>(m, kind, src, U);
-    else setstate_body<14>(m, kind, src, U);
+                                          double* U, float* W, int planar) {
+    if (nf == 5) setstate_body<5>(m, kind, src, U, nullptr, false);
+    else setstate_body<14>(m, kind, src, U, W, planar != 0);
 }
 
 // kind 0 primitive, 1 conserved, 2 raw sigma (one field)

@@ -123,6 +123,7 @@ struct mxe_ctx {
     bool g_planar = false, g_set = false;
     long long g_gen = -1;
     long long gen = 0;                // bumped whenever launch arguments change
+    long long known_steps = -1;       // steps on the device clock, where the host knows them (else -1)
     // dt history of 2D grids (steps counted from set_state)
     double* dth = nullptr;
     long long dth_cap = 0;
@@ -627,12 +628,9 @@ static void launch_resync(mxe_ctx* c, bool planar) {
 // ---------------------------------------------------------------- clocks
 // w_set: W already holds the state's primitives
 static mxe_status reset_clock(mxe_ctx* c, bool w_set) {
+    c->known_steps = 0;
     if (c->tubes) {
-        std::vector<TubeClock> z(c->ntubes);
-        memset(z.data(), 0, sizeof(TubeClock) * c->ntubes);
-        CK(cudaMemcpyAsync(c->tclk, z.data(), sizeof(TubeClock) * c->ntubes,
-                           cudaMemcpyHostToDevice, c->stream));
-        CK(cudaStreamSynchronize(c->stream));
+        CK(cudaMemsetAsync(c->tclk, 0, sizeof(TubeClock) * c->ntubes, c->stream));
         return MXE_OK;
     }
     CK(cudaMemsetAsync(c->clk, 0, sizeof(DevClock), c->stream));
@@ -930,6 +928,7 @@ static MixedTile mixed_tile(const mxe_ctx* c, bool pl) {
 // writes U* (default: the context's stage buffer).
 static mxe_status launch_2d_step(mxe_ctx* c, double t_end, double dt_fixed,
                                  double* ustar = nullptr, bool skip_rate = false) {
+    c->known_steps = -1;
     Stage2DArgs a{};
     a.skip_rate = skip_rate && !c->mixed;
     a.dt_hist = c->dth;
@@ -1341,6 +1340,7 @@ static mxe_status run_tubes_mixed(mxe_ctx* c, int max_steps, double t_end, const
 
 static mxe_status run_tubes(mxe_ctx* c, int max_steps, double t_end, const double* dts,
                             int ndts) {
+    c->known_steps = -1;
     if (c->mixed) return run_tubes_mixed(c, max_steps, t_end, dts, ndts);
     TubeArgs a{};
     a.U = c->U;
@@ -1402,8 +1402,8 @@ extern "C" mxe_status mxe_step(mxe_ctx* c, int max_steps, double t_end, double* 
     if (s != MXE_OK) return s;
     if (c->tubes) {
         if (!bc_planar(c)) c->state_planar = false;      // stays off until set_state
-        long long st0 = 0, st1 = 0;
-        if (steps_out) {
+        long long st0 = c->known_steps, st1 = 0;
+        if (steps_out && st0 < 0) {
             s = tube_status(c, nullptr, &st0);
             if (s != MXE_OK) return s;
         }
@@ -1414,14 +1414,15 @@ extern "C" mxe_status mxe_step(mxe_ctx* c, int max_steps, double t_end, double* 
             s = tube_status(c, &t, &st1);
             if (t_out) *t_out = t;
             if (steps_out) *steps_out = (int)(st1 - st0);
+            if (s == MXE_OK) c->known_steps = st1;
             return s;
         }
         return MXE_OK;
     }
     DevClock h{};
-    long long st0 = 0;
+    long long st0 = c->known_steps;
     bool want = t_out || steps_out;
-    if (want) {
+    if (want && st0 < 0) {
         s = read_clock_2d(c, &h);
         if (s != MXE_OK) return s;
         st0 = h.steps;
@@ -1470,6 +1471,7 @@ extern "C" mxe_status mxe_step(mxe_ctx* c, int max_steps, double t_end, double* 
                         "the CFL step size collapsed to zero at t = %g after %lld steps (a wave "
                         "speed is not finite)", h.t[c->slot], h.steps);
     }
+    if (want) c->known_steps = h.steps;
     return MXE_OK;
 }
 
@@ -1551,6 +1553,7 @@ extern "C" mxe_status mxe_batch_autotune(mxe_ctx* c, double t_probe, int* nt_out
     if (!c->tubes || !c->mixed) return fail(c, MXE_ESTATE, "autotuning needs an MXE_MIXED 1D context");
     if (!c->have_state) return fail(c, MXE_ESTATE, "no state set");
     if (!(t_probe > 0.0) || !std::isfinite(t_probe)) return fail(c, MXE_EINVAL, "t_probe must be > 0");
+    c->known_steps = -1;
     mxe_status s = periodic_ok(c);
     if (s != MXE_OK) return s;
     // save the state and the clocks; every candidate starts from them

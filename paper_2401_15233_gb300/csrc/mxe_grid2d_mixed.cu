@@ -535,23 +535,7 @@ __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const Param
         scdt = (float)(a.coef * sdt[0]);
         cnt = 0u;
     }
-    __syncthreads();
-    const double dt = sdt[0], t = sdt[1];
-    if (a.final_stage && blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) {
-        int s1 = (a.slot + 1) % 3, s2 = (a.slot + 2) % 3;
-        a.clk->rate[s2] = 0ull;
-        if (!(dt > 0.0)) {
-            a.clk->t[s1] = t;
-            a.clk->rate[s1] = a.clk->rate[a.slot];
-        } else {
-            a.clk->t[s1] = t + dt;
-            a.clk->last_dt = dt;
-            if (a.dt_hist && a.clk->steps < a.dt_hist_cap) a.dt_hist[a.clk->steps] = dt;
-            a.clk->steps += 1;
-        }
-    }
-    if (!(dt > 0.0)) return;
-
+    // the box is on its way before the step size is known
     const Grid2D& g = a.g;
     const int i0 = blockIdx.x * G::TX, j0 = blockIdx.y * G::TY;
     // final stage: the owned cells' U^n and W^n are needed only after the
@@ -589,6 +573,21 @@ __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const Param
     }
     asm volatile("cp.async.wait_group 0;\n" ::);
     __syncthreads();
+    const double dt = sdt[0], t = sdt[1];
+    if (a.final_stage && blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) {
+        int s1 = (a.slot + 1) % 3, s2 = (a.slot + 2) % 3;
+        a.clk->rate[s2] = 0ull;
+        if (!(dt > 0.0)) {
+            a.clk->t[s1] = t;
+            a.clk->rate[s1] = a.clk->rate[a.slot];
+        } else {
+            a.clk->t[s1] = t + dt;
+            a.clk->last_dt = dt;
+            if (a.dt_hist && a.clk->steps < a.dt_hist_cap) a.dt_hist[a.clk->steps] = dt;
+            a.clk->steps += 1;
+        }
+    }
+    if (!(dt > 0.0)) return;
     for (int n = tid; n < G::NLIM; n += G::NT) {
         if (n < G::NC) {                   // owned cell: both directions
             const int bx = 2 + n % G::TX, by = 2 + n / G::TX;
@@ -737,7 +736,7 @@ __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const Param
     unsigned wf = __reduce_add_sync(0xffffffffu, nflag);
     if ((tid & 31) == 0 && wf) atomicAdd(&cnt, wf);
     if (a.final_stage) block_max_atomic_m(r, &a.clk->rate[(a.slot + 1) % 3], red);
-    __syncthreads();
+    else __syncthreads();
     if (tid == 0) {
         atomicAdd(&a.clk->n_face, (unsigned long long)(2 * (G::NFX + G::NFY)));
         if (cnt) atomicAdd(&a.clk->n_face64, (unsigned long long)cnt);

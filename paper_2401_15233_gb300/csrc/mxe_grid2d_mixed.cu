@@ -473,12 +473,19 @@ struct TileGeo {
     static constexpr int NFY = TX * (TY + 1);      // y faces
     static constexpr int NPX = (TX + 2) * TY;      // x limiters
     static constexpr int NPY = TX * (TY + 2);      // y limiters
+    // work items of cells and y faces come in rows of RW, of which the last has
+    // none: a warp then reads whole rows of the box (or half-rows), without the
+    // bank conflicts and the divisions of rows of TX.  The items of TX + 1 x
+    // faces fill such rows.
+    static constexpr unsigned RW = TX + 1;
+    static_assert((RW & (RW - 1)) == 0 && RW <= 32, "a row is a part of a warp");
     // limiter work items: the owned cells (both directions), then the halo
     // columns (x only) and the halo rows (y only)
-    static constexpr int NLIM = NC + 2 * TY + 2 * TX;
+    static constexpr int NLC = TY * (TX + 1), NLIM = NLC + 2 * TY + 2 * TX;
+    static constexpr int NYI = (TY + 1) * (TX + 1);      // items of the y faces
     // y faces start on the warp after the last x face where all fit in one pass
     static constexpr int NFXW = (NFX + 31) / 32 * 32;
-    static constexpr int YOFF = NFXW + NFY <= NT ? NFXW : 0;
+    static constexpr int YOFF = NFXW + NYI <= NT ? NFXW : 0;
 };
 using TileP = TileGeo<31, 18, 320>;
 // General states: 14 fields of the box and of the fluxes fill 96 KB, and the
@@ -541,9 +548,9 @@ __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const Param
     // final stage: the owned cells' U^n and W^n are needed only after the
     // face fluxes; start moving them into L2 now
     if (a.final_stage) {
-        for (int c = tid; c < G::NC; c += G::NT) {
-            const int gi = i0 + c % G::TX, gj = j0 + c / G::TX;
-            if (gi < g.nx && gj < g.ny) {
+        for (int c = tid; c < G::NLC; c += G::NT) {
+            const int cx = c % G::RW, gi = i0 + cx, gj = j0 + c / G::RW;
+            if (cx < G::TX && gi < g.nx && gj < g.ny) {
                 const long long o = (long long)gj * g.pitch + gi;
 #pragma unroll
                 for (int k = 0; k < NF; ++k) {
@@ -589,20 +596,21 @@ __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const Param
     }
     if (!(dt > 0.0)) return;
     for (int n = tid; n < G::NLIM; n += G::NT) {
-        if (n < G::NC) {                   // owned cell: both directions
-            const int bx = 2 + n % G::TX, by = 2 + n / G::TX;
+        if (n < G::NLC) {                  // owned cell: both directions
+            const int bx = 2 + n % G::RW, by = 2 + n / G::RW;
+            if (bx >= 2 + G::TX) continue;
             float2 v = make_float2(0.0f, 0.0f);
             if (p.order == 2) v = phi_pair_m<NF, G::NBOX, G::BX>(W, by * G::BX + bx, p.limiter);
             phx[(by - 2) * (G::TX + 2) + bx - 1] = v.x;
             phy[(by - 1) * G::TX + bx - 2] = v.y;
-        } else if (n < G::NC + 2 * G::TY) {     // halo column: x only
-            const int m = n - G::NC;
+        } else if (n < G::NLC + 2 * G::TY) {    // halo column: x only
+            const int m = n - G::NLC;
             const int bx = (m < G::TY) ? 1 : G::TX + 2, by = 2 + m % G::TY;
             float v = 0.0f;
             if (p.order == 2) v = phi_one_m<NF, G::NBOX>(W, by * G::BX + bx, 1, p.limiter);
             phx[(by - 2) * (G::TX + 2) + bx - 1] = v;
         } else {                                // halo row: y only
-            const int m = n - G::NC - 2 * G::TY;
+            const int m = n - G::NLC - 2 * G::TY;
             const int by = (m < G::TX) ? 1 : G::TY + 2, bx = 2 + m % G::TX;
             float v = 0.0f;
             if (p.order == 2) v = phi_one_m<NF, G::NBOX>(W, by * G::BX + bx, G::BX, p.limiter);
@@ -623,9 +631,10 @@ __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const Param
         for (int k = 0; k < NF; ++k) Fx[k * G::NFX + f] = F[k];
     }
 #pragma unroll 1
-    for (int f = tid - G::YOFF; f < G::NFY; f += G::NT) {       // y faces: TY + 1 rows of TX
-        if (G::YOFF > 0 && f < 0) break;
-        const int fx = f % G::TX, fy = f / G::TX;
+    for (int n = tid - G::YOFF; n < G::NYI; n += G::NT) {       // y faces: TY + 1 rows of TX
+        const int fx = n % G::RW, fy = n / G::RW;
+        if (n < 0 || fx >= G::TX) continue;
+        const int f = fy * G::TX + fx;
         float F[NF];
         face_flux_x2<PH, 1, G::NBOX, RUS>(W, (fy + 1) * G::BX + fx + 2, G::BX, phy[fy * G::TX + fx],
                                  phy[(fy + 1) * G::TX + fx], p, mp, sl64, kw64, F, nflag);
@@ -647,10 +656,10 @@ __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const Param
     const float cdt = scdt;
     const bool implicit = p.tau_model != 0 && p.src_implicit;
 #pragma unroll 1
-    for (int c = tid; c < G::NC; c += G::NT) {
-        const int cx = c % G::TX, cy = c / G::TX;
+    for (int c = tid; c < G::NLC; c += G::NT) {
+        const int cx = c % G::RW, cy = c / G::RW;
         const int gi = i0 + cx, gj = j0 + cy;
-        if (gi >= g.nx || gj >= g.ny) continue;
+        if (cx >= G::TX || gi >= g.nx || gj >= g.ny) continue;
         const long long o = (long long)gj * g.pitch + gi;
         const int cb = (cy + 2) * G::BX + cx + 2;
         // final stage: this cell's W^n and U^n, loaded first so that their

@@ -251,7 +251,9 @@ const char *mxe_last_error(const mxe_ctx *ctx);
  * MXE_MIXED (14-moment system): teams of CTAs (thread-block clusters of
  * 1, 2, 4 or 8 CTAs of 128 or 256 threads, see mxe_batch_autotune) take
  * tubes from a device work queue, longest expected work (cells / dx) first;
- * each mxe_batch_run / mxe_step replays a cached CUDA graph of that launch.
+ * until a shape is chosen (mxe_batch_set_shape, mxe_batch_autotune), no more
+ * tubes than SMs have a team per tube as in MXE_FP64.  Each mxe_batch_run /
+ * mxe_step replays a cached CUDA graph of that launch.
  * Errors: MXE_EINVAL for a bad tube list (n < 1, ncells[b] < 4, length[b]
  * <= 0), MXE_ENOMEM / MXE_ECUDA when device allocation fails. */
 mxe_status mxe_batch_create(const mxe_config *cfg, int n, const int *ncells,

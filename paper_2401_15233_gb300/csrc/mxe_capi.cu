@@ -345,7 +345,8 @@ static mxe_status team_plans(mxe_ctx* c) {
         for (int ch : {31, 63}) {
             int v = 0;
             CK(c->mixed ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                              &v, tubes_mixed_kernel(pl, 128, c->sp.flux == MXE_FLUX_RUSANOV), 128, tubes_mixed_smem(pl, 128))
+                              &v, tubes_mixed_kernel(pl, 128, c->sp.flux == MXE_FLUX_RUSANOV), 128,
+                              tubes_mixed_smem(pl, 128))
                         : cudaOccupancyMaxActiveBlocksPerMultiprocessor(
                               &v, tubes_f64_kernel(c->nf, pl, ch), tubes_threads(), 0));
             per = std::min(per, v);

@@ -461,9 +461,10 @@ mxe_stage14_2d_mixed_planar_b3(const Stage2DArgs a, const ParamsT<float> p,
 //   31 x  7, 128 threads, 4 blocks, 128           3.81
 //   31 x  9, 160 threads, 4 blocks, 96            3.84
 //   31 x 11, 192 threads, 4 blocks, 80            4.21
-// 31 x 18 leaves no limiter for a third pass over the threads but 16 and fits
-// 1024 x 1024 in whole waves (3.45 ms and 243 us with the accurate CFL rates;
-// 261 us before).
+// 31 x 18 fits 1024 x 1024 in whole waves better (3.45 ms and 243 us there with
+// the accurate CFL rates; 3.79 ms and 261 us before).  With the limiter in
+// fewer instructions, the box asked for before the step size is known and the
+// items in rows of a warp: 3.00 ms and 216 us.
 template <int TX_, int TY_, int NT_>
 struct TileGeo {
     static constexpr int TX = TX_, TY = TY_, NT = NT_;

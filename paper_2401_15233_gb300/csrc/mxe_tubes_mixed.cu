@@ -17,18 +17,19 @@
 // shared memory, forms one shared limiter per cell (32 of them: one per
 // lane), evaluates one face per lane (planar states: both face states as one
 // packed FP32 pair) and updates its cells.  No block barrier stands inside a
-// stage: warps drift apart and hide one another's loads and arithmetic, which pays for
-// the 7 % of halo work that a chunk of 30 has over one of 254 (256 tubes of
-// 512 to 8192 cells, teams of 8 CTAs of 256 threads: 137 -> 131 us an RK2 step).
-// Cluster barriers separate the stages; the team's CFL maximum and status bits are combined in the shared memory of CTA 0 of the cluster
+// stage: warps drift apart and hide one another's loads and arithmetic, which
+// pays for the 7 % of halo work that a chunk of 30 has over one of 254 (256
+// tubes of 512 to 8192 cells, teams of 8 CTAs of 256 threads: 137 -> 131 us an
+// RK2 step).  Cluster barriers separate the stages; the team's CFL maximum and
+// status bits are combined in the shared memory of CTA 0 of the cluster
 // (distributed shared memory).
 //
 // While the block shape is left to the library and the tubes are few, a tube's
-// team is instead one CTA per chunk, up to the whole chip: a cooperative
-// launch whose CTAs meet at the barrier of mxe_team.cuh.  One tube
-// on one CTA runs on 1/152 of the chip, pass after pass over its chunks, while
-// a stage takes 3 us for one chunk as for many side by side.  4096 cells, planar,
-// per RK2 step: 201 -> 11.5 us (33 CTAs; set-up and read-back not counted).
+// team is instead one CTA of four warps per 120 cells, up to the whole chip: a
+// cooperative launch whose CTAs meet at the barrier of mxe_team.cuh.  One tube
+// on one CTA runs on 1/152 of the chip, pass after pass over its cells, while a
+// stage takes 3 us for one pass as for many side by side.  4096 cells, planar,
+// per RK2 step: 201 -> 9.5 us (35 CTAs; set-up and read-back not counted).
 #include "mxe_internal.h"
 #include "mxe_mixed_x2.cuh"
 #include "mxe_team.cuh"

@@ -898,13 +898,13 @@ static F64Tile f64_tile(const mxe_ctx* c, bool pl) {
 
 // Tile of the packed mixed stage.  Time of an RK2 step on GB300 (152 SMs), us:
 //            48 x 48  130 x 130  200 x 200  300 x 300  400 x 400  512 x 512  1024 x 1024
-//   31 x 18     35        35         35         43         44         76         224
-//   31 x  7     22        22         26         36         51         80         273
-//   15 x  7     18        21         29         41         67        103         386
+//   31 x 18     34        35         35         43         43         72         213
+//   31 x  7     22        21         26         33         47         76         254
+//   15 x  7     19        21         28         40         67        102         371
 // (one tile before: 33 on 48 x 48, 262 on 1024 x 1024); general states:
-//   31 x 15     39        40         40         52         74         93         330
-//   31 x  7     27        27         33         45         67        107         374
-//   15 x  7     22        25         33         52         89        138         540
+//   31 x 15     38        38         39         51         70         87         316
+//   31 x  7     27        27         31         42         64        102         351
+//   15 x  7     21        25         33         51         88        137         535
 // (scalar faces before: 35 on 48 x 48, 92 on 400 x 400).  Small grids pay for the
 // passes of one block, then for each block; the large tiles come two to an SM,
 // in waves.

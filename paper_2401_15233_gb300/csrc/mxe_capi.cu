@@ -353,16 +353,21 @@ static mxe_status team_plans(mxe_ctx* c) {
         }
     if (per < 1) return fail(c, MXE_ECUDA, "the tube kernel does not fit on the device");
     if (c->mixed && c->ntubes > nsm) return MXE_OK;      // one CTA a tube fills the chip
+    // both plans and the barrier slots in one allocation
+    std::vector<TubeTeam> all;
     for (int k = 0; k < 2; ++k) {
         std::vector<TubeTeam> t;
         team_plan(c, k == 1, per * nsm, c->mixed ? 120 : 31, c->mixed ? 120 : 63, t,
                   &c->team_chunk[k], &c->team_coop[k]);
         c->team_ctas[k] = (int)t.size();
-        CK(cudaMalloc(&c->team_d[k], sizeof(TubeTeam) * t.size()));
-        CK(cudaMemcpyAsync(c->team_d[k], t.data(), sizeof(TubeTeam) * t.size(), cudaMemcpyHostToDevice,
-                       c->own_stream));
+        all.insert(all.end(), t.begin(), t.end());
     }
-    CK(cudaMalloc(&c->sync_d, sizeof(TubeSync) * c->ntubes));
+    const size_t slots = sizeof(TubeSync) * c->ntubes;
+    CK(cudaMalloc(&c->sync_d, slots + sizeof(TubeTeam) * all.size()));
+    c->team_d[0] = (TubeTeam*)((char*)c->sync_d + slots);
+    c->team_d[1] = c->team_d[0] + c->team_ctas[0];
+    CK(cudaMemcpyAsync(c->team_d[0], all.data(), sizeof(TubeTeam) * all.size(),
+                       cudaMemcpyHostToDevice, c->own_stream));
     return MXE_OK;
 }
 
@@ -563,9 +568,7 @@ extern "C" void mxe_destroy(mxe_ctx* c) {
     cudaFree(c->order_d);
     cudaFree(c->queue_d);
     cudaFree(c->rates_d);
-    cudaFree(c->team_d[0]);
-    cudaFree(c->team_d[1]);
-    cudaFree(c->sync_d);
+    cudaFree(c->sync_d);              // and the team plans behind it
     cudaFree(c->dth);
     cudaFree(c->tape);
     cudaFree(c->adjP);

@@ -464,7 +464,8 @@ mxe_stage14_2d_mixed_planar_b3(const Stage2DArgs a, const ParamsT<float> p,
 // 31 x 18 fits 1024 x 1024 in whole waves better (3.45 ms and 243 us there with
 // the accurate CFL rates; 3.79 ms and 261 us before).  With the limiter in
 // fewer instructions, the box asked for before the step size is known and the
-// items in rows of a warp: 3.00 ms and 216 us.
+// items in rows of a warp: 3.00 ms and 216 us (31 x 17: 3.02 and 220, 31 x 19:
+// 3.06 and 228).
 template <int TX_, int TY_, int NT_>
 struct TileGeo {
     static constexpr int TX = TX_, TY = TY_, NT = NT_;

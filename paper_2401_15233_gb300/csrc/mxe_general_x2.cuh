@@ -9,6 +9,10 @@
 namespace mxe {
 namespace x2 {
 
+// the jump of a product x y from the jumps of its factors
+__device__ __forceinline__ float djump(v2 x, float dx, v2 y, float dy) {
+    return fmaf(x.y, dy, y.x * dx);
+}
 // cofactors of a symmetric 3 x 3 matrix (xx, xy, xz, yy, yz, zz); returns det
 __device__ __forceinline__ v2 cofactors(const v2* A, v2* c) {
     const v2 n1 = neg(A[1]), n2 = neg(A[2]), n4 = neg(A[4]);
@@ -77,7 +81,7 @@ __device__ __forceinline__ void face_eval14_x2(const v2* Q, const float* D, floa
         lam_core_x2(P[sidx(K, K)], q[K], sqrt_(fma(q[E1], q[E1], mul(q[E2], q[E2]))), sb, isb, ssb,
                     lp, lm);
         const v2 ks = mul(sq, S(k_ws));
-        w = flux_weights<RUS>(fma(lm, neg(ks), u[K]), fma(lp, ks, u[K]));
+        w = flux_weights<RUS>(fma(lm, ks, u[K]), fma(lp, ks, u[K]));
     }
     // ---- closure slice along K: Qk = Q_Kij, Rk = R_Kijj, Sk = S_Kiijj
     v2 Qk[6], Rk[3], Sk;
@@ -150,9 +154,9 @@ __device__ __forceinline__ void face_eval14_x2(const v2* Q, const float* D, floa
         mo[i] = mul(rho, u[i]);
         dmo[i] = RUS ? djump(rho, D[0], u[i], du[i]) : jump(mo[i]);
     }
-    Fn[0] = weigh(w, mo[K], RUS ? D[0] : jump(rho));
+    Fn[0] = weigh<RUS>(w, mo[K], RUS ? D[0] : jump(rho));
 #pragma unroll
-    for (int i = 0; i < 3; ++i) Fn[1 + i] = weigh(w, fma(uK, mo[i], Pd[sidx(i, K)]), dmo[i]);
+    for (int i = 0; i < 3; ++i) Fn[1 + i] = weigh<RUS>(w, fma(uK, mo[i], Pd[sidx(i, K)]), dmo[i]);
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
@@ -161,7 +165,7 @@ __device__ __forceinline__ void face_eval14_x2(const v2* Q, const float* D, floa
             const v2 Un = fma(mo[i], u[j], Pd[n]);
             const v2 c = i == j ? fma(add(u[i], u[i]), Pd[sidx(i, K)], Qk[n])
                                 : fma(u[i], Pd[sidx(j, K)], fma(u[j], Pd[sidx(i, K)], Qk[n]));
-            Fn[4 + n] = weigh(w, fma(uK, Un, c),
+            Fn[4 + n] = weigh<RUS>(w, fma(uK, Un, c),
                               RUS ? djump(mo[i], dmo[i], u[j], du[j]) + dP[n] : jump(Un));
         }
     const v2 u2 = dot3(u[0], u[1], u[2], u), ru2 = mul(rho, u2), e = add(ru2, tr);
@@ -186,7 +190,7 @@ __device__ __forceinline__ void face_eval14_x2(const v2* Q, const float* D, floa
     for (int i = 0; i < 3; ++i) {
         const v2 Un = fma(u[i], e, fma(Pu[i], S(2.0f), Q[10 + i]));
         const v2 c = fma(u[i], gK, fma(u2, Pd[sidx(i, K)], fma(Qu[i], S(2.0f), Rk[i])));
-        Fn[10 + i] = weigh(w, fma(uK, Un, c),
+        Fn[10 + i] = weigh<RUS>(w, fma(uK, Un, c),
                            RUS ? djump(u[i], du[i], e, dru2 + dtr) + fmaf(2.0f, dPu[i], dq[i])
                                : jump(Un));
         Pq[i] = add(Pu[i], Q[10 + i]);
@@ -196,26 +200,9 @@ __device__ __forceinline__ void face_eval14_x2(const v2* Q, const float* D, floa
     const v2 e2 = fma(tr, S(2.0f), ru2);
     const v2 U13 = fma(u2, e2, fma(dot3(u[0], u[1], u[2], Pq), S(4.0f), Q[13]));
     const v2 c13 = fma(add(u2, u2), gK, fma(dot3(u[0], u[1], u[2], Rk), S(4.0f), Sk));
-    Fn[13] = weigh(w, fma(uK, U13, c13),
+    Fn[13] = weigh<RUS>(w, fma(uK, U13, c13),
                    RUS ? djump(u2, du2, e2, fmaf(2.0f, dtr, dru2)) + fmaf(4.0f, duPq, D[13])
                        : jump(U13));
-}
-
-// CFL rates of one cell state in x and y
-__device__ __forceinline__ void rates14_x2(const float* Q, float sigma_lim, float k_ws, float& ax,
-                                           float& ay) {
-    Dimless14<float> d;
-    dimless14(Q, d);
-    const float sb = clamp_sigma(d.sig, sigma_lim), z2 = d.qs[2] * d.qs[2];
-    v2 lp, lm;
-    lam_core_x2(make_float2(d.Ps[0], d.Ps[3]), make_float2(d.qs[0], d.qs[1]),
-                make_float2(sqrtf(d.qs[1] * d.qs[1] + z2), sqrtf(d.qs[0] * d.qs[0] + z2)), S(sb),
-                S(1.0f / sb), S(sqrtf(sb)), lp, lm);
-    const v2 uv = make_float2(Q[1], Q[2]);
-    const v2 ks = S(k_ws * d.sq);
-    const v2 hi = fma(lp, ks, uv), lo = fma(lm, neg(ks), uv);
-    ax = fmaxf(fabsf(lo.x), fabsf(hi.x));
-    ay = fmaxf(fabsf(lo.y), fabsf(hi.y));
 }
 
 }  // namespace x2

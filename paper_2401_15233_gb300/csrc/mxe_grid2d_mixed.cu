@@ -23,7 +23,6 @@
 // planar (ten-moment) state.
 #include "mxe_internal.h"
 #include "mxe_mixed_x2.cuh"
-#include "mxe_rate32.cuh"
 
 namespace mxe {
 
@@ -344,7 +343,7 @@ __device__ __forceinline__ void stage_mixed(const Stage2DArgs& a, const ParamsT<
 #pragma unroll
         for (int k = 0; k < NF; ++k) Qc[k] = W[k * NBOXm + (cy + 2) * BXm + cx + 2];
         if (p.tau_model != 0 && !p.src_implicit) {
-            PH::source(Qc, p, L);
+            PH::source(Qc, PH::tau(p, Qc), L);
         } else {
 #pragma unroll
             for (int k = 0; k < NF; ++k) L[k] = 0.0f;
@@ -506,21 +505,6 @@ constexpr size_t smem_mixed_x2() {
     return sizeof(float) * (NF * (G::NBOX + G::NFX + G::NFY) + G::NPX + G::NPY + G::NT / 32);
 }
 
-// CFL rate of the cell whose conserved state starts at U (see mxe_rate32.cuh)
-template <class PH>
-__device__ __noinline__ float cell_rate(const double* U, long long fstride, float sigma_lim,
-                                        float k_ws, float idx, float idy) {
-    double Uc[PH::NF], Q[PH::NF];
-    float W[PH::NF];
-#pragma unroll
-    for (int k = 0; k < PH::NF; ++k) Uc[k] = U[PH::ufield(k) * fstride];
-    PH::cons2prim_fast(Uc, Q);
-#pragma unroll
-    for (int k = 0; k < PH::NF; ++k) W[k] = f64::to_f32(Q[k]);
-    const float r = rn::rate<PH::NF>(W, sigma_lim, k_ws, idx, idy);
-    return r >= 0.0f ? r : __int_as_float(0x7f800000);             // NaN -> inf
-}
-
 template <class PH, class G, bool RUS>
 __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const ParamsT<float>& p,
                                                const MixedPolicy& mp) {
@@ -533,7 +517,7 @@ __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const Param
     float* phy = phx + G::NPX;                       // [TY+2][TX]
     float* red = phy + G::NPY;                       // [NT / 32]
     __shared__ double sdt[2];
-    __shared__ float scdt, srate;
+    __shared__ float scdt;
     __shared__ unsigned cnt;
 
     const int tid = threadIdx.x;
@@ -643,18 +627,9 @@ __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const Param
 #pragma unroll
         for (int k = 0; k < NF; ++k) Fy[k * G::NFY + f] = F[k];
     }
-    // cells with a smaller approximate rate are not evaluated again: those below
-    // what other blocks have found (that only grows), or 1 % below the last
-    // step's maximum
-    if (a.final_stage && tid == 0) {
-        const volatile unsigned long long* rt = a.clk->rate;
-        srate = fmaxf((float)__longlong_as_double((long long)rt[(a.slot + 1) % 3]) * (1.0f - 0x1p-15f),
-                      (float)__longlong_as_double((long long)rt[a.slot]) * 0.99f);
-    }
     __syncthreads();
 
     float r = 0.0f;
-    long long orate = 0;         // the cell of r
     const float cdt = scdt;
     const bool implicit = p.tau_model != 0 && p.src_implicit;
 #pragma unroll 1
@@ -679,7 +654,7 @@ __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const Param
 #pragma unroll
         for (int k = 0; k < NF; ++k) Qc[k] = W[k * G::NBOX + cb];
         if (p.tau_model != 0 && !p.src_implicit) {
-            PH::source(Qc, p, L);
+            PH::source(Qc, PH::tau(p, Qc), L);
         } else {
 #pragma unroll
             for (int k = 0; k < NF; ++k) L[k] = 0.0f;
@@ -733,17 +708,12 @@ __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const Param
             if (bad) atomicOr(&a.clk->status, ST_NONFINITE);
             float ax, ay;
             if constexpr (NF == NP) x2::rates_x2(Wn, p.sigma_lim, p.k_ws, ax, ay);
-            else x2::rates14_x2(Wn, p.sigma_lim, p.k_ws, ax, ay);
+            else PH::rates(Wn, p.sigma_lim, p.k_ws, ax, ay);
             float rc = ax * a.idxf + ay * a.idyf;
             if (!(rc >= 0.0f)) rc = __int_as_float(0x7f800000);     // NaN -> inf
-            if (rc >= r) {
-                r = rc;
-                orate = o;
-            }
+            r = fmaxf(r, rc);
         }
     }
-    if (a.final_stage && r >= srate && r > 0.0f)
-        r = cell_rate<PH>(a.Uout + orate, g.fstride, p.sigma_lim, p.k_ws, a.idxf, a.idyf);
     unsigned wf = __reduce_add_sync(0xffffffffu, nflag);
     if ((tid & 31) == 0 && wf) atomicAdd(&cnt, wf);
     if (a.final_stage) block_max_atomic_m(r, &a.clk->rate[(a.slot + 1) % 3], red);
@@ -830,7 +800,9 @@ __device__ __forceinline__ void rate_mixed(const float* W, const Grid2D& g, cons
         float Q[PH::NF];
 #pragma unroll
         for (int k = 0; k < PH::NF; ++k) Q[k] = W[o + k * g.fstride];
-        r = rn::rate<PH::NF>(Q, p.sigma_lim, p.k_ws, idxf, idyf);
+        float ax, ay;
+        PH::rates(Q, p.sigma_lim, p.k_ws, ax, ay);
+        r = ax * idxf + ay * idyf;
         if (!(r >= 0.0f)) r = __int_as_float(0x7f800000);
     }
     block_max_atomic_m(r, &clk->rate[slot], red);

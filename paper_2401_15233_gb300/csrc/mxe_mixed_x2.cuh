@@ -9,72 +9,62 @@
 
 namespace mxe {
 
-// Shared limiter by ratios.  r_k = min(|dm|, |dp|) / max(|dm|, |dp|), negative
-// for opposite signs; both limiters increase with r on [0, 1] (minmod
-// 2r/(1+r), van Albada 2r/(1+r^2)), so the field with the smallest ratio sets
-// phi, one division per cell and direction.  With i = 1/max, r = (dm i)(dp i): one
-// approximate reciprocal, three packed multiplications for the two
-// directions of a cell, no overflow.  A field is flat where max(|dm|, |dp|)
-// is within its tolerance, the larger of 2^-20 |w| and T times its natural
-// scale (field_flat's test, with the root taken): once per cell for both
-// directions.  6.5 instructions a field and direction; the same test on
-// cross-multiplied ratios took about 12.
+// One field's contribution to the shared limiter of one direction, tracked
+// as the ratio r = min(|dm|, |dp|) / max(|dm|, |dp|) of the most stringent
+// field so far (n / x).  Both limiters are increasing in r on [0, 1]
+// (minmod 2r/(1+r), van Albada 2r/(1+r^2)), so the field with the smallest
+// r sets phi, and ratios are compared cross-multiplied: one division per
+// cell and direction instead of one per field.  Opposite signs give r = 0;
+// a field with dm = dp = 0, or flat by the tolerance test, never lowers phi.
 template <int NF>
-struct FlatTol {
-    float t[5];                  // by scale class
-    __device__ __forceinline__ FlatTol(const float* w, int fs) {
-        const FlatRef<float> f = flat_ref<NF>(w, fs);
-        const float p = f.s * (1.0f / 3.0f), th = p * f64::rcp32(f.rho), v = sqrtf(th);
-        constexpr float T = FlatConst<float>::tol;
-        t[0] = T * f.rho;
-        t[1] = T * v;
-        t[2] = T * p;
-        t[3] = t[2] * v;
-        t[4] = t[2] * th;
+__device__ __forceinline__ void phi_ratio_step(float dm, float dp, float w0,
+                                               const FlatRef<float>& fr, int k, float& n,
+                                               float& x) {
+    const float am = fabsf(dm), ap = fabsf(dp);
+    const float mx = fmaxf(am, ap);
+    const float mn = dm * dp > 0.0f ? fminf(am, ap) : 0.0f;
+    if (mx > 0.0f && mn * x < n * mx) {
+        if (!(mx <= FLAT_REL_F32 * fabsf(w0) || field_flat<NF>(fr, k, mx))) {
+            n = mn;
+            x = mx;
+        }
     }
-    __device__ __forceinline__ float operator()(int k, float w0) const {
-        return fmaxf(FLAT_REL_F32 * fabsf(w0), t[flat_class<NF>(k)]);
-    }
-};
-__device__ __forceinline__ float phi_of_ratio(float r, int lim) {
-    r = fmaxf(r, 0.0f);
-    return (r + r) * f64::rcp32(1.0f + (lim == 1 ? r * r : r));
+}
+__device__ __forceinline__ float phi_of_ratio(float n, float x, int lim) {
+    return lim == 1 ? __fdividef(2.0f * n * x, n * n + x * x) : __fdividef(2.0f * n, n + x);
 }
 
-// Limiter of box cell c in x (result .x) and y (.y)
+// Shared limiter of box cell c in x (result .x) and y (.y): the stencil
+// centre and the flat-test reference are loaded once for both directions.
 template <int NF, int NBOX, int BX>
 __device__ __forceinline__ float2 phi_pair_m(const float* W, int c, int lim) {
     using namespace x2;
-    const FlatTol<NF> tol(W + c, NBOX);
-    float rx = 1.0f, ry = 1.0f;
+    const FlatRef<float> fr = flat_ref<NF>(W + c, NBOX);
+    float nx = 1.0f, xx = 1.0f, ny = 1.0f, xy = 1.0f;
 #pragma unroll
     for (int k = 0; k < NF; ++k) {
         const float* w = W + k * NBOX + c;
-        const float w0 = w[0], t = tol(k, w0);
-        // the x and y differences as the lanes of packed operations
+        const float w0 = w[0];
+        // the x and y differences as the lanes of packed subtractions
         const v2 dm = sub(S(w0), make_float2(w[-1], w[-BX]));
         const v2 dp = sub(make_float2(w[1], w[BX]), S(w0));
-        const float mx = abs_max(dm.x, dp.x), my = abs_max(dm.y, dp.y);
-        const v2 i = make_float2(f64::rcp32(mx), f64::rcp32(my));
-        const v2 r = mul(mul(dm, i), mul(dp, i));
-        if (mx > t) rx = fminf(rx, r.x);
-        if (my > t) ry = fminf(ry, r.y);
+        phi_ratio_step<NF>(dm.x, dp.x, w0, fr, k, nx, xx);
+        phi_ratio_step<NF>(dm.y, dp.y, w0, fr, k, ny, xy);
     }
-    return make_float2(phi_of_ratio(rx, lim), phi_of_ratio(ry, lim));
+    return make_float2(phi_of_ratio(nx, xx, lim), phi_of_ratio(ny, xy, lim));
 }
 // The same for one direction (stride 1: x, stride BX: y).
 template <int NF, int NBOX>
 __device__ __forceinline__ float phi_one_m(const float* W, int c, int stride, int lim) {
-    const FlatTol<NF> tol(W + c, NBOX);
-    float r = 1.0f;
+    const FlatRef<float> fr = flat_ref<NF>(W + c, NBOX);
+    float n = 1.0f, x = 1.0f;
 #pragma unroll
     for (int k = 0; k < NF; ++k) {
         const float* w = W + k * NBOX + c;
-        const float w0 = w[0], dm = w0 - w[-stride], dp = w[stride] - w0, m = abs_max(dm, dp);
-        const float i = f64::rcp32(m), q = (dm * i) * (dp * i);
-        if (m > tol(k, w0)) r = fminf(r, q);
+        const float w0 = w[0];
+        phi_ratio_step<NF>(w0 - w[-stride], w[stride] - w0, w0, fr, k, n, x);
     }
-    return phi_of_ratio(r, lim);
+    return phi_of_ratio(n, x, lim);
 }
 
 // FP64 face flux of a face whose packed FP32 evaluation found an
@@ -146,17 +136,20 @@ __device__ __forceinline__ void face_flux_x2(const float* W, int cl, int stride,
     };
     reconstruct();
     v2 sig, det;
-    float D[NF];             // the jumps Q_R - Q_L (Rusanov)
-    if (RUS) {
+    if constexpr (NF == NP) {
+        face_eval_x2<K, RUS>(Q, p.sigma_lim, p.k_ws, F, sig, det);
+    } else {
+        float D[NF];             // the jumps Q_R - Q_L (Rusanov)
+        if (RUS) {
 #pragma unroll
-        for (int k = 0; k < NF; ++k) {
-            const float* w = W + k * NBOX + cl;
-            const float w0 = w[0], w1 = w[stride];
-            D[k] = (w1 - w0) - 0.25f * fmaf(phr, w[2 * stride] - w0, phl * (w1 - w[-stride]));
+            for (int k = 0; k < NF; ++k) {
+                const float* w = W + k * NBOX + cl;
+                const float w0 = w[0], w1 = w[stride];
+                D[k] = (w1 - w0) - 0.25f * fmaf(phr, w[2 * stride] - w0, phl * (w1 - w[-stride]));
+            }
         }
+        face_eval14_x2<K, RUS>(Q, D, p.sigma_lim, p.k_ws, F, sig, det);
     }
-    if constexpr (NF == NP) face_eval_x2<K, RUS>(Q, D, p.sigma_lim, p.k_ws, F, sig, det);
-    else face_eval14_x2<K, RUS>(Q, D, p.sigma_lim, p.k_ws, F, sig, det);
     // the policy of face_state_m for both states at once (almost always clear),
     // then state by state
     bool odd = !(sig.x <= mp.sig_hi) || !(sig.y <= mp.sig_hi) || fminf(det.x, det.y) < mp.det_min;

@@ -681,23 +681,24 @@ __device__ __forceinline__ void prim_increment14(const float* W, const float* dU
 }
 
 // BGK sources of Sec. 2.4.
-__device__ __forceinline__ void source14_m(const float* Q, int model, float k, float* C) {
-    const float* u = Q + 1;
-    const float p = (Q[4] + Q[7] + Q[9]) * (1.0f / 3.0f), th = p * (1.0f / Q[0]);
-    const float it = model == 1 ? k : k * Q[0] * sqrtf(th);
-    const float D[6] = {p - Q[4], -Q[5], -Q[6], p - Q[7], -Q[8], p - Q[9]};
-    C[0] = C[1] = C[2] = C[3] = 0.0f;
-#pragma unroll
-    for (int n = 0; n < 6; ++n) C[4 + n] = D[n] * it;
-    float us = 0.0f;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        const float a = D[sidx(i, 0)] * u[0] + D[sidx(i, 1)] * u[1] + D[sidx(i, 2)] * u[2];
-        const float s = a - Q[10 + i];
-        C[10 + i] = it * (a + s);
-        us += u[i] * s;
-    }
-    C[13] = it * (4.0f * us + (15.0f * p * th - Q[13]));
+template <class T>
+__device__ __forceinline__ void source14(const T* Q, T tau, T* C) {
+    T rho = Q[0], ux = Q[1], uy = Q[2], uz = Q[3];
+    T Pxx = Q[4], Pxy = Q[5], Pxz = Q[6], Pyy = Q[7], Pyz = Q[8], Pzz = Q[9];
+    T p = (Pxx + Pyy + Pzz) / T(3);
+    C[0] = T(0); C[1] = T(0); C[2] = T(0); C[3] = T(0);
+    C[4] = -(Pxx - p) / tau; C[5] = -Pxy / tau; C[6] = -Pxz / tau;
+    C[7] = -(Pyy - p) / tau; C[8] = -Pyz / tau; C[9] = -(Pzz - p) / tau;
+    T Pux = Pxx * ux + Pxy * uy + Pxz * uz;
+    T Puy = Pxy * ux + Pyy * uy + Pyz * uz;
+    T Puz = Pxz * ux + Pyz * uy + Pzz * uz;
+    C[10] = -(T(2) * Pux + Q[10] - T(2) * ux * p) / tau;
+    C[11] = -(T(2) * Puy + Q[11] - T(2) * uy * p) / tau;
+    C[12] = -(T(2) * Puz + Q[12] - T(2) * uz * p) / tau;
+    T uPu = ux * Pux + uy * Puy + uz * Puz;
+    T uq = ux * Q[10] + uy * Q[11] + uz * Q[12];
+    T u2 = ux * ux + uy * uy + uz * uz;
+    C[13] = -((T(4) * uPu + T(4) * uq + Q[13]) - (T(4) * u2 * p + T(15) * p * p / rho)) / tau;
 }
 
 template <class T>

@@ -294,20 +294,21 @@ __device__ __forceinline__ T amax_p(const T* Q, const DimlessP<T>& g, T sigma_li
     return x > y ? x : y;
 }
 
-// BGK source of the FP32 stages, 1/tau = k rho sqrt(theta) (hard spheres) or k:
-// (P_M - P, (P_M - P).(2 u) - q, 4 u.((P_M - P) u - q) + 15 p^2/rho - R) / tau
-__device__ __forceinline__ void source_p_m(const float* Q, int model, float k, float* C) {
-    const float rho = Q[0], ux = Q[1], uy = Q[2], Pxy = Q[4];
-    const float p = (Q[3] + Q[5] + Q[6]) * (1.0f / 3.0f), th = p * (1.0f / rho);
-    const float it = model == 1 ? k : k * rho * sqrtf(th);
-    const float dx = p - Q[3], dy = p - Q[5];
-    C[0] = C[1] = C[2] = 0.0f;
-    C[3] = dx * it; C[4] = -Pxy * it; C[5] = dy * it; C[6] = (p - Q[6]) * it;
-    const float ax = dx * ux - Pxy * uy, ay = dy * uy - Pxy * ux;
-    const float sx = ax - Q[7], sy = ay - Q[8];
-    C[7] = it * (ax + sx);
-    C[8] = it * (ay + sy);
-    C[9] = it * (4.0f * (ux * sx + uy * sy) + (15.0f * p * th - Q[9]));
+template <class T>
+__device__ __forceinline__ void source_p(const T* Q, T tau, T* C) {
+    T rho = Q[0], ux = Q[1], uy = Q[2];
+    T Pxx = Q[3], Pxy = Q[4], Pyy = Q[5], Pzz = Q[6];
+    T p = (Pxx + Pyy + Pzz) / T(3);
+    C[0] = T(0); C[1] = T(0); C[2] = T(0);
+    C[3] = -(Pxx - p) / tau; C[4] = -Pxy / tau; C[5] = -(Pyy - p) / tau; C[6] = -(Pzz - p) / tau;
+    T Pux = Pxx * ux + Pxy * uy;
+    T Puy = Pxy * ux + Pyy * uy;
+    C[7] = -(T(2) * Pux + Q[7] - T(2) * ux * p) / tau;
+    C[8] = -(T(2) * Puy + Q[8] - T(2) * uy * p) / tau;
+    T uPu = ux * Pux + uy * Puy;
+    T uq = ux * Q[7] + uy * Q[8];
+    T u2 = ux * ux + uy * uy;
+    C[9] = -((T(4) * uPu + T(4) * uq + Q[9]) - (T(4) * u2 * p + T(15) * p * p / rho)) / tau;
 }
 
 template <class T>

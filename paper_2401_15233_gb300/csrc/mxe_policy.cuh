@@ -15,14 +15,7 @@ struct ParamsT {
     int tau_model;
     T tau_ref, rho_ref, T_ref;
     int src_implicit;           // point-implicit source (relax after each stage)
-    T itau;                     // 1/tau (model 1), or 1/tau / (rho sqrt(theta)) (hard spheres)
 };
-
-// cell-independent factor of 1/tau (see f64::tau_factor)
-__host__ __device__ inline double itau_factor(const RelaxParams& rp) {
-    if (rp.model == 0) return 0.0;
-    return rp.model == 1 ? 1.0 / rp.tau_ref : 1.0 / (rp.tau_ref * rp.rho_ref * sqrt(rp.T_ref));
-}
 
 template <class T>
 __host__ __device__ inline ParamsT<T> make_params(const SchemeParams& sp, const RelaxParams& rp) {
@@ -37,7 +30,6 @@ __host__ __device__ inline ParamsT<T> make_params(const SchemeParams& sp, const 
     p.rho_ref = T(rp.rho_ref);
     p.T_ref = T(rp.T_ref);
     p.src_implicit = rp.implicit;
-    if (sizeof(T) == 4) p.itau = T(itau_factor(rp));      // FP32 stages only
     return p;
 }
 
@@ -96,9 +88,8 @@ struct PhysGeneral {
                                                   T& hi, T& sig, T& det) {
         face_eval14<T, K>(Q, sl, kw, U, F, lo, hi, sig, det);
     }
-    static __device__ __forceinline__ void source(const float* Q, const ParamsT<float>& p, float* C) {
-        source14_m(Q, p.tau_model, p.itau, C);
-    }
+    template <class T>
+    static __device__ __forceinline__ void source(const T* Q, T tau, T* C) { source14(Q, tau, C); }
     template <class T>
     static __device__ __forceinline__ T tau(const ParamsT<T>& p, const T* Q) {
         if (p.tau_model == 1) return p.tau_ref;
@@ -177,9 +168,8 @@ struct PhysPlanar {
                                                   T& hi, T& sig, T& det) {
         face_eval_p<T, K>(Q, sl, kw, U, F, lo, hi, sig, det);
     }
-    static __device__ __forceinline__ void source(const float* Q, const ParamsT<float>& p, float* C) {
-        source_p_m(Q, p.tau_model, p.itau, C);
-    }
+    template <class T>
+    static __device__ __forceinline__ void source(const T* Q, T tau, T* C) { source_p(Q, tau, C); }
     template <class T>
     static __device__ __forceinline__ T tau(const ParamsT<T>& p, const T* Q) {
         return tau_p(p.tau_model, p.tau_ref, p.rho_ref, p.T_ref, Q);

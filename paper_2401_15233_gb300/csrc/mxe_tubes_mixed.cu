@@ -225,7 +225,7 @@ __device__ float tube_stage_m(const TubeMixedArgs& a, const TubeView& v, const M
             for (int k = 0; k < NF; ++k) Qc[k] = Wb[k * BOX + lane + 2];
             const bool implicit = p.tau_model != 0 && p.src_implicit;
             if (p.tau_model != 0 && !implicit) {
-                PH::source(Qc, p, L);
+                PH::source(Qc, PH::tau(p, Qc), L);
             } else {
 #pragma unroll
                 for (int k = 0; k < NF; ++k) L[k] = 0.0f;
@@ -443,7 +443,6 @@ __device__ void tubes_mixed_body(const TubeMixedArgs& a, const ParamsT<float>& p
         v.p.rho_ref = (float)td.rp.rho_ref;
         v.p.T_ref = (float)td.rp.T_ref;
         v.p.src_implicit = td.rp.implicit;
-        v.p.itau = (float)f64::tau_factor(td.rp.model, td.rp.tau_ref, td.rp.rho_ref, td.rp.T_ref);
         TubeClock* ck = a.clk + b;
         const int n = v.n;
 

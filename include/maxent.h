@@ -20,7 +20,8 @@
  *
  * Ownership and threading
  *   - A context owns all device memory it allocates; mxe_destroy frees it.
- *   - Pointers passed in are borrowed for the duration of the call only.
+ *   - Pointers passed in are borrowed for the duration of the call only: device
+ *     arrays too are no longer read when the call returns.
  *   - Work is issued on the context's CUDA stream (mxe_set_stream); calls
  *     that return host data synchronise that stream.  A context must not be
  *     used from two host threads at once.

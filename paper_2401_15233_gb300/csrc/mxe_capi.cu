@@ -673,6 +673,8 @@ static void* pinned_alias(const void* p) {
     return at.type == cudaMemoryTypeHost ? at.devicePointer : nullptr;
 }
 
+constexpr size_t SET_STATE_COPY = size_t(64) << 20;
+
 extern "C" mxe_status mxe_set_state(mxe_ctx* c, int kind, const double* soa, int on_device) {
     if (!c) return MXE_EINVAL;
     if (!soa) return fail(c, MXE_EINVAL, "soa is NULL");
@@ -684,7 +686,16 @@ extern "C" mxe_status mxe_set_state(mxe_ctx* c, int kind, const double* soa, int
     const double* src = soa;
     const double* vsrc = soa;        // what the validation kernel reads
     double* copy = nullptr;          // where it leaves a device copy
-    if (!on_device) {
+    if (on_device) {
+        // The array is borrowed until this call returns; its owner may then reuse the
+        // memory on a stream that this one does not wait for.  The conversion below is
+        // launched after the checks have been waited for, so it reads the copy that
+        // the checks leave, or, where that would cost more than a wait, is itself
+        // waited for (set_state of a mixed grid on GB300, copy / wait: 33 / 36 us at
+        // 1.8 MB, 60 / 64 at 29 MB, 65.5 / 66.4 at 34 MB, 145 / 142 at 117 MB, 1837 / 1634
+        // at 1.9 GB).
+        if (bytes <= SET_STATE_COPY) src = copy = c->stage;
+    } else {
         src = c->stage;
         vsrc = (const double*)pinned_alias(soa);
         if (vsrc) {
@@ -721,6 +732,7 @@ extern "C" mxe_status mxe_set_state(mxe_ctx* c, int kind, const double* soa, int
     mxe_k_setstate<<<grid, 128, 0, c->stream>>>(m, c->nf, kind, src, c->U, w_set ? c->W : nullptr,
                                                 pl);
     CK(cudaGetLastError());
+    if (src == soa) CK(cudaStreamSynchronize(c->stream));
     if (w_set) c->w_planar = pl;
     if (!c->tubes && c->Us) CK(cudaMemsetAsync(c->Us, 0, sizeof(double) * c->nelem, c->stream));
     mxe_status s = reset_clock(c, w_set);

@@ -70,3 +70,30 @@ def test_primitive_and_conserved_input(mx, orc, planar):
         s.step_dt([1e-4, 1e-4])
         out.append(soa_to_aos(s.get_moments("conserved")))
     assert field_rel_err(out[0], out[1]).max() <= 2e-4
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("size", [[300], [97, 1200], (37, 29), (900, 700)])
+def test_device_array_is_free_after_the_call(mx, precision, size):
+    """A device array may be overwritten, on a stream that the solver's does not wait for,
+    as soon as set_state has returned (900 x 700 cells: more than the checks copy)."""
+    import torch
+    rng = np.random.default_rng(3)
+    if isinstance(size, tuple):
+        s = mx.Solver(nx=size[0], ny=size[1], precision=precision)
+        prim = aos_to_soa(wl.smooth_field14(rng, size[0], size[1], planar=False))
+    else:
+        s = mx.Batch(size, [1.0] * len(size), precision=precision)
+        prim = s.pack([wl.smooth_field14(rng, n, 1, planar=False)[0].T for n in size])
+    s.set_state(prim)
+    want = s.get_moments("conserved")
+    keep = torch.from_numpy(prim).cuda()
+    junk = torch.full_like(keep, float("nan"))
+    x = torch.empty_like(keep)
+    torch.cuda.synchronize()
+    for _ in range(20):
+        x.copy_(keep)
+        torch.cuda.synchronize()
+        s.set_state(x)
+        x.copy_(junk)                       # on torch's stream, at once
+        assert np.array_equal(s.get_moments("conserved"), want)

@@ -124,6 +124,8 @@ struct mxe_ctx {
     long long g_gen = -1;
     long long gen = 0;                // bumped whenever launch arguments change
     long long known_steps = -1;       // steps on the device clock, where the host knows them (else -1)
+    bool captured = false;            // a run of this context is in a caller's graph, whose replays move
+                                      // the device clock unseen: no step count is known any more
     // dt history of 2D grids (steps counted from set_state)
     double* dth = nullptr;
     long long dth_cap = 0;
@@ -630,6 +632,19 @@ static void launch_resync(mxe_ctx* c, bool planar) {
 }
 
 // ---------------------------------------------------------------- clocks
+// A run is about to be launched: the device clock moves.
+static void clock_moves(mxe_ctx* c) {
+    c->known_steps = -1;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (c->captured) return;
+    if (cudaStreamIsCapturing(c->stream, &cs) == cudaSuccess)
+        c->captured = cs != cudaStreamCaptureStatusNone;
+    else
+        cudaGetLastError();
+}
+// steps on the device clock, or -1 if they have to be read
+static long long steps_known(const mxe_ctx* c) { return c->captured ? -1 : c->known_steps; }
+
 // w_set: W already holds the state's primitives
 static mxe_status reset_clock(mxe_ctx* c, bool w_set) {
     c->known_steps = 0;
@@ -944,7 +959,7 @@ static MixedTile mixed_tile(const mxe_ctx* c, bool pl) {
 // writes U* (default: the context's stage buffer).
 static mxe_status launch_2d_step(mxe_ctx* c, double t_end, double dt_fixed,
                                  double* ustar = nullptr, bool skip_rate = false) {
-    c->known_steps = -1;
+    clock_moves(c);
     Stage2DArgs a{};
     a.skip_rate = skip_rate && !c->mixed;
     a.dt_hist = c->dth;
@@ -1356,7 +1371,7 @@ static mxe_status run_tubes_mixed(mxe_ctx* c, int max_steps, double t_end, const
 
 static mxe_status run_tubes(mxe_ctx* c, int max_steps, double t_end, const double* dts,
                             int ndts) {
-    c->known_steps = -1;
+    clock_moves(c);
     if (c->mixed) return run_tubes_mixed(c, max_steps, t_end, dts, ndts);
     TubeArgs a{};
     a.U = c->U;
@@ -1418,7 +1433,7 @@ extern "C" mxe_status mxe_step(mxe_ctx* c, int max_steps, double t_end, double* 
     if (s != MXE_OK) return s;
     if (c->tubes) {
         if (!bc_planar(c)) c->state_planar = false;      // stays off until set_state
-        long long st0 = c->known_steps, st1 = 0;
+        long long st0 = steps_known(c), st1 = 0;
         if (steps_out && st0 < 0) {
             s = tube_status(c, nullptr, &st0);
             if (s != MXE_OK) return s;
@@ -1436,7 +1451,7 @@ extern "C" mxe_status mxe_step(mxe_ctx* c, int max_steps, double t_end, double* 
         return MXE_OK;
     }
     DevClock h{};
-    long long st0 = c->known_steps;
+    long long st0 = steps_known(c);
     bool want = t_out || steps_out;
     if (want && st0 < 0) {
         s = read_clock_2d(c, &h);

@@ -45,9 +45,12 @@ __device__ __forceinline__ double raw_sigma(const double* Q, int nf) {
 // A state that is realizable by a clear margin, decided without the FP64 pipe
 // (2 operations a clock and SM here, against 128 in FP32): every |Q| 0 or
 // in [1e-30, 1e30], and in FP32 sigma <= 0.99 and, of P* = 3 P / tr P, the
-// diagonal element > 0, the leading minor > 1e-4 and det >= 1e-3 (a positive
-// definite P* of that determinant has a leading minor of at least det / 3; the FP32
-// errors are orders of magnitude below these margins).
+// diagonal > 0, the leading minor > 1e-4 and det >= 1e-3 (a positive definite P* of
+// that determinant has a leading minor of at least det / 3).  A positive diagonal
+// of trace 3 bounds each of its elements by 3, the minor then P*_xy, and the last
+// condition P*_xz and P*_yz: the FP32 errors of the minor (2e-6) and of det (3e-5)
+// are far below their margins.  Without those bounds both could be cancellation
+// noise of large elements, of any sign.
 __device__ __forceinline__ bool clearly_realizable(const double* Q, int nf) {
     bool screen = true;
     float Qf[14];
@@ -64,8 +67,10 @@ __device__ __forceinline__ bool clearly_realizable(const double* Q, int nf) {
     }
     Dimless14<float> d;
     dimless14(Qf, d);
-    return d.th > 0.0f && d.Ps[0] > 0.0f && d.Ps[0] * d.Ps[3] - d.Ps[1] * d.Ps[1] > 1e-4f && d.det >= 1e-3f &&
-           d.sig <= 0.99f;                                    // false for NaN
+    const float* P = d.Ps;                                    // every test false for NaN
+    return d.th > 0.0f && P[0] > 0.0f && P[3] > 0.0f && P[5] > 0.0f && fabsf(P[2]) <= 3.0f &&
+           fabsf(P[4]) <= 3.0f && P[0] * P[3] - P[1] * P[1] > 1e-4f && d.det >= 1e-3f &&
+           d.sig <= 0.99f;
 }
 
 // 0 ok; 1 non-finite; 2 rho <= 0 or P not positive definite; 3 sigma > 1

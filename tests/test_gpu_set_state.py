@@ -97,3 +97,26 @@ def test_device_array_is_free_after_the_call(mx, precision, size):
         s.set_state(x)
         x.copy_(junk)                       # on torch's stream, at once
         assert np.array_equal(s.get_moments("conserved"), want)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("size,off", [(3e2, 0.0), (3e2, 1e-4), (3e3, 0.0), (3e3, 1e-2)])
+def test_cancelling_pressures_are_refused(mx, precision, size, off):
+    """A negative P_zz beside large P_xx, P_yy that cancel it in the trace, and P_xy near
+    sqrt(P_xx P_yy): in FP32 the minors are noise of any sign, in FP64 they are not."""
+    rng = np.random.default_rng(int(size) + int(1e6 * off))
+    good = _cell([1, 0, 0, 1, 0, 1])
+    s = mx.Solver(nx=8, ny=5, precision=precision)
+    prim = np.repeat(good[:, None], 40, 1).reshape(14, 5, 8).copy()
+    s.set_state(prim)
+    want = s.get_moments("conserved")
+    for _ in range(300):
+        a, d = size * rng.uniform(0.2, 1.0, 2)
+        b = np.sqrt(a * d) * (1.0 + rng.uniform(-1, 1) * 10.0 ** rng.uniform(-9, -6))
+        xz, yz = size * off * rng.uniform(-1, 1, 2)
+        prim[:, 3, 6] = good
+        prim[4:10, 3, 6] = a, b, xz, d, yz, 3.0 - a - d        # tr P = 3
+        prim[13, 3, 6] = 1e6                                   # sigma far below 1
+        with pytest.raises(mx.MaxentError, match="input cell 30"):
+            s.set_state(prim)
+    assert np.array_equal(s.get_moments("conserved"), want)    # and the state is kept

@@ -103,6 +103,7 @@ struct mxe_ctx {
     // and one for runs to a common time (mixed tubes: while the block shape is
     // the library's own choice; team_ctas[0] == 0 if teams do not pay)
     TubeTeam* team_d[2] = {nullptr, nullptr};
+    std::vector<TubeTeam> team_h;     // both plans as they are copied to the device
     int team_ctas[2] = {0, 0}, team_chunk[2] = {63, 63};
     bool team_coop[2] = {false, false};
     TubeSync* sync_d = nullptr;
@@ -356,7 +357,7 @@ static mxe_status team_plans(mxe_ctx* c) {
     if (per < 1) return fail(c, MXE_ECUDA, "the tube kernel does not fit on the device");
     if (c->mixed && c->ntubes > nsm) return MXE_OK;      // one CTA a tube fills the chip
     // both plans and the barrier slots in one allocation
-    std::vector<TubeTeam> all;
+    std::vector<TubeTeam>& all = c->team_h;
     for (int k = 0; k < 2; ++k) {
         std::vector<TubeTeam> t;
         team_plan(c, k == 1, per * nsm, c->mixed ? 120 : 31, c->mixed ? 120 : 63, t,
@@ -373,6 +374,9 @@ static mxe_status team_plans(mxe_ctx* c) {
     return MXE_OK;
 }
 
+// The host arrays that are copied here belong to the context: where the device reads
+// pageable memory itself, such a copy may still be on its way when the call returns.
+//
 // Tube contexts: device descriptors and clocks; for the mixed path also the
 // work queue, its hand-out order (largest n/dx first: a tube's work grows as
 // cells x steps ~ n^2 / length), the capture stream and the kernel
@@ -390,10 +394,10 @@ static mxe_status tubes_setup(mxe_ctx* c) {
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
         return c->tdesc[x].n / c->tdesc[x].dx > c->tdesc[y].n / c->tdesc[y].dx;
     });
-    CK(cudaMalloc(&c->order_d, sizeof(int) * n));
-    CK(cudaMemcpyAsync(c->order_d, order.data(), sizeof(int) * n, cudaMemcpyHostToDevice,
-                       c->own_stream));
     c->order_h = order;
+    CK(cudaMalloc(&c->order_d, sizeof(int) * n));
+    CK(cudaMemcpyAsync(c->order_d, c->order_h.data(), sizeof(int) * n, cudaMemcpyHostToDevice,
+                       c->own_stream));
     CK(cudaMalloc(&c->rates_d, sizeof(float) * n));
     CK(cudaMalloc(&c->queue_d, 2 * sizeof(int)));
     CK(cudaMemsetAsync(c->queue_d, 0, 2 * sizeof(int), c->own_stream));

@@ -55,7 +55,9 @@ typedef enum {
     MXE_EUNREALIZABLE = 4,   /* input state not realizable (rho<=0, P not SPD,
                                 sigma > 1)                                     */
     MXE_ENONFINITE = 5,      /* a non-finite value appeared in the state       */
-    MXE_ETIMEOUT = 6,        /* a bounded device wait gave up                  */
+    MXE_ETIMEOUT = 6,        /* a bounded device wait gave up: the state is partly
+                                advanced, and the context takes a new one
+                                (mxe_set_state) before it runs again           */
     MXE_ESTATE = 7           /* call not valid in the context's current state  */
 } mxe_status;
 
@@ -188,7 +190,10 @@ mxe_status mxe_set_source_scheme(mxe_ctx *ctx, int scheme);
  * (rho <= 0 or a diagonal pressure <= 0: the scheme does not guarantee
  * realizability, and the wave speeds of such a state are undefined) or if
  * the CFL step size collapsed to zero before t_end (a non-finite wave
- * speed); the state is left as the last step wrote it.  These are found
+ * speed); the state is left as the last step wrote it.  1D contexts whose
+ * tubes are marched by teams of thread blocks (mxe_batch_create) return
+ * MXE_ETIMEOUT if the blocks of a team waited in vain for one another (about
+ * 6 s); the state is then of no use.  These are found
  * from the device clock, i.e. when the call synchronises; an asynchronous
  * call (max_steps <= 4, no t_out / steps_out) reports them on the next
  * synchronising call or through mxe_get_diagnostics. */
@@ -268,8 +273,9 @@ mxe_status mxe_batch_set_relaxation(mxe_ctx *ctx, int tube, int model, double ta
 mxe_status mxe_batch_get_clock(mxe_ctx *ctx, double *t, long long *steps);
 
 /* Advance every tube until its own t reaches t_end or it has taken
- * max_steps steps in this call.  MXE_FP64: one launch (see mxe_batch_create);
- * MXE_ETIMEOUT if the blocks of a team lost each other.
+ * max_steps steps in this call.  MXE_FP64: one launch (see mxe_batch_create).
+ * Errors as mxe_step's, found by the next call that synchronises and checks
+ * (mxe_step, mxe_step_dt).
  * MXE_MIXED: one persistent launch of teams of CTAs (clusters) over a work
  * queue ordered by expected work (largest first); when the teams cannot use
  * every CTA slot of the device (clusters are placed whole within a GPU
@@ -418,7 +424,9 @@ mxe_status mxe_adjoint_residual(mxe_ctx *ctx, const double *U, const double *V, 
  *    be serialised by the caller.
  *  - t_out / steps_out (host, may be NULL) receive the final time and the
  *    steps taken; passing either synchronises `stream` (a cudaStream_t, NULL
- *    for the default stream).  A non-finite state (MXE_ENONFINITE) is
+ *    for the default stream).  A non-finite state (MXE_ENONFINITE), or a wait of
+ *    the launch's blocks for one another that gave up after about 6 s
+ *    (MXE_ETIMEOUT, U partly advanced), is
  *    detected from the clock read back for them, so it is reported only
  *    when t_out or steps_out is given; with both NULL the call returns
  *    MXE_OK once the work is queued.

@@ -107,6 +107,7 @@ struct mxe_ctx {
     int team_ctas[2] = {0, 0}, team_chunk[2] = {63, 63};
     bool team_coop[2] = {false, false};
     TubeSync* sync_d = nullptr;
+    int spin = TEAM_SPIN_LIMIT;
     int* queue_d = nullptr;           // mixed tubes: work counters of the team and fill launches
     cudaStream_t fill_stream = nullptr;    // the fill launch (forked from and joined to the work stream)
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
@@ -371,6 +372,21 @@ static mxe_status team_plans(mxe_ctx* c) {
     c->team_d[1] = c->team_d[0] + c->team_ctas[0];
     CK(cudaMemcpyAsync(c->team_d[0], all.data(), sizeof(TubeTeam) * all.size(),
                        cudaMemcpyHostToDevice, c->own_stream));
+    return MXE_OK;
+}
+
+// For the tests of the teams' barrier (not part of the API): launches from now on poll
+// `spin` times at most (0: the default), and the first team of each plan counts on `absent`
+// CTAs that are not launched, so that its wait runs out.
+extern "C" mxe_status mxe_test_team_wait(mxe_ctx* c, int spin, int absent) {
+    if (!c || !c->sync_d) return MXE_ESTATE;
+    CK(cudaStreamSynchronize(c->stream));
+    std::vector<TubeTeam> t = c->team_h;
+    for (TubeTeam& m : t)
+        if (m.tube == 0) m.size += absent;
+    CK(cudaMemcpy(c->team_d[0], t.data(), sizeof(TubeTeam) * t.size(), cudaMemcpyHostToDevice));
+    c->spin = spin > 0 ? spin : TEAM_SPIN_LIMIT;
+    ++c->gen;
     return MXE_OK;
 }
 
@@ -1285,6 +1301,7 @@ static mxe_status launch_tubes_mixed(mxe_ctx* c, cudaStream_t st, const TubeMixe
         TubeMixedArgs at = a;
         at.teams = c->team_d[L.plan];
         at.sync = c->sync_d;
+        at.spin = c->spin;
         CK(cudaMemsetAsync(c->sync_d, 0, sizeof(TubeSync) * c->ntubes, st));
         CK(launch_tube_grid(st, L, 1, c->team_ctas[L.plan], at, p, mp, c->team_coop[L.plan]));
         return MXE_OK;
@@ -1402,6 +1419,7 @@ static mxe_status run_tubes(mxe_ctx* c, int max_steps, double t_end, const doubl
     const int k = dts || !std::isfinite(t_end) ? 0 : 1;
     a.teams = c->team_d[k];
     a.sync = c->sync_d;
+    a.spin = c->spin;
     CK(cudaMemsetAsync(c->sync_d, 0, sizeof(TubeSync) * c->ntubes, c->stream));
     CK(launch_tubes_f64(tubes_f64_kernel(c->nf, tubes_planar(c), c->team_chunk[k]),
                         c->team_ctas[k], c->team_coop[k], a, c->stream));
@@ -1416,8 +1434,11 @@ static mxe_status tube_status(mxe_ctx* c, double* t0, long long* steps0) {
     if (t0) *t0 = h[0].t;
     if (steps0) *steps0 = h[0].steps;
     for (int b = 0; b < c->ntubes; ++b) {
-        if (h[b].status & ST_TIMEOUT)
-            return fail(c, MXE_ETIMEOUT, "tube %d: the CTAs of its team lost each other", b);
+        if (h[b].status & ST_TIMEOUT) {
+            c->have_state = false;        // partly advanced: of no use
+            return fail(c, MXE_ETIMEOUT, "tube %d: the CTAs of its team lost each other; the state "
+                                         "is partly advanced and has to be set again", b);
+        }
         if (h[b].status & ST_NONFINITE)
             return fail(c, MXE_ENONFINITE, "tube %d: non-finite state at t = %g", b, h[b].t);
         if (h[b].status & ST_NONPOSITIVE)

@@ -113,6 +113,7 @@ struct alignas(64) TubeSync {
 struct TubeArgs {
     const TubeTeam* teams;          // per CTA; NULL: all CTAs work on tube 0
     TubeSync* sync;                 // per tube
+    int spin;                       // polls after which a team's wait gives up
     const unsigned* nonplanar;      // general kernel: 0 there selects the planar state (or NULL)
     double* U;                      // all tubes, FP64 conserved
     double* Us;                     // stage buffer (same layout)
@@ -137,6 +138,7 @@ struct TubeMixedArgs {
     const TubeDesc* tubes;
     const TubeTeam* teams;          // per CTA of a launch of teams across the chip (or NULL)
     TubeSync* sync;                 // per tube, of such a launch
+    int spin;                       // polls after which a team's wait gives up
     const int* order;               // tube indices in the order they are handed out
     int* queue;                     // next position in `order` (zero at launch)
     TubeClock* clk;

@@ -168,6 +168,7 @@ extern "C" mxe_status mxe_tube_run_noalloc(const mxe_config* cfg, int bc_lo, int
     a.max_steps = max_steps;
     a.teams = nullptr;            // every CTA of the launch works on the one tube
     a.sync = p.sync;
+    a.spin = TEAM_SPIN_LIMIT;
     a.nonplanar = p.nonplanar;
     // one CTA per 31 cells while they are all resident, else chunks of 63 in
     // equal passes (the rule of a context's team plan)

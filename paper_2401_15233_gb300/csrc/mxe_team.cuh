@@ -6,8 +6,8 @@
 namespace mxe {
 
 // All threads of all `nb` CTAs; `target` counts arrivals since the launch.
-// Returns false (in every thread of the CTA) if the wait gave up.
-__device__ __forceinline__ bool team_barrier(TubeSync* s, unsigned nb, unsigned& target) {
+// Returns false (in every thread of the CTA) if the wait gave up after `spin` polls.
+__device__ __forceinline__ bool team_barrier(TubeSync* s, unsigned nb, unsigned& target, int spin) {
     __shared__ int ok;
     if (nb == 1u) {
         __syncthreads();
@@ -18,7 +18,7 @@ __device__ __forceinline__ bool team_barrier(TubeSync* s, unsigned nb, unsigned&
     if (threadIdx.x == 0) {
         __threadfence();                       // the CTA's writes before its arrival
         atomicAdd(&s->count, 1u);
-        int left = TEAM_SPIN_LIMIT, good = 1;
+        int left = spin, good = 1;
         unsigned v;
         do {
             asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(v) : "l"(&s->count) : "memory");

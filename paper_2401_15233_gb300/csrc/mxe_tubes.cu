@@ -157,7 +157,7 @@ __device__ __forceinline__ double tube_stage(const TubeArgs& a, const ParamsT<do
 // clears slot (e+2) mod 3: every CTA read it (epoch e-1) before arriving at
 // barrier e, and none writes it (epoch e+2) before barrier e+1, which the
 // first CTA reaches only after the clear.
-__device__ __forceinline__ bool team_reduce(TubeSync* s, unsigned rank, unsigned nb,
+__device__ __forceinline__ bool team_reduce(TubeSync* s, int spin, unsigned rank, unsigned nb,
                                             unsigned& target, unsigned& epoch, double r,
                                             unsigned st, double* red, unsigned* sst, double& m,
                                             unsigned& st_out) {
@@ -187,7 +187,7 @@ __device__ __forceinline__ bool team_reduce(TubeSync* s, unsigned rank, unsigned
         atomicMax(&s->rate[slot], (unsigned long long)__double_as_longlong(v));
         if (*sst) atomicOr(&s->stat[slot], *sst);
     }
-    if (!team_barrier(s, nb, target)) return false;
+    if (!team_barrier(s, nb, target, spin)) return false;
     m = __longlong_as_double((long long)__ldcg(&s->rate[slot]));
     st_out = __ldcg(&s->stat[slot]);
     if (rank == 0 && tid == 0) {
@@ -229,7 +229,7 @@ __device__ __forceinline__ void tubes_body(const TubeArgs& a) {
             if (!f64::ge0(ri)) ri = __longlong_as_double(0x7ff0000000000000ll);
             r = f64::max_(r, ri);
         }
-    ok = team_reduce(sy, rank, nb, target, epoch, r, 0u, sh.red, &sh.st, m, st);
+    ok = team_reduce(sy, a.spin, rank, nb, target, epoch, r, 0u, sh.red, &sh.st, m, st);
     double t = ck->t;
     long long steps = ck->steps;
     double last_dt = ck->last_dt;
@@ -249,7 +249,7 @@ __device__ __forceinline__ void tubes_body(const TubeArgs& a) {
         status = 0u;
         if (a.integrator == 1) {
             tube_stage<PH, C>(a, p, td, itau, rank, nb, cur, cur, nxt, 0.5, dt, false, sh, status);
-            if (!(ok = team_barrier(sy, nb, target))) break;
+            if (!(ok = team_barrier(sy, nb, target, a.spin))) break;
             rr = tube_stage<PH, C>(a, p, td, itau, rank, nb, nxt, cur, cur, 1.0, dt, true, sh,
                                    status);
         } else {
@@ -259,7 +259,8 @@ __device__ __forceinline__ void tubes_body(const TubeArgs& a) {
             cur = nxt;
             nxt = tmp;
         }
-        if (!(ok = team_reduce(sy, rank, nb, target, epoch, rr, status, sh.red, &sh.st, m, st)))
+        if (!(ok = team_reduce(sy, a.spin, rank, nb, target, epoch, rr, status, sh.red, &sh.st, m,
+                               st)))
             break;
         t += dt;
         last_dt = dt;

@@ -337,7 +337,7 @@ __device__ __forceinline__ void team_reduce(float r, unsigned st, unsigned& epoc
 // The same for a team across the chip, in the slots of its TubeSync (the
 // rotation of the three slots is that of team_reduce).
 template <int NT>
-__device__ __forceinline__ bool team_reduce_grid(TubeSync* s, float r, unsigned st,
+__device__ __forceinline__ bool team_reduce_grid(TubeSync* s, int spin, float r, unsigned st,
                                                  unsigned& epoch, unsigned& target, unsigned rank,
                                                  unsigned team, float* wred, unsigned* wst,
                                                  float& m, unsigned& st_out) {
@@ -368,7 +368,7 @@ __device__ __forceinline__ bool team_reduce_grid(TubeSync* s, float r, unsigned 
         atomicMax(&s->rate[slot], (unsigned long long)__float_as_uint(rb));
         if (sb) atomicOr(&s->stat[slot], sb);
     }
-    if (!team_barrier(s, team, target)) return false;
+    if (!team_barrier(s, team, target, spin)) return false;
     m = __uint_as_float((unsigned)__ldcg(&s->rate[slot]));
     st_out = __ldcg(&s->stat[slot]);
     if (rank == 0 && tid == 0) {
@@ -412,7 +412,8 @@ __device__ void tubes_mixed_body(const TubeMixedArgs& a, const ParamsT<float>& p
     // the team's CFL maximum and status bits; false if the team's barrier gave up
     auto reduce = [&](float r, unsigned st, float& m, unsigned& st_out) {
         if (grid)
-            return team_reduce_grid<NT>(sy, r, st, epoch, target, rank, team, wred, wst, m, st_out);
+            return team_reduce_grid<NT>(sy, a.spin, r, st, epoch, target, rank, team, wred, wst, m,
+                                        st_out);
         team_reduce<NT>(r, st, epoch, r_red, r_stat, rank, s_red, s_stat, wred, wst, &s_m, &s_st,
                         m, st_out);
         return true;
@@ -495,7 +496,7 @@ __device__ void tubes_mixed_body(const TubeMixedArgs& a, const ParamsT<float>& p
                 tube_stage_m<PH, NT, RUS>(a, v, mp, Wc, nullptr, Wn, (float)(0.5 * dt), false, false,
                                      rank, team, sm, status, nflag);
                 if (grid) {
-                    if (!(ok = team_barrier(sy, team, target))) break;
+                    if (!(ok = team_barrier(sy, team, target, a.spin))) break;
                 } else {
                     cl_sync();
                 }

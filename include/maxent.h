@@ -253,7 +253,8 @@ const char *mxe_last_error(const mxe_ctx *ctx);
  * mxe_get_moments act on the concatenation of all tubes.  The whole batch
  * advances in one persistent launch.  MXE_FP64: a team of thread blocks per
  * tube, as many as the tubes' lengths and the device allow (a cooperative
- * launch; with more tubes than block slots one block per tube).
+ * launch; with more tubes than block slots, or on a stream whose SMs cannot
+ * hold the teams at once, one block per tube).
  * MXE_MIXED (14-moment system): teams of CTAs (thread-block clusters of
  * 1, 2, 4 or 8 CTAs of 128 or 256 threads, see mxe_batch_autotune) take
  * tubes from a device work queue, longest expected work (cells / dx) first;

@@ -102,10 +102,12 @@ struct mxe_ctx {
     // tubes: the teams of the launch, one plan for runs of equal step counts
     // and one for runs to a common time (mixed tubes: while the block shape is
     // the library's own choice; team_ctas[0] == 0 if teams do not pay)
-    TubeTeam* team_d[2] = {nullptr, nullptr};
-    std::vector<TubeTeam> team_h;     // both plans as they are copied to the device
-    int team_ctas[2] = {0, 0}, team_chunk[2] = {63, 63};
-    bool team_coop[2] = {false, false};
+    // FP64, plan 2: one CTA a tube, nothing waits (where the stream has too few SMs for the teams)
+    TubeTeam* team_d[3] = {nullptr, nullptr, nullptr};
+    std::vector<TubeTeam> team_h;     // the plans as they are copied to the device
+    int team_ctas[3] = {0, 0, 0}, team_chunk[3] = {63, 63, 63};
+    bool team_coop[3] = {false, false, false};
+    bool team_refused = false;        // the stream's SMs cannot hold the teams at once
     TubeSync* sync_d = nullptr;
     int spin = TEAM_SPIN_LIMIT;
     int* queue_d = nullptr;           // mixed tubes: work counters of the team and fill launches
@@ -122,7 +124,7 @@ struct mxe_ctx {
     cudaGraphExec_t gexec = nullptr;       // captured [queue reset, persistent launch]
     double g_tend = -1.0;
     int g_steps = -1, g_nt = 0, g_cl = 0;
-    bool g_planar = false, g_set = false;
+    bool g_planar = false, g_set = false, g_refused = false;
     long long g_gen = -1;
     long long gen = 0;                // bumped whenever launch arguments change
     long long known_steps = -1;       // steps on the device clock, where the host knows them (else -1)
@@ -341,7 +343,8 @@ static void team_plan(const mxe_ctx* c, bool to_time, int slots, int small, int 
     }
 }
 
-static mxe_status team_plans(mxe_ctx* c) {
+// slots: CTAs to plan for (0: those of the device)
+static mxe_status team_plans(mxe_ctx* c, int slots) {
     int dev = 0, nsm = 0, per = c->mixed ? 4 : 2;
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
@@ -359,17 +362,19 @@ static mxe_status team_plans(mxe_ctx* c) {
     if (c->mixed && c->ntubes > nsm) return MXE_OK;      // one CTA a tube fills the chip
     // both plans and the barrier slots in one allocation
     std::vector<TubeTeam>& all = c->team_h;
-    for (int k = 0; k < 2; ++k) {
+    all.clear();
+    const int plans = c->mixed ? 2 : 3;
+    for (int k = 0; k < plans; ++k) {
         std::vector<TubeTeam> t;
-        team_plan(c, k == 1, per * nsm, c->mixed ? 120 : 31, c->mixed ? 120 : 63, t,
-                  &c->team_chunk[k], &c->team_coop[k]);
+        team_plan(c, k == 1, k == 2 ? 1 : slots ? slots : per * nsm, c->mixed ? 120 : 31,
+                  c->mixed ? 120 : 63, t, &c->team_chunk[k], &c->team_coop[k]);
         c->team_ctas[k] = (int)t.size();
         all.insert(all.end(), t.begin(), t.end());
     }
-    const size_t slots = sizeof(TubeSync) * c->ntubes;
-    CK(cudaMalloc(&c->sync_d, slots + sizeof(TubeTeam) * all.size()));
-    c->team_d[0] = (TubeTeam*)((char*)c->sync_d + slots);
-    c->team_d[1] = c->team_d[0] + c->team_ctas[0];
+    const size_t sync = sizeof(TubeSync) * c->ntubes;
+    CK(cudaMalloc(&c->sync_d, sync + sizeof(TubeTeam) * all.size()));
+    c->team_d[0] = (TubeTeam*)((char*)c->sync_d + sync);
+    for (int k = 1; k < plans; ++k) c->team_d[k] = c->team_d[k - 1] + c->team_ctas[k - 1];
     CK(cudaMemcpyAsync(c->team_d[0], all.data(), sizeof(TubeTeam) * all.size(),
                        cudaMemcpyHostToDevice, c->own_stream));
     return MXE_OK;
@@ -390,6 +395,18 @@ extern "C" mxe_status mxe_test_team_wait(mxe_ctx* c, int spin, int absent) {
     return MXE_OK;
 }
 
+// For the tests of a refused launch (not part of the API): the plans are made again for
+// `slots` CTAs, whatever the device holds (0: what it holds).
+extern "C" mxe_status mxe_test_team_slots(mxe_ctx* c, int slots) {
+    if (!c || !c->sync_d) return MXE_ESTATE;
+    CK(cudaStreamSynchronize(c->stream));
+    cudaFree(c->sync_d);
+    c->sync_d = nullptr;
+    c->team_refused = false;
+    ++c->gen;
+    return team_plans(c, slots);
+}
+
 // The host arrays that are copied here belong to the context: where the device reads
 // pageable memory itself, such a copy may still be on its way when the call returns.
 //
@@ -404,7 +421,7 @@ static mxe_status tubes_setup(mxe_ctx* c) {
     CK(cudaMemsetAsync(c->tclk, 0, sizeof(TubeClock) * n, c->own_stream));
     CK(cudaMemcpyAsync(c->tdesc_d, c->tdesc.data(), sizeof(TubeDesc) * n, cudaMemcpyHostToDevice,
                        c->own_stream));
-    if (!c->mixed) return team_plans(c);
+    if (!c->mixed) return team_plans(c, 0);
     std::vector<int> order(n);
     for (int b = 0; b < n; ++b) order[b] = b;
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
@@ -429,7 +446,7 @@ static mxe_status tubes_setup(mxe_ctx* c) {
             CK(cudaFuncSetAttribute(tubes_mixed_kernel(pl, nt, c->sp.flux == MXE_FLUX_RUSANOV),
                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)tubes_mixed_smem(pl, nt)));
-    return team_plans(c);
+    return team_plans(c, 0);
 }
 
 extern "C" mxe_status mxe_create(const mxe_config* cfg, mxe_ctx** out) {
@@ -613,6 +630,7 @@ extern "C" mxe_status mxe_set_stream(mxe_ctx* c, void* stream) {
     if (!c) return MXE_EINVAL;
     CK(cudaStreamSynchronize(c->stream));
     c->stream = stream ? (cudaStream_t)stream : c->own_stream;
+    c->team_refused = false;
     return MXE_OK;
 }
 
@@ -1247,7 +1265,7 @@ static mxe_status tube_launch_shape(mxe_ctx* c, int nt, int cl, TubeLaunch* L,
 static mxe_status tube_launch(mxe_ctx* c, bool to_time, TubeLaunch* L,
                               const std::vector<double>* est) {
     const int k = to_time ? 1 : 0;
-    if (c->shape_set || c->team_ctas[k] == 0)
+    if (c->shape_set || c->team_ctas[k] == 0 || c->team_refused)
         return tube_launch_shape(c, c->tune_nt, c->tune_cl, L, est);
     const bool pl = tubes_planar(c);
     L->kern = tubes_mixed_kernel(pl, 128, c->sp.flux == MXE_FLUX_RUSANOV);
@@ -1286,6 +1304,18 @@ static cudaError_t launch_tube_grid(cudaStream_t st, const TubeLaunch& L, int cl
     return cudaLaunchKernelExC(&lc, L.kern, args);
 }
 
+// A team launch's CTAs have to be resident at once.  The plans are made for the whole device;
+// a stream may have fewer SMs (a green context's), and then the launch is refused: tubes are
+// marched without teams until the context is given another stream.
+static mxe_status launch_refused(mxe_ctx* c, cudaError_t e) {
+    if (e == cudaErrorCooperativeLaunchTooLarge) {
+        c->team_refused = true;
+        cudaGetLastError();
+    }
+    return e == cudaSuccess ? MXE_OK
+                            : fail(c, MXE_ECUDA, "tube launch: %s", cudaGetErrorString(e));
+}
+
 // Queue reset + the persistent team launch on `st`, and the fill launch on
 // the fill stream, forked after the reset and joined back into `st` (runtime
 // calls that can be captured into a graph).  The two launches share no data
@@ -1303,8 +1333,8 @@ static mxe_status launch_tubes_mixed(mxe_ctx* c, cudaStream_t st, const TubeMixe
         at.sync = c->sync_d;
         at.spin = c->spin;
         CK(cudaMemsetAsync(c->sync_d, 0, sizeof(TubeSync) * c->ntubes, st));
-        CK(launch_tube_grid(st, L, 1, c->team_ctas[L.plan], at, p, mp, c->team_coop[L.plan]));
-        return MXE_OK;
+        return launch_refused(
+            c, launch_tube_grid(st, L, 1, c->team_ctas[L.plan], at, p, mp, c->team_coop[L.plan]));
     }
     CK(cudaMemsetAsync(c->queue_d, 0, 2 * sizeof(int), st));
     if (L.fill > 0) {
@@ -1329,7 +1359,7 @@ static mxe_status launch_tubes_mixed(mxe_ctx* c, cudaStream_t st, const TubeMixe
 // Run through the cached CUDA graph [queue reset, persistent launch]; the
 // graph is captured again when t_end, max_steps, the block shape or any
 // launch argument changed.
-static mxe_status run_tubes_mixed(mxe_ctx* c, int max_steps, double t_end, const double* dts,
+static mxe_status try_tubes_mixed(mxe_ctx* c, int max_steps, double t_end, const double* dts,
                                   int ndts) {
     TubeLaunch L;
     std::vector<double> est;
@@ -1346,7 +1376,7 @@ static mxe_status run_tubes_mixed(mxe_ctx* c, int max_steps, double t_end, const
     }
     if (!c->gexec || c->g_tend != t_end || c->g_steps != max_steps || c->g_nt != c->tune_nt ||
         c->g_cl != c->tune_cl || c->g_set != c->shape_set || c->g_gen != c->gen ||
-        c->g_planar != tubes_planar(c)) {
+        c->g_refused != c->team_refused || c->g_planar != tubes_planar(c)) {
         if (c->gexec) {
             cudaGraphExecDestroy(c->gexec);
             c->gexec = nullptr;
@@ -1363,6 +1393,7 @@ static mxe_status run_tubes_mixed(mxe_ctx* c, int max_steps, double t_end, const
         cudaError_t e = cudaStreamEndCapture(c->cap_stream, &g);
         if (s != MXE_OK) {
             if (g) cudaGraphDestroy(g);
+            cudaGetLastError();
             return s;
         }
         if (e != cudaSuccess) return fail(c, MXE_ECUDA, "graph capture: %s", cudaGetErrorString(e));
@@ -1370,6 +1401,7 @@ static mxe_status run_tubes_mixed(mxe_ctx* c, int max_steps, double t_end, const
         cudaGraphDestroy(g);
         if (e != cudaSuccess) {
             c->gexec = nullptr;
+            launch_refused(c, e);
             return fail(c, MXE_ECUDA, "graph instantiate: %s", cudaGetErrorString(e));
         }
         c->g_tend = t_end;
@@ -1377,17 +1409,28 @@ static mxe_status run_tubes_mixed(mxe_ctx* c, int max_steps, double t_end, const
         c->g_nt = c->tune_nt;
         c->g_cl = c->tune_cl;
         c->g_set = c->shape_set;
+        c->g_refused = c->team_refused;
         c->g_gen = c->gen;
         c->g_planar = tubes_planar(c);
         c->g_lay_teams = c->lay_teams;
         c->g_lay_nA = c->lay_nA;
         c->g_lay_fill = c->lay_fill;
     }
-    CK(cudaGraphLaunch(c->gexec, c->stream));
+    s = launch_refused(c, cudaGraphLaunch(c->gexec, c->stream));
+    if (s != MXE_OK) return s;
     c->lay_teams = c->g_lay_teams;
     c->lay_nA = c->g_lay_nA;
     c->lay_fill = c->g_lay_fill;
     return MXE_OK;
+}
+
+static mxe_status run_tubes_mixed(mxe_ctx* c, int max_steps, double t_end, const double* dts,
+                                  int ndts) {
+    const bool refused = c->team_refused;
+    mxe_status s = try_tubes_mixed(c, max_steps, t_end, dts, ndts);
+    if (s != MXE_OK && c->team_refused && !refused)       // teams refused just now
+        s = try_tubes_mixed(c, max_steps, t_end, dts, ndts);
+    return s;
 }
 
 static mxe_status run_tubes(mxe_ctx* c, int max_steps, double t_end, const double* dts,
@@ -1416,14 +1459,20 @@ static mxe_status run_tubes(mxe_ctx* c, int max_steps, double t_end, const doubl
         a.n_fixed = ndts;
         a.max_steps = ndts;
     }
-    const int k = dts || !std::isfinite(t_end) ? 0 : 1;
-    a.teams = c->team_d[k];
     a.sync = c->sync_d;
     a.spin = c->spin;
     CK(cudaMemsetAsync(c->sync_d, 0, sizeof(TubeSync) * c->ntubes, c->stream));
-    CK(launch_tubes_f64(tubes_f64_kernel(c->nf, tubes_planar(c), c->team_chunk[k]),
-                        c->team_ctas[k], c->team_coop[k], a, c->stream));
-    return MXE_OK;
+    auto launch = [&](int k) {
+        a.teams = c->team_d[k];
+        return launch_refused(
+            c, launch_tubes_f64(tubes_f64_kernel(c->nf, tubes_planar(c), c->team_chunk[k]),
+                                c->team_ctas[k], c->team_coop[k], a, c->stream));
+    };
+    if (!c->team_refused) {
+        const mxe_status s = launch(dts || !std::isfinite(t_end) ? 0 : 1);
+        if (!c->team_refused) return s;
+    }
+    return launch(2);
 }
 
 static mxe_status tube_status(mxe_ctx* c, double* t0, long long* steps0) {

@@ -178,9 +178,13 @@ extern "C" mxe_status mxe_tube_run_noalloc(const mxe_config* cfg, int bc_lo, int
         const int ch = (cfg->nx + 62) / 63, pass = (ch + p.slots - 1) / p.slots;
         ctas = (ch + pass - 1) / pass;
     }
-    if (launch_tubes_f64(tubes_f64_kernel(cfg->system, false, chunk), ctas, ctas > 1, a, st) !=
-        cudaSuccess)
-        return MXE_ECUDA;
+    cudaError_t e =
+        launch_tubes_f64(tubes_f64_kernel(cfg->system, false, chunk), ctas, ctas > 1, a, st);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {       // a stream of fewer SMs: one CTA alone
+        cudaGetLastError();
+        e = launch_tubes_f64(tubes_f64_kernel(cfg->system, false, 63), 1, false, a, st);
+    }
+    if (e != cudaSuccess) return MXE_ECUDA;
     if (t_out || steps_out) {
         if (cudaMemcpyAsync(&ck, p.clock, sizeof ck, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
             cudaStreamSynchronize(st) != cudaSuccess)

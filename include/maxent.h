@@ -291,9 +291,11 @@ mxe_status mxe_batch_run(mxe_ctx *ctx, int max_steps, double t_end);
 /* MXE_MIXED tube contexts: time every block shape (128 or 256 threads per
  * CTA x teams of 1, 2, 4 or 8 CTAs) on the current state advanced by t_probe
  * (each candidate from the same saved state and clocks, which are restored
- * afterwards) and keep the fastest for later runs.  Shapes that cannot be
- * resident on the device are skipped.  Outputs (may be NULL): the chosen
- * threads per CTA, CTAs per team and its time in ms.  Allocates (and frees)
+ * afterwards), and the library's own teams of few tubes (mxe_batch_create),
+ * and keep the fastest for later runs.  Shapes that cannot be
+ * resident on the device are skipped.  Outputs (may be NULL): the fastest
+ * shape's threads per CTA and CTAs per team, and the time in ms of what is
+ * kept, that shape or the library's teams.  Allocates (and frees)
  * one temporary copy of the state; synchronises the context stream.
  * Errors: MXE_ESTATE (not an MXE_MIXED 1D context, or no state),
  * MXE_EINVAL (t_probe <= 0), MXE_ECUDA. */

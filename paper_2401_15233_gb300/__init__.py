@@ -563,8 +563,9 @@ class Batch(Solver):
         mxe_batch_run(self.ctx, max_steps, t_end)
 
     def autotune(self, t_probe):
-        """Time every block shape over t_probe (state restored); returns
-        (threads per CTA, CTAs per team, ms of the fastest)."""
+        """Time every block shape, and the library's teams of few tubes, over t_probe (state
+        restored) and keep the fastest; returns (threads per CTA and CTAs per team of the
+        fastest shape, ms of what is kept)."""
         return mxe_batch_autotune(self.ctx, t_probe)
 
     def set_shape(self, nt, cl):

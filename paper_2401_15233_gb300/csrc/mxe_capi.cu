@@ -117,7 +117,6 @@ struct mxe_ctx {
     int lay_teams = 0, lay_nA = 0, lay_fill = 0;   // layout of the last mixed tube launch
     int g_lay_teams = 0, g_lay_nA = 0, g_lay_fill = 0;   // layout captured in the graph
     int tune_nt = 128, tune_cl = 1;   // block shape of the mixed tube launch
-    bool tuned = false;
     bool shape_set = false;           // the caller chose a block shape (or had it tuned)
     int nsm = 0;
     cudaStream_t cap_stream = nullptr;     // graph capture only (never executes work)
@@ -1260,13 +1259,8 @@ static mxe_status tube_launch_shape(mxe_ctx* c, int nt, int cl, TubeLaunch* L,
     return MXE_OK;
 }
 
-// Launch of a run: the caller's block shape, or while there is none teams
-// across the chip where the tubes are few enough.
-static mxe_status tube_launch(mxe_ctx* c, bool to_time, TubeLaunch* L,
-                              const std::vector<double>* est) {
-    const int k = to_time ? 1 : 0;
-    if (c->shape_set || c->team_ctas[k] == 0 || c->team_refused)
-        return tube_launch_shape(c, c->tune_nt, c->tune_cl, L, est);
+// Teams across the chip, by plan k
+static void tube_launch_teams(const mxe_ctx* c, int k, TubeLaunch* L) {
     const bool pl = tubes_planar(c);
     L->kern = tubes_mixed_kernel(pl, 128, c->sp.flux == MXE_FLUX_RUSANOV);
     L->smem = tubes_mixed_smem(pl, 128);
@@ -1275,6 +1269,16 @@ static mxe_status tube_launch(mxe_ctx* c, bool to_time, TubeLaunch* L,
     L->teams = L->nA = c->ntubes;
     L->fill = 0;
     L->plan = k;
+}
+
+// Launch of a run: the caller's block shape, or while there is none teams
+// across the chip where the tubes are few enough.
+static mxe_status tube_launch(mxe_ctx* c, bool to_time, TubeLaunch* L,
+                              const std::vector<double>* est) {
+    const int k = to_time ? 1 : 0;
+    if (c->shape_set || c->team_ctas[k] == 0 || c->team_refused)
+        return tube_launch_shape(c, c->tune_nt, c->tune_cl, L, est);
+    tube_launch_teams(c, k, L);
     return MXE_OK;
 }
 
@@ -1680,37 +1684,43 @@ extern "C" mxe_status mxe_batch_autotune(mxe_ctx* c, double t_probe, int* nt_out
     if (e == cudaSuccess && tube_steps(c, 1 << 30, t0 + t_probe, 0, est) != MXE_OK)
         e = cudaErrorUnknown;
     const int nts[2] = {128, 256}, cls[4] = {1, 2, 4, 8};
-    float best = INFINITY;
+    float best = INFINITY, own = INFINITY;      // of the shapes; of the library's teams
     int bnt = c->tune_nt, bcl = c->tune_cl;
-    for (int i = 0; i < 2 && e == cudaSuccess; ++i)
-        for (int j = 0; j < 4 && e == cudaSuccess; ++j) {
-            TubeLaunch L;
-            if (tube_launch_shape(c, nts[i], cls[j], &L, &est) != MXE_OK) {
-                cudaGetLastError();
-                continue;                       // shape does not fit on this device
-            }
-            e = cudaMemcpyAsync(c->U, Usave, sizeof(double) * c->nelem, cudaMemcpyDeviceToDevice,
-                                c->stream);
-            if (e == cudaSuccess)
-                e = cudaMemcpyAsync(c->tclk, ck.data(), sizeof(TubeClock) * c->ntubes,
-                                    cudaMemcpyHostToDevice, c->stream);
-            if (e == cudaSuccess) e = cudaEventRecord(e0, c->stream);
-            if (e != cudaSuccess) break;
-            TubeMixedArgs a = tubes_mixed_args(c, 1 << 30, t0 + t_probe);
-            if (launch_tubes_mixed(c, c->stream, a, L) != MXE_OK) {
-                cudaGetLastError();
-                continue;
-            }
-            e = cudaEventRecord(e1, c->stream);
-            if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-            float ms = 0.0f;
-            if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-            if (e == cudaSuccess && ms < best) {
-                best = ms;
-                bnt = nts[i];
-                bcl = cls[j];
-            }
+    const int first = c->team_ctas[1] > 0 && !c->team_refused ? -1 : 0;
+    for (int n = first - 1; n < 8 && e == cudaSuccess; ++n) {
+        const int i = std::max(n, first);        // the first one twice: its code may not be loaded
+        TubeLaunch L;
+        if (i < 0) {
+            tube_launch_teams(c, 1, &L);
+        } else if (tube_launch_shape(c, nts[i / 4], cls[i % 4], &L, &est) != MXE_OK) {
+            cudaGetLastError();
+            continue;                           // shape does not fit on this device
         }
+        e = cudaMemcpyAsync(c->U, Usave, sizeof(double) * c->nelem, cudaMemcpyDeviceToDevice,
+                            c->stream);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(c->tclk, ck.data(), sizeof(TubeClock) * c->ntubes,
+                                cudaMemcpyHostToDevice, c->stream);
+        if (e == cudaSuccess) e = cudaEventRecord(e0, c->stream);
+        if (e != cudaSuccess) break;
+        TubeMixedArgs a = tubes_mixed_args(c, 1 << 30, t0 + t_probe);
+        if (launch_tubes_mixed(c, c->stream, a, L) != MXE_OK) {
+            cudaGetLastError();
+            continue;
+        }
+        e = cudaEventRecord(e1, c->stream);
+        if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+        float ms = 0.0f;
+        if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+        if (e != cudaSuccess) break;
+        if (i < 0) {
+            own = std::min(own, ms);
+        } else if (ms < best) {
+            best = ms;
+            bnt = nts[i / 4];
+            bcl = cls[i % 4];
+        }
+    }
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(c->U, Usave, sizeof(double) * c->nelem, cudaMemcpyDeviceToDevice,
                             c->stream);
@@ -1725,11 +1735,11 @@ extern "C" mxe_status mxe_batch_autotune(mxe_ctx* c, double t_probe, int* nt_out
     if (!(best < INFINITY)) return fail(c, MXE_ECUDA, "autotune: no block shape could be launched");
     c->tune_nt = bnt;
     c->tune_cl = bcl;
-    c->tuned = c->shape_set = true;
+    c->shape_set = best < own;       // else the library's teams stay
     c->lay_nA = 0;                   // the layout of the next launch is not known yet
     if (nt_out) *nt_out = bnt;
     if (cl_out) *cl_out = bcl;
-    if (ms_out) *ms_out = best;
+    if (ms_out) *ms_out = std::min(best, own);
     return MXE_OK;
 }
 

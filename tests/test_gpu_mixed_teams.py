@@ -77,3 +77,32 @@ def test_single_tube_to_a_time_and_prescribed_steps(mx):
         s.step_dt([1e-5, 2e-5, 1e-5])
         got.append(s.get_moments("conserved").reshape(-1))
     assert np.array_equal(*got)
+
+
+@pytest.mark.parametrize("sizes", [[8192], [700] * 9])
+def test_autotune_keeps_the_teams_where_they_are_faster(mx, sizes):
+    """A tuned batch of few tubes is no slower than an untuned one (measured: the teams of one
+    8192-cell tube take under a tenth of the best shape's time)."""
+    import time
+    b = mx.Batch(sizes, [1.0] * len(sizes), precision="mixed")
+    prims = [_prim(n, n, True) for n in sizes]
+    state = b.pack(prims)
+
+    def ms():
+        best = np.inf
+        for _ in range(5):
+            b.set_state(state)
+            t = time.perf_counter()
+            b.run(400, float("inf"))
+            b.clock()
+            best = min(best, time.perf_counter() - t)
+        return 1e3 * best
+
+    own = ms()
+    b.set_state(state)
+    nt, cl, kept = b.autotune(1e-3)
+    tuned = ms()
+    assert nt in (128, 256) and cl in (1, 2, 4, 8) and kept > 0
+    assert tuned <= 1.5 * own
+    b.set_shape(nt, cl)                         # and a chosen shape still counts
+    assert ms() > 1.5 * own or len(sizes) > 1

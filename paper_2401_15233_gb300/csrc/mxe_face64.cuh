@@ -506,7 +506,7 @@ __device__ __forceinline__ void source_14(const double* Q, double p, double it, 
 // =========================================================================
 // shared limiter (Sec. 3.2) and reconstruction
 // =========================================================================
-// phi = min_k phi_k over the fields that are not flat (phi_accumulate).  The
+// phi = min_k phi_k over the fields that are not flat.  The
 // fields that cannot set phi are ruled out in FP32: r_k = min / max of
 // |dm|, |dp| (their common exponent removed first, so that no magnitude is out
 // of range) orders the fields as phi_k does, and a field clearly inside or

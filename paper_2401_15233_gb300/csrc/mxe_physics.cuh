@@ -144,127 +144,10 @@ __device__ __forceinline__ void cons2prim5_rn(const double* U, double* Q) {
     Q[0] = rho; Q[1] = u; Q[2] = P; Q[3] = q; Q[4] = r;
 }
 
-// Baradaran fit, Eq. (ws-max-baradaran-orig), with shared E, C, Y.
-template <class T>
-__device__ __forceinline__ T lam5_star(T qs, T sb, T E, T C, T Y) {
-    T D0 = T(-0.8) * qs * sb * C + T(4) * sb * sb * Y;
-    return hyp_bracket(qs, D0) / (T(2) * sb) + E;
-}
-
-// Primitive moments of cons5(W) + dU from the increment alone (FP32 path;
-// every term scales with the increment, see prim_increment14).
-__device__ __forceinline__ void prim_increment5(const float* W, const float* dU, float* Wn) {
-    float rho = W[0], u = W[1], P = W[2], q = W[3];
-    float drho = dU[0];
-    float rho1 = rho + drho;
-    float du = (dU[1] - u * drho) / rho1;
-    float u1 = u + du;
-    float dP = dU[2] - drho * u * u - rho1 * (2.0f * u * du + du * du);
-    float P1 = P + dP;
-    float s = 2.0f * u * du + du * du;                      // u1^2 - u^2
-    // G = rho u^3 + 3 u P
-    float dG = drho * u * u * u + rho1 * du * (3.0f * u * u + 3.0f * u * du + du * du)
-             + 3.0f * (du * P1 + u * dP);
-    float dq = dU[3] - dG;
-    float q1 = q + dq;
-    // K = rho u^4 + 6 u^2 P + 4 u q
-    float dK = drho * u * u * u * u + rho1 * s * (2.0f * u * u + s) + 6.0f * (s * P1 + u * u * dP)
-             + 4.0f * (du * q1 + u * dq);
-    Wn[0] = rho1; Wn[1] = u1; Wn[2] = P1; Wn[3] = q1;
-    Wn[4] = W[4] + (dU[4] - dK);
-}
-
 // Raw sigma of Eq. (sigma-mapping-5mom) from the dimensionless q*, r*.
 template <class T>
 __device__ __forceinline__ T sigma5(T qs, T rs) {
     return sigma_root(T(3) - rs, T(8) * qs * qs, T(1));
-}
-
-// Face-state evaluation: conserved U, x-flux F (Eq. 5mom-sys-eqs with the
-// closure of Eq. closure-1D1V-s-approx) and wave speeds.
-template <class T>
-__device__ __forceinline__ void face_eval5(const T* Q, T sigma_lim, T k_ws, T* U, T* F,
-                                           T& lmin, T& lmax) {
-    T rho = Q[0], u = Q[1], P = Q[2], q = Q[3], r = Q[4];
-    T th = P / rho;
-    T sq = M<T>::sqrt_(th);
-    T sc3 = rho * th * sq;
-    T qs = q / sc3;
-    T rs = r / (rho * th * th);
-    T sb = clamp_sigma(sigma5(qs, rs), sigma_lim);
-    T ssb = M<T>::sqrt_(sb);
-    T ss = qs * qs * qs / (sb * sb) + (T(10) - T(8) * ssb) * qs;
-    T s = ss * sc3 * th;
-    prim2cons5(Q, U);
-    F[0] = rho * u;
-    F[1] = rho * u * u + P;
-    F[2] = rho * u * u * u + T(3) * u * P + q;
-    F[3] = rho * u * u * u * u + T(6) * u * u * P + T(4) * u * q + r;
-    F[4] = rho * u * u * u * u * u + T(10) * u * u * u * P + T(10) * u * u * q + T(5) * u * r + s;
-    T C = M<T>::sqrt_(T(3) - T(3) * sb);
-    T E = T(0.8) * C;
-    T B, Y;
-    WsTerms<T>::get(ssb, sb, E, B, Y);
-    lmax = u + k_ws * lam5_star(qs, sb, E, C, Y) * sq;
-    lmin = u - k_ws * lam5_star(-qs, sb, E, C, Y) * sq;
-}
-
-template <class T>
-__device__ __forceinline__ void face_eval5(const T* Q, const SchemeParams& sp, T* U, T* F,
-                                           T& lmin, T& lmax) {
-    T rho = Q[0], u = Q[1], P = Q[2], q = Q[3], r = Q[4];
-    T th = P / rho;
-    T sq = M<T>::sqrt_(th);
-    T sc3 = rho * th * sq;
-    T qs = q / sc3;
-    T rs = r / (rho * th * th);
-    T sb = clamp_sigma(sigma5(qs, rs), T(sp.sigma_lim));
-    T ssb = M<T>::sqrt_(sb);
-    T ss = qs * qs * qs / (sb * sb) + (T(10) - T(8) * ssb) * qs;
-    T s = ss * sc3 * th;
-    prim2cons5(Q, U);
-    F[0] = rho * u;
-    F[1] = rho * u * u + P;
-    F[2] = rho * u * u * u + T(3) * u * P + q;
-    F[3] = rho * u * u * u * u + T(6) * u * u * P + T(4) * u * q + r;
-    F[4] = rho * u * u * u * u * u + T(10) * u * u * u * P + T(10) * u * u * q + T(5) * u * r + s;
-    T C = M<T>::sqrt_(T(3) - T(3) * sb);
-    T E = T(0.8) * C;
-    T B = T(5) - T(4) * ssb + M<T>::sqrt_(T(10) - T(16) * ssb + T(6) * sb);
-    T Y = B + E * E - T(2) * E * M<T>::sqrt_(B);
-    T k = T(sp.k_ws);
-    lmax = u + k * lam5_star(qs, sb, E, C, Y) * sq;
-    lmin = u - k * lam5_star(-qs, sb, E, C, Y) * sq;
-}
-
-template <class T>
-__device__ __forceinline__ void rate5(const T* Q, const SchemeParams& sp, T& amax, T& sig_raw) {
-    T rho = Q[0], u = Q[1], P = Q[2], q = Q[3], r = Q[4];
-    T th = P / rho;
-    T sq = M<T>::sqrt_(th);
-    T qs = q / (rho * th * sq);
-    T rs = r / (rho * th * th);
-    sig_raw = sigma5(qs, rs);
-    T sb = clamp_sigma(sig_raw, T(sp.sigma_lim));
-    T ssb = M<T>::sqrt_(sb);
-    T C = M<T>::sqrt_(T(3) - T(3) * sb);
-    T E = T(0.8) * C;
-    T B = T(5) - T(4) * ssb + M<T>::sqrt_(T(10) - T(16) * ssb + T(6) * sb);
-    T Y = B + E * E - T(2) * E * M<T>::sqrt_(B);
-    T k = T(sp.k_ws);
-    T lmax = u + k * lam5_star(qs, sb, E, C, Y) * sq;
-    T lmin = u - k * lam5_star(-qs, sb, E, C, Y) * sq;
-    T a = fabs(lmin), b = fabs(lmax);
-    amax = a > b ? a : b;
-}
-
-// BGK source of Eq. (5mom-sys-eqs).
-template <class T>
-__device__ __forceinline__ void source5(const T* Q, T tau, T* C) {
-    T rho = Q[0], u = Q[1], P = Q[2], q = Q[3], r = Q[4];
-    C[0] = T(0); C[1] = T(0); C[2] = T(0);
-    C[3] = -q / tau;
-    C[4] = -(T(4) * u * q + r - T(3) * P * P / rho) / tau;
 }
 
 // =========================================================================
@@ -615,11 +498,6 @@ __device__ __forceinline__ T amax14(const T* Q, const Dimless14<T>& d, T sigma_l
     return a > b ? a : b;
 }
 
-template <class T, int K>
-__device__ __forceinline__ T amax14(const T* Q, const Dimless14<T>& d, const SchemeParams& sp) {
-    return amax14<T, K>(Q, d, T(sp.sigma_lim), T(sp.k_ws));
-}
-
 // Primitive moments of cons(W) + dU from the increment alone (FP32 path):
 // every term below is proportional to the increment, so nothing of the size
 // of the bulk-motion contributions (rho u^4 against R at high Mach number)
@@ -699,13 +577,6 @@ __device__ __forceinline__ void source14(const T* Q, T tau, T* C) {
     T uq = ux * Q[10] + uy * Q[11] + uz * Q[12];
     T u2 = ux * ux + uy * uy + uz * uz;
     C[13] = -((T(4) * uPu + T(4) * uq + Q[13]) - (T(4) * u2 * p + T(15) * p * p / rho)) / tau;
-}
-
-template <class T>
-__device__ __forceinline__ T tau_of(const RelaxParams& rp, const T* Q, int system) {
-    if (rp.model == 1) return T(rp.tau_ref);
-    T Tt = system == 5 ? Q[2] / Q[0] : (Q[4] + Q[7] + Q[9]) / (T(3) * Q[0]);
-    return T(rp.tau_ref) * (T(rp.rho_ref) / Q[0]) * M<T>::sqrt_(T(rp.T_ref) / Tt);
 }
 
 // ---------------------------------------------------------------- point-implicit BGK
@@ -863,25 +734,6 @@ __device__ __forceinline__ T phi_field(T dm, T dp, int lim) {
         return mn / mul_rn(T(0.5), add_rn(am, ap));
     }
     return (dm == T(0) && dp == T(0)) ? T(1) : T(0);
-}
-
-// phi = min(phi, phi_k) for field k (compile-time index) of the stencil
-// centred on the cell fr.  A flat field has phi_k = 1, which never lowers
-// phi, so the flat test runs only where phi_k without it would: the result
-// is the min over all fields either way.
-template <int NF, class T>
-__device__ __forceinline__ void phi_accumulate(T& phi, T dm, T dp, int lim, const FlatRef<T>& fr,
-                                               int k) {
-    const T pk = phi_field(dm, dp, lim);
-    if (pk < phi && !field_flat<NF>(fr, k, abs_max(dm, dp))) phi = pk;
-}
-
-// MUSCL face value Q0 + sgn/2 (phi c) with the central difference
-// c = ((Q0 - Qm) + (Qp - Q0))/2, explicitly rounded.
-template <class T>
-__device__ __forceinline__ T muscl_face(T qm, T q0, T qp, T phi, T half_sgn) {
-    T cen = mul_rn(T(0.5), add_rn(sub_rn(q0, qm), sub_rn(qp, q0)));
-    return add_rn(q0, mul_rn(half_sgn, mul_rn(phi, cen)));
 }
 
 }  // namespace mxe

@@ -113,6 +113,28 @@ __device__ __forceinline__ void load_w(const TubeMixedArgs& a, const float* Wt, 
     for (int k = 0; k < PH::NF; ++k) Q[k] = __ldcg(Wt + (long long)k * n + gi);
 }
 
+// One face state of the general system (face_state_m), out of line: one function for all kernels
+// of this file.  Compiled into each by itself, its scalar arithmetic was contracted into
+// fused multiply-adds in another way for 128 threads than for 256, and a run's result
+// depended on the block shape.  Arguments and result by value, so that the caller's
+// arrays stay in registers.
+template <class PH>
+struct FaceState {
+    float v[2 * PH::NF + 2];
+    bool flag;
+};
+template <class PH>
+static __device__ __noinline__ FaceState<PH> face_state_1d(FaceIn<PH::NF> in, float sigma_lim,
+                                                           float k_ws, MixedPolicy mp, double sl64,
+                                                           double kw64) {
+    ParamsT<float> p;
+    p.sigma_lim = sigma_lim;
+    p.k_ws = k_ws;
+    FaceState<PH> r;
+    r.flag = face_state_m<PH, 0>(in.q, p, mp, sl64, kw64, r.v);
+    return r;
+}
+
 // Face flux of the face between box cells cl and cl + 1; the left face state
 // is staged in this lane's column of Ls.
 template <class PH, int BOX>
@@ -122,22 +144,27 @@ __device__ __forceinline__ void face_flux_1d(const float* W, int cl, float phl, 
                                              unsigned& nflag) {
     constexpr int NF = PH::NF;
     constexpr int FS = 2 * NF + 2;
-    float Qf[NF], R[FS], Lv[FS];
     const int cr = cl + 1;
+    FaceIn<NF> Q;
 #pragma unroll
     for (int k = 0; k < NF; ++k) {
         const float* w = W + k * BOX + cl;
-        Qf[k] = w[0] + (0.5f * phl) * (0.5f * (w[1] - w[-1]));
+        Q.q[k] = w[0] + (0.5f * phl) * (0.5f * (w[1] - w[-1]));
     }
-    nflag += face_state_m<PH, 0>(Qf, p, mp, sl64, kw64, Lv) ? 1u : 0u;
+    {
+        const FaceState<PH> L = face_state_1d<PH>(Q, p.sigma_lim, p.k_ws, mp, sl64, kw64);
+        nflag += L.flag ? 1u : 0u;
 #pragma unroll
-    for (int n = 0; n < FS; ++n) Ls[n * 32] = Lv[n];
+        for (int n = 0; n < FS; ++n) Ls[n * 32] = L.v[n];
+    }
 #pragma unroll
     for (int k = 0; k < NF; ++k) {
         const float* w = W + k * BOX + cr;
-        Qf[k] = w[0] - (0.5f * phr) * (0.5f * (w[1] - w[-1]));
+        Q.q[k] = w[0] - (0.5f * phr) * (0.5f * (w[1] - w[-1]));
     }
-    nflag += face_state_m<PH, 0>(Qf, p, mp, sl64, kw64, R) ? 1u : 0u;
+    const FaceState<PH> Rs = face_state_1d<PH>(Q, p.sigma_lim, p.k_ws, mp, sl64, kw64);
+    nflag += Rs.flag ? 1u : 0u;
+    const float* R = Rs.v;
     float lminL = Ls[(2 * NF) * 32], lmaxL = Ls[(2 * NF + 1) * 32];
     float lminR = R[2 * NF], lmaxR = R[2 * NF + 1];
     if (p.flux == 1) {

@@ -106,3 +106,20 @@ def test_autotune_keeps_the_teams_where_they_are_faster(mx, sizes):
     assert tuned <= 1.5 * own
     b.set_shape(nt, cl)                         # and a chosen shape still counts
     assert ms() > 1.5 * own or len(sizes) > 1
+
+
+# a warp's chunk is 30 cells, a CTA's pass 120: the edges of both, and of one CTA and two
+@pytest.mark.parametrize("sizes", [[29], [30], [31], [60, 61], [119], [120], [121], [240, 241, 59]])
+@pytest.mark.parametrize("planar", [True, False])
+@pytest.mark.parametrize("integ,bc", [("rk2", "transmissive"), ("fe", "periodic")])
+def test_chunk_edges(mx, sizes, planar, integ, bc):
+    prims = [_prim(n, n, planar) for n in sizes]
+    out = []
+    for shape in (None, (128, 1), (256, 2)):
+        b = mx.Batch(sizes, [1.0] * len(sizes), precision="mixed", integrator=integ)
+        if shape:
+            b.set_shape(*shape)
+        out.append(_march(b, prims, bc, (17, 2), mx))
+    for got in out[1:]:
+        for n, x, y in zip(sizes, out[0], got):
+            assert np.array_equal(x, y), n

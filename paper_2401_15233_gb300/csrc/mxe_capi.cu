@@ -521,7 +521,7 @@ extern "C" mxe_status mxe_create(const mxe_config* cfg, mxe_ctx** out) {
             e = cudaFuncSetAttribute(mxe_stage14_2d_mixed_planar_b3,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)stage14_2d_mixed_smem(true, 3));
-        for (int n = 0; n < 12 && e == cudaSuccess && c->mixed; ++n) {
+        for (int n = 0; n < 16 && e == cudaSuccess && c->mixed; ++n) {
             const MixedTile f = mixed_tile_kernel(n & 1, n & 2, n >> 2);
             e = cudaFuncSetAttribute(f.kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)f.smem);
@@ -963,33 +963,42 @@ static F64Tile f64_tile(const mxe_ctx* c, bool pl) {
     return best;
 }
 
-// Tile of the packed mixed stage.  Time of an RK2 step on GB300 (152 SMs), us:
-//            48 x 48  130 x 130  200 x 200  300 x 300  400 x 400  512 x 512  1024 x 1024
-//   31 x 18     34        35         35         43         43         72         213
-//   31 x  7     22        21         26         33         47         76         254
-//   15 x  7     19        21         28         40         67        102         371
-// (one tile before: 33 on 48 x 48, 262 on 1024 x 1024); general states:
-//   31 x 15     38        38         39         51         70         87         316
-//   31 x  7     27        27         31         42         64        102         351
-//   15 x  7     21        25         33         51         88        137         535
-// (scalar faces before: 35 on 48 x 48, 92 on 400 x 400).  Small grids pay for the
-// passes of one block, then for each block; the large tiles come two to an SM,
-// in waves.
+// Tile of the packed mixed stage.  Time of an RK2 step on GB300 (152 SMs), us, planar states:
+//            48 x 48  130 x 130  200 x 200  300 x 300  450 x 450  500 x 500  550 x 550  1024 x 1024
+//   31 x 18     32.5       33.1       33.0       43.6       64.0       77.2       78.7        228
+//   31 x 15     30.2       31.1       31.1       43.7       56.3       70.9       85.9        254
+//   31 x  7     18.6       18.7       23.2       34.7       64.3       78.5       85.8        270
+//   15 x  7     16.5       18.7       29.2       42.0       85.1      106.1      121.2        406
+// (the one tile there was, 31 x 15 with the wave speeds last: 32, 33, 33, 44, 58, 73, 88 and
+// 258), general states, HLL (Rusanov takes 1.05 to 1.25 times as long):
+//   31 x 15     35.0       36.3       36.3       52.0       75.0       92.9      113.2        335
+//   31 x  7     22.8       22.8       31.1       45.6       87.3      104.6      119.0        381
+//   15 x  7     18.7       22.9       35.4       54.9      112.1      136.2      159.0        549
+// (scalar faces: 34, 36, 46, 59, 109, 131, 155 and 488).  That is at least `first`, and `off`
+// with `wave` per block of the fullest SM: over 28 sizes from 48 x 48 to 1500 x 1500, 64 x 2000
+// and 2600 x 120 the choice is within 2 % of the fastest tile.
 static MixedTile mixed_tile(const mxe_ctx* c, bool pl) {
+    static const struct {
+        double first, off, wave;
+    } t[3][4] = {{{33.0, 11.0, 16.6}, {18.7, 9.0, 7.95}, {16.5, 9.0, 5.75}, {31.0, 11.5, 15.2}},
+                 {{36.0, 12.0, 20.1}, {22.8, 11.5, 11.15}, {18.6, 11.0, 8.0}},
+                 {{39.0, 11.0, 24.8}, {26.8, 9.5, 14.2}, {20.7, 11.0, 10.3}}};
     const bool rus = c->sp.flux == MXE_FLUX_RUSANOV;
-    auto blocks = [&](int n) {
+    const auto& w = t[pl ? 0 : rus ? 2 : 1];
+    MixedTile best{};
+    double cost = 0.0;
+    for (int n = 0; n < (pl ? 4 : 3); ++n) {
         const MixedTile f = mixed_tile_kernel(pl, rus, n);
-        return (double)((c->g.nx + f.tx - 1) / f.tx) * ((c->g.ny + f.ty - 1) / f.ty) * 152.0 /
-               c->nsm;
-    };
-    // us: large tile alone, offset and wave; small tiles alone, offset and block
-    static const double t[2][9] = {{39.5, 8.0, 43.0, 27.0, 18.0, 0.0705, 22.5, 14.0, 0.0465},
-                                   {35.0, 9.0, 34.5, 22.3, 14.0, 0.0523, 20.0, 11.0, 0.0365}};
-    const double* w = t[pl];
-    const double b = blocks(0), p = b <= 152.0 ? w[0] : w[1] + w[2] * std::ceil(b / 304.0);
-    const double m = std::max(w[3], w[4] + w[5] * blocks(1));
-    const double s = std::max(w[6], w[7] + w[8] * blocks(2));
-    return mixed_tile_kernel(pl, rus, p <= m && p <= s ? 0 : m <= s ? 1 : 2);
+        const long long blocks = (long long)((c->g.nx + f.tx - 1) / f.tx) *
+                                 ((c->g.ny + f.ty - 1) / f.ty);
+        const double us = std::max(w[n].first, w[n].off + w[n].wave * (double)((blocks + c->nsm - 1) /
+                                                                               c->nsm));
+        if (n == 0 || us < cost) {
+            cost = us;
+            best = f;
+        }
+    }
+    return best;
 }
 
 // One step of a 2D grid.  ustar (FP64 RK2 only, optional): where stage 1

@@ -460,11 +460,9 @@ mxe_stage14_2d_mixed_planar_b3(const Stage2DArgs a, const ParamsT<float> p,
 //   31 x  7, 128 threads, 4 blocks, 128           3.81
 //   31 x  9, 160 threads, 4 blocks, 96            3.84
 //   31 x 11, 192 threads, 4 blocks, 80            4.21
-// 31 x 18 fits 1024 x 1024 in whole waves better (3.45 ms and 243 us there with
-// the accurate CFL rates; 3.79 ms and 261 us before).  With the limiter in
-// fewer instructions, the box asked for before the step size is known and the
-// items in rows of a warp: 3.00 ms and 216 us (31 x 17: 3.02 and 220, 31 x 19:
-// 3.06 and 228).
+// (taken before the box was asked for ahead of the step size and the items came in
+// rows of a warp; with both, 31 x 18: 3.21 ms, and 228 us at 1024 x 1024, which it fits
+// in whole waves; 31 x 17: 3.26 and 233, 31 x 19: 3.29 and 243, TileO: 3.62 and 253).
 template <int TX_, int TY_, int NT_>
 struct TileGeo {
     static constexpr int TX = TX_, TY = TY_, NT = NT_;
@@ -495,6 +493,9 @@ using TileG = TileGeo<31, 15, 256>;
 // Smaller tiles for grids of few TileP tiles, which would leave SMs idle; x
 // and y faces of the smallest one are evaluated side by side by different
 // warps.  mixed_tile() in mxe_capi.cu chooses and has the times.
+// TileO, three blocks an SM of 80 registers, is slower on large grids and faster on those
+// in between whose TileP tiles begin another wave (450 x 450: 56 against 64 us).
+using TileO = TileGeo<31, 15, 256>;
 using TileM = TileGeo<31, 7, 256>;
 using TileS = TileGeo<15, 7, 256>;
 
@@ -724,35 +725,38 @@ __device__ __forceinline__ void stage_mixed_x2(const Stage2DArgs& a, const Param
     }
 }
 
-// packed face-state pairs, two blocks per SM
-#define MXE_X2(NAME, PH, G, RUS)                                                             \
-    extern "C" __global__ void __launch_bounds__(G::NT, 2)                                \
+// packed face-state pairs, BLK blocks per SM
+#define MXE_X2(NAME, PH, G, RUS, BLK)                                                        \
+    extern "C" __global__ void __launch_bounds__(G::NT, BLK)                              \
     NAME(const Stage2DArgs a, const ParamsT<float> p, const MixedPolicy mp) {             \
         stage_mixed_x2<PH, G, RUS>(a, p, mp);                                                  \
     }
-MXE_X2(mxe_stage14_2d_mixed_planar_x2, PhysPlanar, TileP, false)
-MXE_X2(mxe_stage14_2d_mixed_planar_x2_rus, PhysPlanar, TileP, true)
-MXE_X2(mxe_stage14_2d_mixed_planar_x2_m, PhysPlanar, TileM, false)
-MXE_X2(mxe_stage14_2d_mixed_planar_x2_m_rus, PhysPlanar, TileM, true)
-MXE_X2(mxe_stage14_2d_mixed_planar_x2_s, PhysPlanar, TileS, false)
-MXE_X2(mxe_stage14_2d_mixed_planar_x2_s_rus, PhysPlanar, TileS, true)
-MXE_X2(mxe_stage14_2d_mixed_x2, PhysGeneral, TileG, false)
-MXE_X2(mxe_stage14_2d_mixed_x2_rus, PhysGeneral, TileG, true)
-MXE_X2(mxe_stage14_2d_mixed_x2_m, PhysGeneral, TileM, false)
-MXE_X2(mxe_stage14_2d_mixed_x2_m_rus, PhysGeneral, TileM, true)
-MXE_X2(mxe_stage14_2d_mixed_x2_s, PhysGeneral, TileS, false)
-MXE_X2(mxe_stage14_2d_mixed_x2_s_rus, PhysGeneral, TileS, true)
+MXE_X2(mxe_stage14_2d_mixed_planar_x2, PhysPlanar, TileP, false, 2)
+MXE_X2(mxe_stage14_2d_mixed_planar_x2_rus, PhysPlanar, TileP, true, 2)
+MXE_X2(mxe_stage14_2d_mixed_planar_x2_o, PhysPlanar, TileO, false, 3)
+MXE_X2(mxe_stage14_2d_mixed_planar_x2_o_rus, PhysPlanar, TileO, true, 3)
+MXE_X2(mxe_stage14_2d_mixed_planar_x2_m, PhysPlanar, TileM, false, 2)
+MXE_X2(mxe_stage14_2d_mixed_planar_x2_m_rus, PhysPlanar, TileM, true, 2)
+MXE_X2(mxe_stage14_2d_mixed_planar_x2_s, PhysPlanar, TileS, false, 2)
+MXE_X2(mxe_stage14_2d_mixed_planar_x2_s_rus, PhysPlanar, TileS, true, 2)
+MXE_X2(mxe_stage14_2d_mixed_x2, PhysGeneral, TileG, false, 2)
+MXE_X2(mxe_stage14_2d_mixed_x2_rus, PhysGeneral, TileG, true, 2)
+MXE_X2(mxe_stage14_2d_mixed_x2_m, PhysGeneral, TileM, false, 2)
+MXE_X2(mxe_stage14_2d_mixed_x2_m_rus, PhysGeneral, TileM, true, 2)
+MXE_X2(mxe_stage14_2d_mixed_x2_s, PhysGeneral, TileS, false, 2)
+MXE_X2(mxe_stage14_2d_mixed_x2_s_rus, PhysGeneral, TileS, true, 2)
 #undef MXE_X2
 
 template <class PH, class G>
 static MixedTile tile_of(void (*kern)(const Stage2DArgs, const ParamsT<float>, const MixedPolicy)) {
     return {(const void*)kern, G::TX, G::TY, G::NT, smem_mixed_x2<G, PH::NF>()};
 }
-// n = 0: TileP or TileG, 1: TileM, 2: TileS
+// n = 0: TileP or TileG, 1: TileM, 2: TileS, 3: TileO (planar)
 MixedTile mixed_tile_kernel(bool planar, bool rus, int n) {
 #define MXE_TILE(NAME, PH, G) tile_of<PH, G>(rus ? NAME##_rus : NAME)
     if (planar)
-        return n == 2   ? MXE_TILE(mxe_stage14_2d_mixed_planar_x2_s, PhysPlanar, TileS)
+        return n == 3   ? MXE_TILE(mxe_stage14_2d_mixed_planar_x2_o, PhysPlanar, TileO)
+               : n == 2 ? MXE_TILE(mxe_stage14_2d_mixed_planar_x2_s, PhysPlanar, TileS)
                : n == 1 ? MXE_TILE(mxe_stage14_2d_mixed_planar_x2_m, PhysPlanar, TileM)
                         : MXE_TILE(mxe_stage14_2d_mixed_planar_x2, PhysPlanar, TileP);
     return n == 2   ? MXE_TILE(mxe_stage14_2d_mixed_x2_s, PhysGeneral, TileS)

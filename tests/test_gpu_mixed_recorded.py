@@ -28,6 +28,10 @@ RECORD = os.path.join(os.path.dirname(os.path.abspath(__file__)), "golden", "mix
 RUNS = {
     "grid_97x65_hll_minmod": ((97, 65), "hll", "minmod", 8, mx.TAU_HARDSPHERE),
     "grid_331x260_hll_minmod": ((331, 260), "hll", "minmod", 20, mx.TAU_HARDSPHERE),
+    "grid_450x440_hll_minmod": ((450, 440), "hll", "minmod", 6, mx.TAU_HARDSPHERE),
+    "grid_640x600_hll_minmod": ((640, 600), "hll", "minmod", 6, mx.TAU_HARDSPHERE),
+    "grid_450x450_rusanov_vanalbada": ((450, 450), "rusanov", "vanalbada", 6, mx.TAU_HARDSPHERE),
+    "grid_700x690_rusanov_minmod": ((700, 690), "rusanov", "minmod", 6, mx.TAU_CONST),
     "grid_61x50_hll_vanalbada": ((61, 50), "hll", "vanalbada", 8, mx.TAU_CONST),
     "grid_120x83_rusanov_minmod": ((120, 83), "rusanov", "minmod", 8, mx.TAU_NONE),
     "tubes_hll_minmod": ([97, 240, 241, 700, 1531], "hll", "minmod", 40, mx.TAU_HARDSPHERE),

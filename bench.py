@@ -53,7 +53,7 @@ TRAFFIC_PER_CELL_UPDATE = {("mixed", True): 336.4}
 # issue, not by DRAM): thread instructions per cell-update over both stages
 # (ncu smsp__inst_executed.sum x 32 / cells, the same two launches) against
 # 152 SMs x 4 schedulers x 32 lanes x the sampled SM clock.
-THREAD_INST_PER_CELL_UPDATE = {("mixed", True): 4365.2}
+THREAD_INST_PER_CELL_UPDATE = {("mixed", True): 4963.3}
 KERNEL = {("fp64", False): "mxe_stage14_2d_f64", ("mixed", False): "mxe_stage14_2d_mixed_x2",
           ("fp64", True): "mxe_stage14_2d_f64_planar",
           ("mixed", True): "mxe_stage14_2d_mixed_planar_x2"}

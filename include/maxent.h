@@ -221,8 +221,8 @@ mxe_status mxe_set_mixed_policy(mxe_ctx *ctx, double sigma_lo, double sigma_hi,
  * most 80 registers per thread, three blocks per SM, the final stage's own
  * cells prefetched into L2; 2: up to 128 registers per thread, two blocks per
  * SM (planar: the final stage prefetches its own cells' U^n and W^n into
- * shared memory).  The results do not depend on it (the arithmetic is the
- * same).  MXE_EINVAL for another value, MXE_ESTATE on another kind of
+ * shared memory).  The results of planar states do not depend on it (the
+ * arithmetic is the same), those of general states to FP32 rounding.  MXE_EINVAL for another value, MXE_ESTATE on another kind of
  * context. */
 mxe_status mxe_set_stage_occupancy(mxe_ctx *ctx, int blocks_per_sm);
 

@@ -6,7 +6,7 @@
 // and coef = c dt, the kernels form
 //   out = b1 + b2 + coef (dL/dU(U_in))^T V
 // plus the adjoints of the imposed boundary states and of tau_ref:
-//   mxe_adj_prims   primitives of U_in (FP64, oracle-order rounding)
+//   mxe_adj_prims   primitives of U_in (FP64, the oracle's order of operations)
 //   mxe_adj_faces   two lanes per face, one per face state: recompute the
 //                   reconstruction and the face state once (intermediates
 //                   kept), reverse HLL / Rusanov together with the partner

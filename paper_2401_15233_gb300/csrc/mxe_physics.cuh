@@ -130,8 +130,8 @@ __device__ __forceinline__ void cons2prim5(const T* U, T* Q) {
     Q[0] = rho; Q[1] = u; Q[2] = P; Q[3] = q; Q[4] = r;
 }
 
-// Primitive recovery with every operation explicitly rounded, in the order
-// rho, u = U1/rho, P = U2 - (rho u) u, q = U3 - ((rho u) u) u - (3u) P,
+// Primitive recovery with every operation explicitly rounded (the quotient by
+// f64::div_by), in the order rho, u = U1/rho, P = U2 - (rho u) u, q = U3 - ((rho u) u) u - (3u) P,
 // r = U4 - (((rho u) u) u) u - ((6u) u) P - (4u) q.
 __device__ __forceinline__ void cons2prim5_rn(const double* U, double* Q) {
     double rho = U[0];

@@ -20,7 +20,8 @@
 // stage: warps drift apart and hide one another's loads and arithmetic, which
 // pays for the 7 % of halo work that a chunk of 30 has over one of 254 (256
 // tubes of 512 to 8192 cells, teams of 8 CTAs of 256 threads: 137 -> 131 us an
-// RK2 step).  Cluster barriers separate the stages; the team's CFL maximum and
+// RK2 step with the lighter limiter it was measured with; 40 steps with set-up and the
+// present one 5.75 ms, 6.28 with the kernel before).  Cluster barriers separate the stages; the team's CFL maximum and
 // status bits are combined in the shared memory of CTA 0 of the cluster
 // (distributed shared memory).
 //
@@ -29,7 +30,7 @@
 // cooperative launch whose CTAs meet at the barrier of mxe_team.cuh.  One tube
 // on one CTA runs on 1/152 of the chip, pass after pass over its cells, while a
 // stage takes 3 us for one pass as for many side by side.  4096 cells, planar,
-// per RK2 step: 201 -> 9.5 us (35 CTAs; set-up and read-back not counted).
+// per RK2 step: 199 -> 10.1 us (35 CTAs; set-up and read-back not counted).
 #include "mxe_internal.h"
 #include "mxe_mixed_x2.cuh"
 #include "mxe_team.cuh"

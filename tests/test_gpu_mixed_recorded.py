@@ -1,4 +1,4 @@
-"""The mixed path's results on record: planar runs of the packed 2D stage and of the tubes.
+"""The mixed path's results on record: planar runs of the packed 2D stage, and tubes.
 
 Where a field passes an extremum, the shared limiter turns on the last bits of the
 FP32 primitives, and two roundings of the same formulas end up as far from one
@@ -37,6 +37,8 @@ RUNS = {
     "tubes_hll_minmod": ([97, 240, 241, 700, 1531], "hll", "minmod", 40, mx.TAU_HARDSPHERE),
     "tubes_hll_vanalbada": ([64, 391], "hll", "vanalbada", 40, mx.TAU_NONE),
     "tubes_rusanov_minmod": ([119, 620], "rusanov", "minmod", 40, mx.TAU_CONST),
+    "general_tubes_hll_minmod": ([97, 240, 1531], "hll", "minmod", 40, mx.TAU_HARDSPHERE),
+    "general_tubes_rusanov_vanalbada": ([119, 620], "rusanov", "vanalbada", 40, mx.TAU_NONE),
 }
 TUBE_SHAPES = {"teams": None, "128x1": (128, 1), "256x8": (256, 8)}
 
@@ -66,9 +68,21 @@ def _state(x, y):
                       1.12 + 0.1 * x)
 
 
+def _general(x):
+    """Primitives with all 14 moments along a tube."""
+    s = 16.0 * x * (1.0 - x) * (0.5 - x)
+    rho = 1.0 / (1.0 + 1.3 * x) + 0.05 * s
+    p = rho * (1.0 - 0.25 * x)
+    return np.stack([rho, 0.4 + 0.6 * x, 0.3 - 0.2 * x, 0.1 + 0.2 * x + 0.04 * s, p * (1.1 + 0.05 * x),
+                     p * (0.06 - 0.03 * x), p * (0.04 + 0.02 * s), p * 0.95, p * (0.03 + 0.02 * x),
+                     p * (0.95 - 0.05 * x), 0.12 * p * (1.0 + 0.4 * s), 0.1 * p * (1.0 - 0.3 * x),
+                     0.08 * p * (1.0 + x), 15.0 * p * p / rho * (1.12 + 0.1 * x)])
+
+
 def march(name, shape=None):
     """Times (one a tube) and the final conserved state in FP32."""
     size, flux, limiter, steps, tau = RUNS[name]
+    general = name.startswith("general")
     kw = dict(system=14, precision="mixed", flux=flux, limiter=limiter)
     if isinstance(size, tuple):
         nx, ny = size
@@ -79,9 +93,10 @@ def march(name, shape=None):
         s = mx.Batch(size, [1.0] * len(size), **kw)
         if shape:
             s.set_shape(*shape)
-        U = np.concatenate([_state((np.arange(n) + 0.5) / n, np.zeros(n)).reshape(-1) for n in size])
+        x = [(np.arange(n) + 0.5) / n for n in size]
+        U = np.concatenate([(_general(v) if general else _state(v, 0.0 * v)).reshape(-1) for v in x])
     s.set_relaxation(tau, 0.05, 1.0, 1.0)
-    s.set_state(np.ascontiguousarray(U), kind="conserved")
+    s.set_state(np.ascontiguousarray(U), kind="primitive" if general else "conserved")
     if isinstance(size, tuple):
         t = [s.step(steps)[0]]
     else:
